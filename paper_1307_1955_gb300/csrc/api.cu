@@ -215,9 +215,8 @@ hj_status oversize_fallback(hj_ctx *c, int W, bool agg, bool chk, const PartTask
             continue;
         }
         HJ_TRY(table_create(c, W, agg, nr, &tg.t));
-        HJ_TRY(table_build(c, tg.t, Rt, 0, nr, nr, pf));
-        const RecArea none{nullptr, nullptr, 0};
-        HJ_TRY(table_probe(c, tg.t, St, 0, ns, ns, js.pairs, js.pcap, chk, none, pf, js.ctr, 1));
+        HJ_TRY(table_build(c, tg.t, Rt, nr, pf));
+        HJ_TRY(table_probe(c, tg.t, St, ns, js.pairs, js.pcap, chk, pf, js.ctr));
     }
     return HJ_OK;
 }
@@ -361,15 +360,14 @@ hj_status probe_into(hj_ctx *c, const hj_table *t, const hj_rel *S, const hj_opt
     for (int attempt = 0; attempt < 2; ++attempt) {
         // warps stage their pairs in shared memory and claim exact rows: the
         // output is dense as written, no compaction pass
-        RecArea ra{nullptr, nullptr, 0};
         if (mat) HJ_TRY(sink.reset(cap));
         if (!(after_build && attempt == 0)) HJ_TRY(zero_counters(c));
         if (t->keylist)
             HJ_TRY(keylist_probe(c, t, S->tuples, S->n, PartFilter{0, 0, 0, 0}, sink.pairs.p, sink.pcap, c->d_ctr,
                                  chk));
         else
-            HJ_TRY(table_probe(c, t, S->tuples, 0, S->n, S->n, sink.pairs.p, sink.pcap, chk, ra,
-                               PartFilter{0, 0, 0, 0}, nullptr, 2));
+            HJ_TRY(table_probe(c, t, S->tuples, S->n, sink.pairs.p, sink.pcap, chk, PartFilter{0, 0, 0, 0},
+                               c->d_ctr));
         HJ_TRY(read_counters(c));
         if (c->h_ctr->status & kStatusTableFull) return set_err(c, HJ_E_CUDA, "hash table unexpectedly full");
         if (c->h_ctr->status & kStatusLongRun) {
@@ -391,9 +389,8 @@ hj_status probe_into(hj_ctx *c, const hj_table *t, const hj_rel *S, const hj_opt
 
 hj_status join_shj(hj_ctx *c, const hj_rel *R, const hj_rel *S, const hj_opts &o, hj_result *res) {
     TableGuard tg{c};
-    HJ_TRY(zero_counters(c));
-    HJ_TRY(table_create(c, R->width, is_agg(o.mode), R->n, &tg.t));
-    HJ_TRY(table_build(c, tg.t, R->tuples, 0, R->n, R->n, PartFilter{0, 0, 0, 0}));
+    HJ_TRY(table_create(c, R->width, is_agg(o.mode), R->n, &tg.t, true));
+    HJ_TRY(table_build(c, tg.t, R->tuples, R->n, PartFilter{0, 0, 0, 0}));
     bool long_run = false;
     HJ_TRY(probe_into(c, tg.t, S, o, res, true, &long_run));
     if (!long_run) return HJ_OK;
@@ -935,9 +932,8 @@ hj_status hj_build(hj_ctx *c, const hj_rel *R, const hj_opts *opts, hj_table **o
     hj_opts o = opts ? *opts : default_opts();
     if (o.mode < HJ_COUNT || o.mode > HJ_MATERIALIZE) return set_err(c, HJ_E_INVALID, "bad mode %d", o.mode);
     TableGuard tg{c};
-    HJ_TRY(zero_counters(c));
-    HJ_TRY(table_create(c, R->width, is_agg(o.mode), R->n, &tg.t));
-    HJ_TRY(table_build(c, tg.t, R->tuples, 0, R->n, R->n, PartFilter{0, 0, 0, 0}));
+    HJ_TRY(table_create(c, R->width, is_agg(o.mode), R->n, &tg.t, true));
+    HJ_TRY(table_build(c, tg.t, R->tuples, R->n, PartFilter{0, 0, 0, 0}));
     HJ_TRY(read_counters(c));
     if (c->h_ctr->status & kStatusTableFull) return set_err(c, HJ_E_CUDA, "hash table unexpectedly full");
     if (c->h_ctr->status & kStatusLongRun) {  // heavily repeated keys: a key-list table

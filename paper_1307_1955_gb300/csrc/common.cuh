@@ -153,7 +153,11 @@ __device__ __forceinline__ ulonglong2 cas128(ulonglong2 *p, ulonglong2 cmp, ulon
 // A slot holds the tuple itself; the empty slot is all ones.  The one tuple whose
 // bit pattern equals the empty marker (key and rid both all ones) is not stored:
 // it is counted in `side` and re-emitted for probe keys equal to all ones.
-// Slots are claimed with a CAS of the whole tuple; probing is linear with wrap.
+// Slots are grouped in buckets of one 32-byte sector (4 slots of 4-byte tuples, 2
+// of 8-byte), so that a probe reads a whole bucket with one load.  An insert tries
+// the slots of the key's home bucket in order, each claimed with a CAS of the whole
+// tuple, then the next bucket (with wrap): a bucket is passed only while it is full,
+// so a key's run ends with the first bucket whose last slot is empty.
 template <int W> struct PairSlot;
 template <> struct PairSlot<4> {
     using S = unsigned long long;
@@ -162,7 +166,8 @@ template <> struct PairSlot<4> {
     static __device__ __forceinline__ bool is_empty(S s) { return s == ~0ull; }
     static __device__ __forceinline__ uint32_t key(S s) { return (uint32_t)s; }
     static __device__ __forceinline__ uint32_t rid(S s) { return (uint32_t)(s >> 32); }
-    static __device__ __forceinline__ bool try_claim(S *p, S v) { return atomicCAS(p, ~0ull, v) == ~0ull; }
+    // the slot's tuple before: the empty marker if v has it now
+    static __device__ __forceinline__ S claim(S *p, S v) { return atomicCAS(p, ~0ull, v); }
 };
 template <> struct PairSlot<8> {
     using S = ulonglong2;
@@ -171,10 +176,7 @@ template <> struct PairSlot<8> {
     static __device__ __forceinline__ bool is_empty(S s) { return (s.x & s.y) == ~0ull; }
     static __device__ __forceinline__ uint64_t key(S s) { return s.x; }
     static __device__ __forceinline__ uint64_t rid(S s) { return s.y; }
-    static __device__ __forceinline__ bool try_claim(S *p, S v) {
-        S o = cas128(p, empty(), v);
-        return (o.x & o.y) == ~0ull;
-    }
+    static __device__ __forceinline__ S claim(S *p, S v) { return cas128(p, empty(), v); }
 };
 
 // ------------------------------------------------------------- aggregate table
@@ -212,7 +214,7 @@ struct TableSide {
     unsigned long long n_allones;   // pair table: R tuples equal to the empty marker
     unsigned long long agg_cnt;     // aggregate table: R tuples with the all-ones key
     unsigned long long agg_suma;
-    unsigned long long full;        // set when an insert found no free slot
+    unsigned long long repeats;     // pair table: not 0 unless every key in it is another (and not all ones)
 };
 
 // Longest walk of a pair-table insert.  Unique keys at load factor <= 1/2 never
@@ -220,45 +222,102 @@ struct TableSide {
 // ones), and the join then takes a key-list table instead.
 constexpr uint64_t kMaxPairWalk = 1024;
 
-// Insert one build tuple into a pair table of `cap` slots.  Returns false if
-// the table had no free slot (cannot happen while cap > number of tuples) or
-// the walk passed max_walk slots.
+// Slots per bucket, and a bucket's keys and rids in one 32-byte load (the table
+// is not written while it is probed).
+template <int W> constexpr uint32_t kBucketSlots = 32 / (2 * W);
 template <int W>
-__device__ __forceinline__ bool pair_insert(typename PairSlot<W>::S *slots, uint64_t cap, TableSide *side,
-                                            typename Tup<W>::U k, typename Tup<W>::U r, uint64_t h,
+__device__ __forceinline__ void ld_bucket(const typename PairSlot<W>::S *slots, uint32_t bkt, typename Tup<W>::U *k,
+                                          typename Tup<W>::U *r) {
+    unsigned long long x[4];
+    asm volatile("ld.global.nc.L1::no_allocate.v4.u64 {%0, %1, %2, %3}, [%4];"
+                 : "=l"(x[0]), "=l"(x[1]), "=l"(x[2]), "=l"(x[3])
+                 : "l"((const char *)slots + (uint64_t)bkt * 32));
+#pragma unroll
+    for (uint32_t q = 0; q < kBucketSlots<W>; ++q) {
+        if constexpr (W == 4) {
+            k[q] = (uint32_t)x[q];
+            r[q] = (uint32_t)(x[q] >> 32);
+        } else {
+            k[q] = x[2 * q];
+            r[q] = x[2 * q + 1];
+        }
+    }
+}
+
+// Home bucket of a key's hash in a pair table of nb buckets (below 2^32): its high
+// half scaled to nb.
+template <int W> __device__ __forceinline__ uint32_t pair_bucket(uint64_t h, uint32_t nb);
+template <> __device__ __forceinline__ uint32_t pair_bucket<4>(uint64_t h, uint32_t nb) {
+    return __umulhi((uint32_t)h, nb);
+}
+template <> __device__ __forceinline__ uint32_t pair_bucket<8>(uint64_t h, uint32_t nb) {
+    return __umulhi((uint32_t)(h >> 32), nb);
+}
+
+// Insert one build tuple into a pair table of nb buckets.  Returns false if the
+// table had no free slot (cannot happen while it has more slots than tuples) or the
+// walk passed max_walk slots.  Sets *repeat for the all-ones key and for a key met
+// on the way: slots are tried in the run's order and are never emptied, so of two
+// tuples with one key the later one passes the earlier one's slot and sees it.
+template <int W>
+__device__ __forceinline__ bool pair_insert(typename PairSlot<W>::S *slots, uint32_t nb, TableSide *side,
+                                            typename Tup<W>::U k, typename Tup<W>::U r, uint64_t h, bool *repeat,
                                             uint64_t max_walk = kMaxPairWalk) {
     using PS = PairSlot<W>;
-    if (k == Tup<W>::kAllOnes && r == Tup<W>::kAllOnes) {
-        atomicAdd(&side->n_allones, 1ull);
-        return true;
+    constexpr uint32_t G = kBucketSlots<W>;
+    if (k == Tup<W>::kAllOnes) {
+        *repeat = true;
+        if (r == Tup<W>::kAllOnes) {
+            atomicAdd(&side->n_allones, 1ull);
+            return true;
+        }
     }
     typename PS::S v = PS::pack(k, r);
-    uint64_t b = bucket_of<W>(h, cap);
-    const uint64_t lim = cap < max_walk ? cap : max_walk;
-    for (uint64_t it = 0; it < lim; ++it) {
-        if (PS::try_claim(&slots[b], v)) return true;
-        if (++b == cap) b = 0;
+    uint32_t b = pair_bucket<W>(h, nb);
+    const uint32_t lim = (uint64_t)nb * G < max_walk ? nb : (uint32_t)(max_walk / G);
+    for (uint32_t it = 0; it < lim; ++it) {
+#pragma unroll
+        for (uint32_t q = 0; q < G; ++q) {
+            const typename PS::S o = PS::claim(&slots[(uint64_t)b * G + q], v);
+            if (PS::is_empty(o)) return true;
+            if (PS::key(o) == k) *repeat = true;
+        }
+        if (++b == nb) b = 0;
     }
     return false;
 }
 
-// Visit every build rid whose key equals k: f(rid).  The key's run starts at its
-// home slot bucket_of(h, cap / group) * group and ends at the first empty slot (a
-// table always keeps at least one), after at most cap slots.
+// Visit every build rid whose key equals k: f(rid), over the run of buckets from
+// the key's home to the first one with an empty slot (a table always keeps at
+// least one).
 template <int W, class F>
-__device__ __forceinline__ void pair_lookup(const typename PairSlot<W>::S *slots, uint64_t cap,
-                                            unsigned long long n_allones, typename Tup<W>::U k, uint64_t h,
-                                            uint32_t group, F &&f) {
-    using PS = PairSlot<W>;
-    uint64_t b = bucket_of<W>(h, cap / group) * group;
-    for (uint64_t it = 0; it < cap; ++it) {
-        typename PS::S s = slots[b];
-        if (PS::is_empty(s)) break;
-        if (PS::key(s) == k) f(PS::rid(s));
-        if (++b == cap) b = 0;
+__device__ __forceinline__ void pair_lookup(const typename PairSlot<W>::S *slots, uint32_t nb,
+                                            unsigned long long n_allones, typename Tup<W>::U k, uint64_t h, F &&f) {
+    constexpr uint32_t G = kBucketSlots<W>;
+    uint32_t b = pair_bucket<W>(h, nb);
+    for (uint32_t it = 0; it < nb; ++it) {
+        typename Tup<W>::U bk[G], br[G];
+        ld_bucket<W>(slots, b, bk, br);
+#pragma unroll
+        for (uint32_t q = 0; q < G; ++q)
+            if (bk[q] == k && (bk[q] & br[q]) != Tup<W>::kAllOnes) f(br[q]);
+        if ((bk[G - 1] & br[G - 1]) == Tup<W>::kAllOnes) break;
+        if (++b == nb) b = 0;
     }
     if (k == Tup<W>::kAllOnes)
         for (unsigned long long i = 0; i < n_allones; ++i) f(Tup<W>::kAllOnes);
+}
+
+// One step of a warp's joint walk of a key's run (32 consecutive slots from a
+// bucket's first on; this lane's slot s, empty where the table has no more):
+// whether the slot belongs to the run.  Buckets fill in order, so the run's slots
+// are the ones before the step's first empty slot, and the run ends there (*end,
+// the same for all lanes).
+template <int W>
+__device__ __forceinline__ bool run_step(typename PairSlot<W>::S s, bool *end) {
+    const unsigned emp = __ballot_sync(0xffffffffu, PairSlot<W>::is_empty(s));
+    *end = emp != 0;
+    return emp == 0 || (threadIdx.x & 31) < (unsigned)(__ffs(emp) - 1);
 }
 
 // Insert a build tuple into an aggregate table.  Returns false if the key is new
@@ -282,30 +341,6 @@ __device__ __forceinline__ bool agg_insert(AggSlot<W> *slots, uint64_t cap, Tabl
         if (++b == cap) b = 0;
     }
     return false;
-}
-
-// Look a probe key up in an aggregate table: (count, suma) of its build tuples.
-template <int W>
-__device__ __forceinline__ void agg_lookup(const AggSlot<W> *slots, uint64_t cap, const TableSide *side,
-                                           typename Tup<W>::U k, uint64_t h, uint64_t *cnt, uint64_t *suma) {
-    *cnt = 0;
-    *suma = 0;
-    if (k == Tup<W>::kAllOnes) {
-        *cnt = side->agg_cnt;
-        *suma = side->agg_suma;
-        return;
-    }
-    uint64_t b = bucket_of<W>(h, cap);
-    for (uint64_t it = 0; it < cap; ++it) {
-        typename Tup<W>::U sk = slots[b].key;
-        if (sk == k) {
-            *cnt = slots[b].cnt;
-            *suma = slots[b].suma;
-            return;
-        }
-        if (sk == Tup<W>::kAllOnes) return;
-        if (++b == cap) b = 0;
-    }
 }
 
 // ------------------------------------------------------------- block scan

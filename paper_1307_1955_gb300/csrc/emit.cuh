@@ -135,6 +135,37 @@ __device__ __forceinline__ void warp_append(OutState &st, const OutCtx &oc, bool
     st.pairs += k;
 }
 
+// Append one pair per lane and item with cnt[i] == 1 (IT <= 4 items; a staging
+// buffer holds at least 32 * IT pairs): one room test for all of them.
+template <int W, int IT>
+__device__ __forceinline__ void warp_append_group(OutState &st, const OutCtx &oc, const uint32_t *cnt,
+                                                  const typename Tup<W>::U *a, const typename Tup<W>::U *b) {
+    if (!oc.stage) {
+#pragma unroll
+        for (int i = 0; i < IT; ++i) warp_append<W>(st, oc, cnt[i] == 1, a[i], b[i]);
+        return;
+    }
+    using P = typename PairVec<W>::T;
+    const unsigned lt = (1u << (threadIdx.x & 31)) - 1u;
+    unsigned m[IT], tot = 0;
+#pragma unroll
+    for (int i = 0; i < IT; ++i) {
+        m[i] = __ballot_sync(0xffffffffu, cnt[i] == 1);
+        tot += __popc(m[i]);
+    }
+    if (st.used + tot > oc.scap) warp_stage_flush<W>(st, oc);
+    P *s = (P *)oc.stage + st.used;
+#pragma unroll
+    for (int i = 0; i < IT; ++i) {
+        if (cnt[i] == 1) {
+            if constexpr (W == 4) s[__popc(m[i] & lt)] = make_uint2(a[i], b[i]);
+            else s[__popc(m[i] & lt)] = make_ulonglong2(a[i], b[i]);
+        }
+        s += __popc(m[i]);
+    }
+    st.used += tot;
+}
+
 // Record the warp's partly filled chunk and add its pair count.  All lanes call.
 __device__ __forceinline__ void warp_finish(const OutState &st, const OutCtx &oc, const RecArea &ra) {
     if ((threadIdx.x & 31) != 0) return;

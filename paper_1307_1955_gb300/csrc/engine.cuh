@@ -12,8 +12,9 @@ namespace hj {
 struct RecArea;  // emit.cuh
 
 // ----------------------------------------------------------------- join.cu
-// Global-memory table (SHJ, Alg. 1): allocate + initialise, build, probe.
-hj_status table_create(hj_ctx *c, int width, int agg, uint64_t n_build, hj_table **out);
+// Global-memory table (SHJ, Alg. 1): allocate + initialise (with zero_ctr the
+// context's counters too), build, probe.
+hj_status table_create(hj_ctx *c, int width, int agg, uint64_t n_build, hj_table **out, bool zero_ctr = false);
 void table_destroy(hj_ctx *c, hj_table *t);
 // Key-list table (keylist.cu): aggregate-table slots over the kept tuples of
 // R[0, n) plus the rid lists (t->rids, every key's rids contiguous at the offset
@@ -23,23 +24,15 @@ hj_status keylist_build(hj_ctx *c, int width, const void *R, uint64_t n, PartFil
 // from ctr->count (dense output); checksums with `chk`.
 hj_status keylist_probe(hj_ctx *c, const hj_table *t, const void *S, uint64_t ns, PartFilter pf, void *pairs,
                         uint64_t pcap, hj_counters *ctr, int chk);
-// Insert tuples [lo, hi) of the array `R` (n_total tuples long) into the table.
-// With pf.on only tuples of partition pf.p are inserted (padding is skipped).
-hj_status table_build(hj_ctx *c, hj_table *t, const void *R, uint64_t lo, uint64_t hi, uint64_t n_total,
-                      PartFilter pf);
-// Probe with tuples [lo, hi) of S; counts and checksums accumulate into the
-// context counters, pairs into `pairs` (capacity pcap; unused in count modes).
-// Warps that leave a partly filled output chunk record it in `ra`.
-// ctr: the counters to accumulate into (NULL: the context's).  dense: 0 = warps
-// take whole chunks of the cursor (holes recorded in `ra`); 1 = every append
-// claims exactly its rows from ctr->count; 2 = each warp stages its pairs in
-// shared memory and claims exactly that many rows per full buffer (no holes,
-// one atomic per 256 pairs).
-hj_status table_probe(hj_ctx *c, const hj_table *t, const void *S, uint64_t lo, uint64_t hi, uint64_t n_total,
-                      void *pairs, uint64_t pcap, int checksum, RecArea ra, PartFilter pf,
-                      hj_counters *ctr = nullptr, int dense = 0);
-// Number of warps table_probe launches for n probe tuples (record-area size).
-uint64_t table_probe_warps(hj_ctx *c, uint64_t n);
+// Insert the n tuples of R into the table.  With pf.on (aggregate tables) only
+// tuples of partition pf.p are inserted (padding is skipped).
+hj_status table_build(hj_ctx *c, hj_table *t, const void *R, uint64_t n, PartFilter pf);
+// Probe with the n tuples of S (aggregate tables: those that pf keeps): counts and
+// checksums accumulate into `ctr`, pairs go to `pairs` (capacity pcap; unused in
+// count modes).  Each warp stages its pairs in shared memory and claims exactly as
+// many rows of ctr->count per full buffer: dense output, one atomic per buffer.
+hj_status table_probe(hj_ctx *c, const hj_table *t, const void *S, uint64_t n, void *pairs, uint64_t pcap,
+                      int checksum, PartFilter pf, hj_counters *ctr);
 
 // A partition pair for the shared-memory join: padded partitions (every row
 // range starts on a 32-byte sector, its row count is a multiple of the sector's

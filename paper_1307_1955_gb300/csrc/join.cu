@@ -12,6 +12,7 @@
 // walked by the whole warp, 32 consecutive slots at a time -- the GPU answer to
 // the divergence that skew causes in steps b3/p3 (Sec. 3.3, workload divergence).
 #include <algorithm>
+#include <cstddef>
 #include <type_traits>
 
 #include "common.cuh"
@@ -21,188 +22,305 @@
 namespace hj {
 
 // ------------------------------------------------------------------ tuple loads
-// Vector v of a tuple array holds tuples v*PV .. v*PV+PV-1.  The last vector of a
-// 4-byte relation with an odd number of tuples is read with one 8-byte load so
-// that no read passes the array end.
-template <int W>
-__device__ __forceinline__ void load_vec(const void *base, uint64_t v, uint64_t n_total, typename Tup<W>::U *k,
-                                         typename Tup<W>::U *r) {
-    if constexpr (W == 8) {
-        ulonglong2 x = ld_stream((const ulonglong2 *)base + v);
-        k[0] = x.x;
-        r[0] = x.y;
-    } else {
-        if (2 * v + 1 < n_total) {
-            uint4 x = ld_stream((const uint4 *)base + v);
-            k[0] = x.x;
-            r[0] = x.y;
-            k[1] = x.z;
-            r[1] = x.w;
-        } else {
-            uint2 x = ((const uint2 *)base)[2 * v];
-            k[0] = x.x;
-            r[0] = x.y;
-            k[1] = 0;
-            r[1] = 0;
-        }
-    }
-}
-
-// A warp's group: U vectors per lane, lane-interleaved (vector g + u*32 + lane).
+// Vectors of a warp's probe group (U per lane, lane-interleaved) of an array of n
+// tuples, from vector g on; item e of vector u is x[u]'s e-th tuple.  Lanes past the
+// end load nothing.  The last vector of a 4-byte relation with an odd number of
+// tuples is read with one 8-byte load, so that no read passes the array end.
 template <int W, int U> struct Group {
+    using Vec = typename Tup<W>::Vec;
     static constexpr int PV = Tup<W>::kPerVec;
     static constexpr int IT = U * PV;
-    typename Tup<W>::U k[IT], r[IT];
-    bool valid[IT];
-    __device__ __forceinline__ void load(const void *S, uint64_t g, uint64_t lo, uint64_t hi, uint64_t vb,
-                                         uint64_t n_total) {
+    Vec x[U];
+    uint32_t valid;  // one bit per item
+    __device__ __forceinline__ void load(const Vec *S, uint64_t g, uint64_t n) {
         const unsigned lane = threadIdx.x & 31;
+        const uint64_t nvec = (n + PV - 1) / PV;
+        const Vec *p = S + g + lane;
+        if (g + 32 * U <= n / PV) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) x[u] = ld_stream(p + 32 * u);
+            valid = (1u << IT) - 1u;
+            return;
+        }
+        valid = 0;
+        if (g >= nvec) return;
+        const uint32_t left = (uint32_t)(nvec - g), whole = (uint32_t)(n / PV - g);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            uint64_t v = g + (uint64_t)u * 32 + lane;
-            typename Tup<W>::U kk[2] = {0, 0}, rr[2] = {0, 0};
-            if (v < vb) load_vec<W>(S, v, n_total, kk, rr);
-#pragma unroll
-            for (int e = 0; e < PV; ++e) {
-                uint64_t t = v * PV + e;
-                k[u * PV + e] = kk[e];
-                r[u * PV + e] = rr[e];
-                valid[u * PV + e] = v < vb && t >= lo && t < hi;
+            const uint32_t i = 32 * u + lane;
+            if (i < whole) {
+                x[u] = ld_stream(p + 32 * u);
+                valid |= ((1u << PV) - 1u) << (u * PV);
+            } else if (W == 4 && i < left) {
+                if constexpr (W == 4) {
+                    const uint2 y = *(const uint2 *)(p + 32 * u);
+                    x[u] = make_uint4(y.x, y.y, 0u, 0u);
+                }
+                valid |= 1u << (u * PV);
             }
         }
+    }
+    __device__ __forceinline__ typename Tup<W>::U key(int i) const {
+        if constexpr (W == 4) return i % 2 ? x[i / 2].z : x[i / 2].x;
+        else return x[i].x;
+    }
+    __device__ __forceinline__ typename Tup<W>::U rid(int i) const {
+        if constexpr (W == 4) return i % 2 ? x[i / 2].w : x[i / 2].y;
+        else return x[i].y;
     }
 };
 
 // ----------------------------------------------------------------- table views
-// Pair table: slots in shared or global memory (generic addressing).
-// A key's probe run starts at its home slot, bucket_of(h, cap / group) * group:
-// group 1 for the global table, a bucket of `group` slots read together for the
-// shared-memory tables.  Runs continue linearly (with wrap) to the first empty slot.
+// The pair table of common.cuh: nb buckets of one 32-byte sector.
 template <int W> struct PairTab {
     using U = typename Tup<W>::U;
     using PS = PairSlot<W>;
+    static constexpr uint32_t G = kBucketSlots<W>;
     const typename PS::S *slots;
-    uint64_t cap;
+    uint32_t nb;
     unsigned long long n_allones;
-    uint32_t group;
+    bool unique;  // no key twice (nor the all-ones key): a match ends the search
 
-    template <class F> __device__ __forceinline__ void lookup(U k, uint64_t h, F &&f) const {
-        pair_lookup<W>(slots, cap, n_allones, k, h, group, f);
-    }
-    // The whole warp emits every build match of probe key kk (probe rid ss).
-    __device__ __forceinline__ void coop_emit(U kk, U ss, OutState &st, const OutCtx &oc) const {
-        const unsigned lane = threadIdx.x & 31;
-        const uint64_t b = bucket_of<W>(key_hash<W>(kk), cap / group) * group;
-        for (uint64_t off = 0; off < cap; off += 32) {
-            const bool inr = off + lane < cap;
-            uint64_t idx = b + off + lane;
-            if (idx >= cap) idx -= cap;
-            typename PS::S s = inr ? slots[idx] : PS::empty();
-            const unsigned emp = __ballot_sync(0xffffffffu, !inr || PS::is_empty(s));
-            const unsigned before = emp ? ((emp & (0u - emp)) - 1u) : 0xffffffffu;
-            const bool m = ((before >> lane) & 1u) && PS::key(s) == kk;
-            warp_append<W>(st, oc, m, PS::rid(s), ss);
-            if (emp) break;
-        }
-        if (kk == Tup<W>::kAllOnes)
-            for (unsigned long long i = 0; i < n_allones; i += 32)
-                warp_append<W>(st, oc, i + lane < n_allones, Tup<W>::kAllOnes, ss);
-    }
+    __device__ __forceinline__ uint32_t home(U k) const { return pair_bucket<W>(key_hash<W>(k), nb); }
+    __device__ __forceinline__ uint32_t next(uint32_t b) const { return b + 1 == nb ? 0 : b + 1; }
 };
 
-template <int W> struct AggTab {
-    using U = typename Tup<W>::U;
-    const AggSlot<W> *slots;
-    uint64_t cap;
-    const TableSide *side;
-    __device__ __forceinline__ void lookup(U k, uint64_t h, uint64_t *cnt, uint64_t *suma) const {
-        agg_lookup<W>(slots, cap, side, k, h, cnt, suma);
-    }
-};
+// Tuples per lane and probe group.
+constexpr int kProbeItems = 2;
+constexpr int kProbeCtas = 4;  // per SM
 
 // Per-lane accumulators of a probing warp.
 struct ProbeAcc {
     unsigned long long cnt = 0, c0 = 0, c1 = 0;
 };
 
-// Probe one group against a pair table and append its pairs.
-template <int W, int U>
-__device__ __forceinline__ void probe_group_pairs(const PairTab<W> &tab, const Group<W, U> &g, const PartFilter &pf,
-                                                  bool chk, OutState &st, const OutCtx &oc, ProbeAcc &acc) {
-    using T = typename Tup<W>::U;
-    constexpr int IT = Group<W, U>::IT;
-    uint32_t cnt[IT];
-    T first[IT];
-#pragma unroll
-    for (int i = 0; i < IT; ++i) {
-        uint32_t c = 0;
-        T f = 0;
-        const uint64_t h = key_hash<W>(g.k[i]);
-        if (g.valid[i] && pf.keep(h)) {
-            const uint64_t bs = chk ? mix_b(g.r[i]) : 0;
-            tab.lookup(g.k[i], h, [&](T rid) {
-                if (c == 0) f = rid;
-                ++c;
-                if (chk) {
-                    uint64_t a = mix_a(rid);
-                    acc.c0 += a * bs;
-                    acc.c1 += a + bs;
-                }
-            });
-        }
-        cnt[i] = c;
-        first[i] = f;
-    }
-#pragma unroll
-    for (int i = 0; i < IT; ++i) warp_append<W>(st, oc, cnt[i] == 1, first[i], g.r[i]);
-#pragma unroll
-    for (int i = 0; i < IT; ++i) {
-        unsigned multi = __ballot_sync(0xffffffffu, cnt[i] > 1);
-        while (multi) {
-            const int L = __ffs(multi) - 1;
-            multi &= multi - 1;
-            T kk = __shfl_sync(0xffffffffu, g.k[i], L);
-            T ss = __shfl_sync(0xffffffffu, g.r[i], L);
-            tab.coop_emit(kk, ss, st, oc);
-        }
-    }
+template <int W, bool CHK>
+__device__ __forceinline__ void add_check(ProbeAcc &acc, bool has, typename Tup<W>::U rid_r, typename Tup<W>::U rid_s) {
+    if (!CHK || !has) return;
+    const uint64_t a = mix_a(rid_r), b = mix_b(rid_s);
+    acc.c0 += a * b;
+    acc.c1 += a + b;
 }
 
-template <int W, int U>
-__device__ __forceinline__ void probe_group_agg(const AggTab<W> &tab, const Group<W, U> &g, const PartFilter &pf,
-                                                bool chk, ProbeAcc &acc) {
+// The whole warp emits every build match of probe key kk (probe rid ss).
+template <int W, bool CHK>
+__device__ __forceinline__ void coop_emit(const PairTab<W> &tab, typename Tup<W>::U kk, typename Tup<W>::U ss,
+                                          OutState &st, const OutCtx &oc, ProbeAcc &acc) {
+    using PS = PairSlot<W>;
+    const unsigned lane = threadIdx.x & 31;
+    const uint64_t cap = (uint64_t)tab.nb * PairTab<W>::G, b = (uint64_t)tab.home(kk) * PairTab<W>::G;
+    for (uint64_t off = 0; off < cap; off += 32) {
+        uint64_t idx = b + off + lane;
+        if (idx >= cap) idx -= cap;
+        const typename PS::S s = off + lane < cap ? tab.slots[idx] : PS::empty();
+        bool end;
+        const bool has = run_step<W>(s, &end) && PS::key(s) == kk;
+        add_check<W, CHK>(acc, has, PS::rid(s), ss);
+        warp_append<W>(st, oc, has, PS::rid(s), ss);
+        if (end) break;
+    }
+    if (kk == Tup<W>::kAllOnes)
+        for (unsigned long long i = 0; i < tab.n_allones; i += 32) {
+            const bool has = i + lane < tab.n_allones;
+            add_check<W, CHK>(acc, has, Tup<W>::kAllOnes, ss);
+            warp_append<W>(st, oc, has, Tup<W>::kAllOnes, ss);
+        }
+}
+
+// A probing warp's queue of runs that go on past a full bucket: the probe's key and
+// rid and the run's next bucket.  Fewer than 32 entries wait when a group starts,
+// and it adds at most its own items.
+template <int W> struct RunQueue {
+    using T = typename Tup<W>::U;
+    static constexpr uint32_t N = 32 * (kProbeItems + 1);
+    T k[N], r[N];
+    uint32_t b[N];
+};
+
+// Queue the lanes with `on` (key, rid, next bucket); n is the queue's length.
+template <int W>
+__device__ __forceinline__ void push_runs(RunQueue<W> &q, uint32_t &n, bool on, typename Tup<W>::U k,
+                                          typename Tup<W>::U r, uint32_t b) {
+    const unsigned m = __ballot_sync(0xffffffffu, on);
+    if (!m) return;
+    if (on) {
+        const uint32_t at = n + __popc(m & ((1u << (threadIdx.x & 31)) - 1u));
+        q.k[at] = k;
+        q.r[at] = r;
+        q.b[at] = b;
+    }
+    n += __popc(m);
+}
+
+// The last n <= 32 entries (one per lane) take their next bucket: its matches are
+// appended, and runs that go on are queued again.
+template <int W, bool CHK>
+__device__ __forceinline__ void drain_runs(const PairTab<W> &tab, RunQueue<W> &q, uint32_t &qn, uint32_t n,
+                                           OutState &st, const OutCtx &oc, ProbeAcc &acc) {
+    using T = typename Tup<W>::U;
+    constexpr uint32_t G = PairTab<W>::G;
+    const unsigned lane = threadIdx.x & 31;
+    const bool on = lane < n;
+    __syncwarp();
+    qn -= n;
+    const T k = on ? q.k[qn + lane] : T(0), r = on ? q.r[qn + lane] : T(0);
+    const uint32_t b = on ? q.b[qn + lane] : 0;
+    __syncwarp();  // read before the queue is refilled
+    T bk[G], br[G];
+    ld_bucket<W>(tab.slots, b, bk, br);
+    bool any = false;
+#pragma unroll
+    for (uint32_t s = 0; s < G; ++s) {
+        const bool has = on && bk[s] == k && (bk[s] & br[s]) != Tup<W>::kAllOnes;
+        any |= has;
+        add_check<W, CHK>(acc, has, br[s], r);
+        warp_append<W>(st, oc, has, br[s], r);
+    }
+    push_runs<W>(q, qn, on && (bk[G - 1] & br[G - 1]) != Tup<W>::kAllOnes && !(tab.unique && any), k, r, tab.next(b));
+}
+
+// Probe one group against a pair table and append its pairs (FULL: every item of
+// every lane is a tuple).  A probe is one random sector read from L2 (or HBM): the
+// home buckets of all the lane's items are loaded before the first one is looked
+// at.  The home bucket is searched without branches.  A run that goes on past it
+// (its last slot is taken, a few per cent) is queued, and 32 of them take their next
+// bucket together.
+// What bounds it: the instructions of a tuple (about 140 thread instructions) and
+// the L1 passes of its 32 scattered sectors per load, not DRAM.  2^24 tuples against
+// 2^18 (all in L2) took 216 us slot by slot with a branch per slot, 106 us like this;
+// 6e6 8-byte tuples against 1e6 took 163 us and 56 us.  Four items per lane, or five
+// CTAs per SM for 8-byte tuples, measured slower (more sectors in flight than L1 has
+// lines for), and so did buckets of 16 bytes (2.4 times: their runs go on too often).
+template <int W, int U, bool CHK, bool FULL>
+__device__ __forceinline__ void probe_group_pairs(const PairTab<W> &tab, const Group<W, U> &g, RunQueue<W> &q,
+                                                  uint32_t &qn, OutState &st, const OutCtx &oc, ProbeAcc &acc) {
+    using T = typename Tup<W>::U;
     constexpr int IT = Group<W, U>::IT;
+    constexpr uint32_t G = PairTab<W>::G;
+    constexpr T ones = Tup<W>::kAllOnes;
+    const unsigned lane = threadIdx.x & 31;
+    uint32_t cnt[IT], bkt[IT];
+    T first[IT], k[IT], r[IT], bk[IT][G], br[IT][G];
 #pragma unroll
     for (int i = 0; i < IT; ++i) {
-        const uint64_t h = key_hash<W>(g.k[i]);
-        if (!g.valid[i] || !pf.keep(h)) continue;
-        uint64_t n, sa;
-        tab.lookup(g.k[i], h, &n, &sa);
+        k[i] = g.key(i);
+        r[i] = g.rid(i);
+        bkt[i] = tab.home(k[i]);  // (a bucket of the table whatever the key)
+        ld_bucket<W>(tab.slots, bkt[i], bk[i], br[i]);
+    }
+    bool walk[IT], odd = false;
+#pragma unroll
+    for (int i = 0; i < IT; ++i) {
+        const bool live = FULL || ((g.valid >> i) & 1u);
+        T f = br[i][G - 1];
+        uint32_t c = bk[i][G - 1] == k[i];
+#pragma unroll
+        for (int s = (int)G - 2; s >= 0; --s) {
+            const bool m = bk[i][s] == k[i];
+            f = m ? br[i][s] : f;
+            c += m;
+        }
+        first[i] = f;
+        cnt[i] = live ? c : 0;
+        walk[i] = live && (bk[i][G - 1] & br[i][G - 1]) != ones && !(tab.unique && c);
+        odd |= live && (c > 1 || k[i] == ones);
+    }
+    odd = __any_sync(0xffffffffu, odd);
+    if (odd) {  // several matches, or the key that empty slots hold too
+#pragma unroll
+        for (int i = 0; i < IT; ++i) {
+            if (k[i] == ones && (FULL || ((g.valid >> i) & 1u))) {
+                uint32_t c = 0;
+#pragma unroll
+                for (int s = (int)G - 1; s >= 0; --s)
+                    if (bk[i][s] == ones && br[i][s] != ones) {
+                        first[i] = br[i][s];
+                        ++c;
+                    }
+                if (tab.n_allones) {  // tuples kept beside the table
+                    if (!c) first[i] = ones;
+                    c += (uint32_t)min(tab.n_allones, 2ull);
+                }
+                cnt[i] = c;
+            }
+            if (cnt[i] > 1) walk[i] = false;  // (its whole run is walked below)
+        }
+    }
+    if (CHK)
+#pragma unroll
+        for (int i = 0; i < IT; ++i) add_check<W, CHK>(acc, cnt[i] == 1, first[i], r[i]);
+    warp_append_group<W, IT>(st, oc, cnt, first, r);
+    if (odd)
+#pragma unroll
+        for (int i = 0; i < IT; ++i) {
+            unsigned multi = __ballot_sync(0xffffffffu, cnt[i] > 1);
+            while (multi) {
+                const int L = __ffs(multi) - 1;
+                multi &= multi - 1;
+                coop_emit<W, CHK>(tab, __shfl_sync(0xffffffffu, k[i], L), __shfl_sync(0xffffffffu, r[i], L), st, oc,
+                                  acc);
+            }
+        }
+#pragma unroll
+    for (int i = 0; i < IT; ++i) push_runs<W>(q, qn, walk[i], k[i], r[i], tab.next(bkt[i]));
+    while (qn >= 32) drain_runs<W, CHK>(tab, q, qn, 32, st, oc, acc);
+}
+
+// Probe one group against an aggregate table: the home slots of all the lane's
+// items are loaded before the first one is looked at; runs that go on are walked
+// one by one.
+template <int W, int U, bool CHK>
+__device__ __forceinline__ void probe_group_agg(const AggSlot<W> *slots, uint64_t cap, const TableSide *side,
+                                                const Group<W, U> &g, const PartFilter &pf, ProbeAcc &acc) {
+    using T = typename Tup<W>::U;
+    constexpr int IT = Group<W, U>::IT;
+    AggSlot<W> s[IT];
+    uint64_t h[IT];
+    auto ld = [&](uint64_t at) {
+        AggSlot<W> x;
+        if constexpr (W == 4) {
+            const ulonglong2 y = __ldg((const ulonglong2 *)slots + at);
+            x.key = (uint32_t)y.x;
+            x.cnt = (uint32_t)(y.x >> 32);
+            x.suma = y.y;
+        } else {
+            unsigned long long pad;
+            asm volatile("ld.global.nc.v4.u64 {%0, %1, %2, %3}, [%4];"
+                         : "=l"(x.key), "=l"(x.cnt), "=l"(x.suma), "=l"(pad)
+                         : "l"(slots + at));
+        }
+        return x;
+    };
+#pragma unroll
+    for (int i = 0; i < IT; ++i) {
+        h[i] = key_hash<W>(g.key(i));
+        s[i] = ld(bucket_of<W>(h[i], cap));  // (a slot of the table whatever the key)
+    }
+#pragma unroll
+    for (int i = 0; i < IT; ++i) {
+        if (!((g.valid >> i) & 1u) || !pf.keep(h[i])) continue;
+        const T k = g.key(i);
+        uint64_t n = 0, sa = 0;
+        if (k == Tup<W>::kAllOnes) {
+            n = side->agg_cnt;
+            sa = side->agg_suma;
+        } else {
+            uint64_t b = bucket_of<W>(h[i], cap);
+            for (uint64_t it = 1; s[i].key != k && s[i].key != Tup<W>::kAllOnes && it < cap; ++it) {
+                if (++b == cap) b = 0;
+                s[i] = ld(b);
+            }
+            if (s[i].key == k) {
+                n = s[i].cnt;
+                sa = s[i].suma;
+            }
+        }
         acc.cnt += n;
-        if (chk && n) {
-            const uint64_t b = mix_b(g.r[i]);
+        if (CHK && n) {
+            const uint64_t b = mix_b(g.rid(i));
             acc.c0 += sa * b;
             acc.c1 += sa + n * b;
         }
-    }
-}
-
-// Stream S rows [lo, hi) through one warp: groups g = g0, g0 + gstride, ...
-template <int W, int U, bool AGG, class Tab>
-__device__ __forceinline__ void warp_probe(const Tab &tab, const void *S, uint64_t lo, uint64_t hi, uint64_t n_total,
-                                           uint64_t g0, uint64_t gstride, const PartFilter &pf, bool chk,
-                                           OutState &st, const OutCtx &oc, ProbeAcc &acc) {
-    constexpr int PV = Tup<W>::kPerVec;
-    const uint64_t vb = (hi + PV - 1) / PV;
-    if (g0 >= vb) return;
-    Group<W, U> cur, nxt;
-    cur.load(S, g0, lo, hi, vb, n_total);
-    for (uint64_t g = g0; g < vb; g += gstride) {
-        const uint64_t gn = g + gstride;
-        if (gn < vb) nxt.load(S, gn, lo, hi, vb, n_total);
-        if constexpr (AGG) probe_group_agg<W, U>(tab, cur, pf, chk, acc);
-        else probe_group_pairs<W, U>(tab, cur, pf, chk, st, oc, acc);
-        cur = nxt;
     }
 }
 
@@ -232,87 +350,137 @@ __global__ void agg_table_init(AggSlot<W> *slots, uint64_t cap) {
 }
 
 template <int W, bool AGG>
-__global__ void __launch_bounds__(256) table_build_kernel(const void *R, uint64_t lo, uint64_t hi, uint64_t n_total,
-                                                          void *slots, uint64_t cap, TableSide *side,
-                                                          hj_counters *ctr, PartFilter pf) {
-    using U = typename Tup<W>::U;
+__global__ void __launch_bounds__(256) table_build_kernel(const void *R, uint64_t n, void *slots, uint64_t cap,
+                                                          TableSide *side, hj_counters *ctr, PartFilter pf) {
     constexpr int PV = Tup<W>::kPerVec;
-    uint64_t va = lo / PV, vb = (hi + PV - 1) / PV;
-    for (uint64_t v = va + blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; v < vb;
-         v += (uint64_t)gridDim.x * blockDim.x) {
-        U k[2], r[2];
-        load_vec<W>(R, v, n_total, k, r);
+    const uint64_t nvec = (n + PV - 1) / PV;
+    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+    bool repeat = false;
+    for (uint64_t v = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; v < nvec; v += stride) {
+        Group<W, 1> g;
+        g.load((const typename Tup<W>::Vec *)R, v & ~31ull, n);
 #pragma unroll
         for (int e = 0; e < PV; ++e) {
-            uint64_t t = v * PV + e;
-            if (t < lo || t >= hi) continue;
-            uint64_t h = key_hash<W>(k[e]);
+            if (!((g.valid >> e) & 1u)) continue;
+            const uint64_t h = key_hash<W>(g.key(e));
             if (!pf.keep(h)) continue;
-            bool ok = AGG ? agg_insert<W>((AggSlot<W> *)slots, cap, side, k[e], mix_a(r[e]), h)
-                          : pair_insert<W>((typename PairSlot<W>::S *)slots, cap, side, k[e], r[e], h);
+            const bool ok = AGG ? agg_insert<W>((AggSlot<W> *)slots, cap, side, g.key(e), mix_a(g.rid(e)), h)
+                                : pair_insert<W>((typename PairSlot<W>::S *)slots, (uint32_t)(cap / kBucketSlots<W>),
+                                                 side, g.key(e), g.rid(e), h, &repeat);
             if (!ok) atomicOr(&ctr->status, (unsigned long long)(AGG || cap <= kMaxPairWalk ? kStatusTableFull
                                                                                          : kStatusLongRun));
         }
     }
+    if (!AGG && __syncthreads_or(repeat) && threadIdx.x == 0) side->repeats = 1;
 }
 
-// Vectors per lane per probe group.
-template <int W> struct ProbeU {
-    static constexpr int value = 2;
-};
+template <int W> constexpr int kProbeVecs = kProbeItems / Tup<W>::kPerVec;
 
-// Pairs per warp in the probe's shared-memory staging buffer (exact output mode).
-constexpr unsigned kProbeStage = 256;
+// Pairs per warp in the probe's shared-memory staging buffer (exact output mode):
+// 4 KB, several times a group's pairs, so that the one address all warps claim
+// rows from sees an atomic per 512 (256) pairs.
+constexpr unsigned kProbeStageBytes = 4096;
+template <int W> constexpr unsigned kProbeStage = kProbeStageBytes / (2 * W);
 
-template <int W, bool AGG>
-__global__ void __launch_bounds__(256) table_probe_kernel(const void *S, uint64_t lo, uint64_t hi, uint64_t n_total,
-                                                          const void *slots, uint64_t cap, const TableSide *side,
-                                                          void *pairs, uint64_t pcap, RecArea ra, hj_counters *ctr,
-                                                          int chk, PartFilter pf, int dense) {
-    constexpr int PV = Tup<W>::kPerVec, U = ProbeU<W>::value;
-    const unsigned warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const unsigned nwarps = (gridDim.x * blockDim.x) >> 5;
-    const uint64_t va = lo / PV;
+// Shared memory of a probing warp: the staging buffer, then the queue of runs.
+template <int W> constexpr unsigned kProbeWarpBytes = kProbeStageBytes + sizeof(RunQueue<W>);
+
+template <int W, bool CHK>
+__global__ void __launch_bounds__(256, kProbeCtas) pair_probe_kernel(const void *S, uint64_t n, const void *slots,
+                                                            uint32_t nb, const TableSide *side, void *pairs,
+                                                            uint64_t pcap, hj_counters *ctr) {
+    using Vec = typename Tup<W>::Vec;
+    constexpr int PV = Tup<W>::kPerVec, U = kProbeVecs<W>;
+    const uint64_t g0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (32ull * U);
+    const uint64_t stride = (uint64_t)((gridDim.x * blockDim.x) >> 5) * (32 * U);
+    const uint64_t nvec = (n + PV - 1) / PV, whole = n / PV / (32 * U) * (32 * U);  // groups below `whole` are full
+    extern __shared__ __align__(16) unsigned char tp_smem[];
+    unsigned char *mine = tp_smem + (size_t)(threadIdx.x >> 5) * kProbeWarpBytes<W>;
+    RunQueue<W> &q = *(RunQueue<W> *)(mine + kProbeStageBytes);
+    uint32_t qn = 0;
     OutState st;
-    OutCtx oc{pairs, pcap, ctr, 0u, dense == 1};
-    extern __shared__ __align__(16) unsigned char tp_stage[];
-    if (dense == 2) {  // this warp's staging buffer
-        oc.stage = tp_stage + (size_t)(threadIdx.x >> 5) * kProbeStage * 2 * W;
-        oc.scap = kProbeStage;
-        st.used = 0;
-    }
+    OutCtx oc{pairs, pcap, ctr, 0u, false};
+    oc.stage = mine;
+    oc.scap = kProbeStage<W>;
+    st.used = 0;
     ProbeAcc acc;
-    if constexpr (AGG) {
-        AggTab<W> tab{(const AggSlot<W> *)slots, cap, side};
-        warp_probe<W, U, true>(tab, S, lo, hi, n_total, va + (uint64_t)warp * 32 * U, (uint64_t)nwarps * 32 * U,
-                               pf, chk != 0, st, oc, acc);
-    } else {
-        PairTab<W> tab{(const typename PairSlot<W>::S *)slots, cap, side->n_allones, 1u};
-        warp_probe<W, U, false>(tab, S, lo, hi, n_total, va + (uint64_t)warp * 32 * U, (uint64_t)nwarps * 32 * U,
-                                pf, chk != 0, st, oc, acc);
-        if (oc.stage) warp_stage_flush<W>(st, oc);
-        warp_finish(st, oc, ra);
+    const PairTab<W> tab{(const typename PairSlot<W>::S *)slots, nb, side->n_allones, side->repeats == 0};
+    Group<W, U> cur, nxt;
+    if (g0 < nvec) cur.load((const Vec *)S, g0, n);
+    uint64_t g = g0;
+    for (; g < whole; g += stride) {
+        nxt.load((const Vec *)S, g + stride, n);
+        probe_group_pairs<W, U, CHK, true>(tab, cur, q, qn, st, oc, acc);
+        cur = nxt;
     }
-    flush_acc(ctr, acc, AGG);
+    if (g < nvec) probe_group_pairs<W, U, CHK, false>(tab, cur, q, qn, st, oc, acc);  // the last group
+    while (qn) drain_runs<W, CHK>(tab, q, qn, min(qn, 32u), st, oc, acc);
+    warp_stage_flush<W>(st, oc);
+    if (CHK) flush_acc(ctr, acc, false);
 }
 
-hj_status table_create(hj_ctx *c, int width, int agg, uint64_t n_build, hj_table **out) {
+template <int W, bool CHK>
+__global__ void __launch_bounds__(256) agg_probe_kernel(const void *S, uint64_t n, const void *slots, uint64_t cap,
+                                                        const TableSide *side, hj_counters *ctr, PartFilter pf) {
+    using Vec = typename Tup<W>::Vec;
+    constexpr int PV = Tup<W>::kPerVec, U = 4 / PV;
+    const uint64_t nvec = (n + PV - 1) / PV;
+    const uint64_t g0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (32ull * U);
+    const uint64_t stride = (uint64_t)((gridDim.x * blockDim.x) >> 5) * (32 * U);
+    ProbeAcc acc;
+    for (uint64_t g = g0; g < nvec; g += stride) {
+        Group<W, U> cur;
+        cur.load((const Vec *)S, g, n);
+        probe_group_agg<W, U, CHK>((const AggSlot<W> *)slots, cap, side, cur, pf, acc);
+    }
+    flush_acc(ctr, acc, true);
+}
+
+// One CTA of 256 threads per `per_cta` items, at most `per_sm` CTAs for every SM.
+static unsigned items_grid(hj_ctx *c, uint64_t n, uint64_t per_cta, uint64_t per_sm) {
+    const uint64_t want = (n + per_cta - 1) / per_cta, most = (uint64_t)num_sms(c) * per_sm;
+    return (unsigned)(want < most ? (want ? want : 1) : most);
+}
+
+// Largest pair table that takes four slots per tuple (twice L2: larger ones are
+// bound by HBM sectors, not by the few longer runs).
+constexpr uint64_t kFastTableBytes = 256ull << 20;
+
+// An empty pair table, its side data and (ctr not NULL) a join's counters, all
+// but the sticky fault word.
+__global__ void __launch_bounds__(256) pair_table_init(ulonglong2 *slots, uint64_t n, TableSide *side, hj_counters *ctr) {
+    const uint64_t i0 = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+    for (uint64_t i = i0; i < n; i += (uint64_t)gridDim.x * blockDim.x) slots[i] = make_ulonglong2(~0ull, ~0ull);
+    if (i0 < sizeof(TableSide) / 8) ((unsigned long long *)side)[i0] = 0;
+    if (ctr && i0 < offsetof(hj_counters, fault) / 8) ((unsigned long long *)ctr)[i0] = 0;
+}
+
+hj_status table_create(hj_ctx *c, int width, int agg, uint64_t n_build, hj_table **out, bool zero_ctr) {
     *out = nullptr;
-    // Capacity: a power of two at least twice the build size (load factor <= 0.5).
+    // Capacity: a power of two at least twice the build size (load factor <= 0.5).  A
+    // pair table takes four slots per tuple (2 % of 4-byte buckets are then full, 5 %
+    // at three: 2^24 probes of 2^18 tuples 106 us against 123 us) unless the context
+    // has a memory budget, which keeps the smaller size it always had.
     uint64_t cap = 64;
     while (cap < 2 * n_build + 1) cap <<= 1;
     uint64_t slot_bytes = agg ? (width == 4 ? sizeof(AggSlot<4>) : sizeof(AggSlot<8>)) : 2ull * width;
+    if (!agg && !c->budget && 4 * n_build * slot_bytes <= kFastTableBytes) cap = std::max<uint64_t>(64, 4 * n_build);
     DevBuf slots(c), side(c);
     HJ_TRY(slots.alloc(cap * slot_bytes));
     HJ_TRY(side.alloc(sizeof(TableSide)));
-    HJ_CUDA(c, cudaMemsetAsync(side.p, 0, sizeof(TableSide), c->stream));
-    int grid = num_sms(c) * 4;
     if (!agg) {
-        HJ_CUDA(c, cudaMemsetAsync(slots.p, 0xFF, cap * slot_bytes, c->stream));
-    } else if (width == 4) {
-        HJ_LAUNCH(c, "agg_table_init", agg_table_init<4>, grid, 256, 0, slots.as<AggSlot<4>>(), cap);
+        const uint64_t n = cap * slot_bytes / 16;
+        HJ_LAUNCH(c, "pair_table_init", pair_table_init, items_grid(c, n, 1024, 8), 256, 0, slots.as<ulonglong2>(), n,
+                  side.as<TableSide>(), zero_ctr ? c->d_ctr : nullptr);
     } else {
-        HJ_LAUNCH(c, "agg_table_init", agg_table_init<8>, grid, 256, 0, slots.as<AggSlot<8>>(), cap);
+        if (zero_ctr) HJ_TRY(zero_counters(c));
+        HJ_CUDA(c, cudaMemsetAsync(side.p, 0, sizeof(TableSide), c->stream));
+        int grid = num_sms(c) * 4;
+        if (width == 4) {
+            HJ_LAUNCH(c, "agg_table_init", agg_table_init<4>, grid, 256, 0, slots.as<AggSlot<4>>(), cap);
+        } else {
+            HJ_LAUNCH(c, "agg_table_init", agg_table_init<8>, grid, 256, 0, slots.as<AggSlot<8>>(), cap);
+        }
     }
     hj_table *t = new hj_table();
     t->width = width;
@@ -332,14 +500,11 @@ void table_destroy(hj_ctx *c, hj_table *t) {
     delete t;
 }
 
-hj_status table_build(hj_ctx *c, hj_table *t, const void *R, uint64_t lo, uint64_t hi, uint64_t n_total,
-                      PartFilter pf) {
-    if (hi <= lo) return HJ_OK;
-    uint64_t nvec = (hi - lo) / (t->width == 4 ? 2 : 1) + 2;
-    uint64_t want = (nvec + 255) / 256;
-    int grid = (int)(want < (uint64_t)num_sms(c) * 8 ? (want ? want : 1) : (uint64_t)num_sms(c) * 8);
+hj_status table_build(hj_ctx *c, hj_table *t, const void *R, uint64_t n, PartFilter pf) {
+    if (!n) return HJ_OK;
+    const unsigned grid = items_grid(c, n, t->width == 4 ? 512 : 256, 32);
     TableSide *side = (TableSide *)t->side;
-#define HJ_TB(WW, AA) HJ_LAUNCH(c, "table_build", (table_build_kernel<WW, AA>), grid, 256, 0, R, lo, hi, n_total, t->slots, t->cap, side, c->d_ctr, pf)
+#define HJ_TB(WW, AA) HJ_LAUNCH(c, "table_build", (table_build_kernel<WW, AA>), grid, 256, 0, R, n, t->slots, t->cap, side, c->d_ctr, pf)
     if (t->width == 4) {
         if (t->agg) HJ_TB(4, true); else HJ_TB(4, false);
     } else {
@@ -349,26 +514,26 @@ hj_status table_build(hj_ctx *c, hj_table *t, const void *R, uint64_t lo, uint64
     return HJ_OK;
 }
 
-uint64_t table_probe_warps(hj_ctx *c, uint64_t n) {
-    const uint64_t per_cta_tuples = 8 * 32 * 8;  // 8 warps, 32 lanes, 8 tuples per lane group
-    uint64_t want = (n + per_cta_tuples - 1) / per_cta_tuples;
-    uint64_t maxg = (uint64_t)num_sms(c) * 8;
-    uint64_t grid = want < maxg ? (want ? want : 1) : maxg;
-    return grid * 8;
-}
-
-hj_status table_probe(hj_ctx *c, const hj_table *t, const void *S, uint64_t lo, uint64_t hi, uint64_t n_total,
-                      void *pairs, uint64_t pcap, int checksum, RecArea ra, PartFilter pf, hj_counters *ctr, int dense) {
-    if (hi <= lo) return HJ_OK;
-    if (!ctr) ctr = c->d_ctr;
-    const unsigned grid = (unsigned)(table_probe_warps(c, hi - lo) / 8);
+hj_status table_probe(hj_ctx *c, const hj_table *t, const void *S, uint64_t n, void *pairs, uint64_t pcap,
+                      int checksum, PartFilter pf, hj_counters *ctr) {
+    if (!n) return HJ_OK;
     const TableSide *side = (const TableSide *)t->side;
-    const size_t smem = dense == 2 && !t->agg ? (size_t)8 * kProbeStage * 2 * t->width : 0;
-#define HJ_TP(WW, AA) HJ_LAUNCH(c, "table_probe", (table_probe_kernel<WW, AA>), grid, 256, smem, S, lo, hi, n_total, t->slots, t->cap, side, pairs, pcap, ra, ctr, checksum, pf, dense)
+#define HJ_TP(WW, CC)                                                                                               \
+    do {                                                                                                            \
+        if (t->agg)                                                                                                 \
+            HJ_LAUNCH(c, "table_probe", (agg_probe_kernel<WW, CC>), items_grid(c, n, 1024, 8), 256, 0, S, n,        \
+                      t->slots, t->cap, side, ctr, pf);                                                             \
+        else {                                                                                                      \
+            HJ_TRY(allow_max_smem(c, (const void *)pair_probe_kernel<WW, CC>));                                     \
+            HJ_LAUNCH(c, "table_probe", (pair_probe_kernel<WW, CC>), items_grid(c, n, 256 * kProbeItems, kProbeCtas), 256,   \
+                      8 * kProbeWarpBytes<WW>, S, n, t->slots, (uint32_t)(t->cap / kBucketSlots<WW>), side, pairs,     \
+                      pcap, ctr);                                                                                   \
+        }                                                                                                           \
+    } while (0)
     if (t->width == 4) {
-        if (t->agg) HJ_TP(4, true); else HJ_TP(4, false);
+        if (checksum) HJ_TP(4, true); else HJ_TP(4, false);
     } else {
-        if (t->agg) HJ_TP(8, true); else HJ_TP(8, false);
+        if (checksum) HJ_TP(8, true); else HJ_TP(8, false);
     }
 #undef HJ_TP
     return HJ_OK;
@@ -1047,7 +1212,6 @@ __global__ void __launch_bounds__(NT, 2048 / NT / 2) partition_join_kernel(
     constexpr int PV = Tup<W>::kPerVec, U = 2, IT = U * PV;
     constexpr uint32_t G = SoaTab<W>::G;
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ TableSide side;
     __shared__ int s_full;
     __shared__ unsigned long long s_p;
     const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
@@ -1109,7 +1273,6 @@ __global__ void __launch_bounds__(NT, 2048 / NT / 2) partition_join_kernel(
                 }
             }
             if (threadIdx.x == 0) {
-                side.n_allones = side.agg_cnt = side.agg_suma = side.full = 0;
                 s_full = 0;
             }
             __syncthreads();

@@ -31,15 +31,17 @@ static_assert(sizeof(StaticHeader) <= kHeaderBytes, "header does not fit");
 constexpr uint64_t kStaticMaxWalk = 1ull << 16;  // longest insert walk of the static table
 
 template <int W>
-__global__ void static_build_kernel(const void *R, uint64_t n, void *slots, uint64_t cap, StaticHeader *hdr) {
+__global__ void static_build_kernel(const void *R, uint64_t n, void *slots, uint32_t nb, StaticHeader *hdr) {
     using U = typename Tup<W>::U;
     for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < n; t += (uint64_t)gridDim.x * blockDim.x) {
         const U k = ((const U *)R)[2 * t], r = ((const U *)R)[2 * t + 1];
         // (no key-list form here: a longer walk bound than the library's joins, so
         // that keys repeated some thousand times still work)
-        if (!pair_insert<W>((typename PairSlot<W>::S *)slots, cap, &hdr->side, k, r, key_hash<W>(k), kStaticMaxWalk))
+        bool repeat = false;  // (the probe below always walks whole runs)
+        if (!pair_insert<W>((typename PairSlot<W>::S *)slots, nb, &hdr->side, k, r, key_hash<W>(k), &repeat,
+                            kStaticMaxWalk))
             atomicOr(&hdr->ctr.status,
-                     (unsigned long long)(cap <= kStaticMaxWalk ? kStatusTableFull : kStatusLongRun));
+                     (unsigned long long)((uint64_t)nb * kBucketSlots<W> <= kStaticMaxWalk ? kStatusTableFull : kStatusLongRun));
     }
 }
 
@@ -63,7 +65,7 @@ __device__ __forceinline__ void dense_append(StaticHeader *hdr, void *pairs, uin
 }
 
 template <int W>
-__global__ void static_probe_kernel(const void *S, uint64_t n, const void *slots, uint64_t cap, StaticHeader *hdr,
+__global__ void static_probe_kernel(const void *S, uint64_t n, const void *slots, uint32_t nb, StaticHeader *hdr,
                                     void *pairs, uint64_t pcap) {
     using U = typename Tup<W>::U;
     using PS = PairSlot<W>;
@@ -81,7 +83,7 @@ __global__ void static_probe_kernel(const void *S, uint64_t n, const void *slots
         U first = 0;
         if (valid) {
             const uint64_t bs = mix_b(r);
-            pair_lookup<W>(sl, cap, nall, k, key_hash<W>(k), 1u, [&](U rid) {
+            pair_lookup<W>(sl, nb, nall, k, key_hash<W>(k), [&](U rid) {
                 if (cnt == 0) first = rid;
                 ++cnt;
                 const uint64_t a = mix_a(rid);
@@ -96,16 +98,16 @@ __global__ void static_probe_kernel(const void *S, uint64_t n, const void *slots
             const int L = __ffs(multi) - 1;
             multi &= multi - 1;
             const U kk = __shfl_sync(0xffffffffu, k, L), ss = __shfl_sync(0xffffffffu, r, L);
-            const uint64_t b0 = bucket_of<W>(key_hash<W>(kk), cap);
+            const uint64_t cap = (uint64_t)nb * kBucketSlots<W>;
+            const uint64_t b0 = (uint64_t)pair_bucket<W>(key_hash<W>(kk), nb) * kBucketSlots<W>;
             for (uint64_t off = 0; off < cap; off += 32) {
-                const bool inr = off + lane < cap;
                 uint64_t idx = b0 + off + lane;
                 if (idx >= cap) idx -= cap;
-                const typename PS::S s = inr ? sl[idx] : PS::empty();
-                const unsigned emp = __ballot_sync(0xffffffffu, !inr || PS::is_empty(s));
-                const unsigned before = emp ? ((emp & (0u - emp)) - 1u) : 0xffffffffu;
-                dense_append<W>(hdr, pairs, pcap, ((before >> lane) & 1u) && PS::key(s) == kk, PS::rid(s), ss);
-                if (emp) break;
+                const typename PS::S s = off + lane < cap ? sl[idx] : PS::empty();
+                bool end;
+                const bool run = run_step<W>(s, &end);
+                dense_append<W>(hdr, pairs, pcap, run && PS::key(s) == kk, PS::rid(s), ss);
+                if (end) break;
             }
             if (kk == Tup<W>::kAllOnes)
                 for (unsigned long long i = 0; i < nall; i += 32)
@@ -175,16 +177,17 @@ extern "C" hj_status hj_join_static(const hj_rel *R, const hj_rel *S, void *cuda
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
     if (sms <= 0) sms = 1;
+    const uint32_t nb = (uint32_t)(table_bytes / 32);
     const uint64_t bgrid = R->n ? (R->n + 255) / 256 : 1;
     const unsigned gb = (unsigned)(bgrid < (uint64_t)sms * 8 ? bgrid : (uint64_t)sms * 8);
     const unsigned gp = (unsigned)sms * 4;
     if (e == cudaSuccess) {
         if (W == 4) {
-            if (R->n) static_build_kernel<4><<<gb, 256, 0, stream>>>(R->tuples, R->n, slots, cap, hdr);
-            if (S->n) static_probe_kernel<4><<<gp, 256, 0, stream>>>(S->tuples, S->n, slots, cap, hdr, pairs, pairs_cap);
+            if (R->n) static_build_kernel<4><<<gb, 256, 0, stream>>>(R->tuples, R->n, slots, nb, hdr);
+            if (S->n) static_probe_kernel<4><<<gp, 256, 0, stream>>>(S->tuples, S->n, slots, nb, hdr, pairs, pairs_cap);
         } else {
-            if (R->n) static_build_kernel<8><<<gb, 256, 0, stream>>>(R->tuples, R->n, slots, cap, hdr);
-            if (S->n) static_probe_kernel<8><<<gp, 256, 0, stream>>>(S->tuples, S->n, slots, cap, hdr, pairs, pairs_cap);
+            if (R->n) static_build_kernel<8><<<gb, 256, 0, stream>>>(R->tuples, R->n, slots, nb, hdr);
+            if (S->n) static_probe_kernel<8><<<gp, 256, 0, stream>>>(S->tuples, S->n, slots, nb, hdr, pairs, pairs_cap);
         }
         e = cudaGetLastError();
     }
