@@ -445,12 +445,11 @@ uint64_t hj_debug_bytes_in_use(const hj_ctx *ctx);
  * change: no GPU fault is involved.  HJ_E_INVALID for a NULL context. */
 hj_status hj_debug_wait_limit(hj_ctx *ctx, uint64_t n);
 /* Test and measurement hook: which kernel scatters a padded partition pass at
- * 2^9 .. 2^11 digits.  HJ_SCATTER_AUTO (the default) takes the ring scatter where
- * it measured faster than the region scatter (4-byte tuples at 2^10 and 2^11
- * digits, 8-byte tuples at 2^9 .. 2^11) and the region scatter elsewhere; HJ_SCATTER_REGION and HJ_SCATTER_RING force one
- * (other fan-outs always take the region scatter).  Results are identical either
- * way; only the kernel changes.  HJ_E_INVALID for a NULL context or another
- * value. */
+ * 2^9 .. 2^11 digits.  HJ_SCATTER_AUTO (the default) takes the region scatter, which
+ * measured faster at every width and fan-out, unless hj_debug_wait_limit limits the
+ * waits (only the ring scatter has any); HJ_SCATTER_REGION and HJ_SCATTER_RING force
+ * one (other fan-outs always take the region scatter).  Results are identical either
+ * way; only the kernel changes.  HJ_E_INVALID for a NULL context or another value. */
 #define HJ_SCATTER_AUTO 0
 #define HJ_SCATTER_REGION 1
 #define HJ_SCATTER_RING 2
