@@ -160,7 +160,7 @@ hj_status launch_wave(hj_ctx *c, int W, const JoinSlot *slots, bool agg, bool ch
     w.oversize = newbuf(c, w);
     HJ_TRY(w.oversize->alloc(std::max<uint64_t>(ntasks, 1) * 4));
     RecArea ra{nullptr, nullptr, 0};
-    HJ_TRY(partition_join(c, W, agg, w.tasks->as<PartTask>(), ntasks, slots, 8192, chk, w.oversize->as<uint32_t>(), ra,
+    HJ_TRY(partition_join(c, W, agg, w.tasks->as<PartTask>(), ntasks, ntasks, slots, 8192, chk, w.oversize->as<uint32_t>(), ra,
                           agg ? nullptr : stage.p, kStagePairs));
     return HJ_OK;
 }

@@ -80,13 +80,14 @@ uint64_t tail_split_from(hj_ctx *c, int width, int agg, uint64_t NP, uint64_t ex
 
 // Per-partition join (Alg. 2's "apply SHJ on each partition pair") with the
 // table in shared memory; persistent CTAs take tasks from c->d_ctr->work (which
-// must be zero at launch).  Tasks whose table does not fit are appended to
+// must be zero at launch), one ahead while more than two per CTA of the first `lead`
+// (the ones that are sure to hold rows) remain.  Tasks whose table does not fit are appended to
 // `oversize` (task indices) and counted in c->d_ctr->n_oversize.  Pairs go to
 // each task's join slot: with `stage` (a staging area of scap pairs per warp, for
 // partition_join_warps(c) warps) by
 // exact claims, otherwise by per-warp chunks recorded in `ra`.
-hj_status partition_join(hj_ctx *c, int width, int agg, const PartTask *tasks, uint64_t ntasks, const JoinSlot *slots,
-                         uint64_t expect_r, int checksum, uint32_t *oversize, RecArea ra, void *stage,
+hj_status partition_join(hj_ctx *c, int width, int agg, const PartTask *tasks, uint64_t ntasks, uint64_t lead,
+                         const JoinSlot *slots, uint64_t expect_r, int checksum, uint32_t *oversize, RecArea ra, void *stage,
                          uint32_t scap);
 uint64_t partition_join_warps(hj_ctx *c);
 uint64_t partition_join_ctas(hj_ctx *c, int width, int agg, uint64_t expect_r);

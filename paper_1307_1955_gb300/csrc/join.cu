@@ -584,21 +584,23 @@ __device__ __forceinline__ typename HashT<W>::type hashw(typename Tup<W>::U k) {
 // Bucketised open addressing in shared memory for one partition pair.  Bucket b is
 // G slots (G = 4 for 4-byte tuples, 2 for 8-byte): its G keys are 16 bytes of the
 // key region and its G rids 16 bytes of the rid region (separate regions, so that
-// the key loads of random buckets spread over all shared-memory banks).
+// the key loads of random buckets spread over all shared-memory banks).  (Two keys of
+// 4 bytes per bucket load in half the time, but one hit in six is then in a bucket
+// that overflowed, one in twenty with four, and following those costs more.)
 // Every real key of partition p hashes to p, so a key that hashes to another
 // partition can never be stored or probed: it marks empty slots (no value of the
 // key domain needs reserving).  A key's run starts at its home bucket and moves
-// linearly over buckets; a bucket's overflow bit records that some insert moved
-// past it, so a lookup stops at the first bucket that has an empty slot or no
-// overflow bit.
+// linearly over buckets.  A bucket's 16-bit count says how many inserts tried it:
+// the count before its own tells an insert its slot (or, from G on, to move to the
+// next bucket), and a lookup stops at the first bucket tried by no more than G.
 template <int W> struct SoaTab {
     using T = typename Tup<W>::U;
     static constexpr uint32_t G = 16 / W;
     uint32_t nb;     // buckets
     T empty;
-    const uint32_t *ovf;
+    const uint16_t *cnt;  // inserts that tried the bucket (each once)
 
-    __device__ __forceinline__ bool overflowed(uint32_t b) const { return (ovf[b >> 5] >> (b & 31)) & 1u; }
+    __device__ __forceinline__ bool overflowed(uint32_t b) const { return cnt[b] > G; }
     // keys (half 0) or rids (half 1) of bucket b.  Plain loads through the
     // shared-memory pointers: the compiler orders them with the barriers and may
     // overlap the independent lookups of a thread's items.
@@ -715,6 +717,8 @@ template <int W> struct ChunkSink {
     using T = typename Tup<W>::U;
     OutState st;
     OutCtx oc;
+    typename PairVec<W>::T *open = nullptr;  // the open chunk (append_runs)
+    unsigned room = 0;                       // rows of it that append_runs may fill without a test
     unsigned join = ~0u;
     const JoinSlot *slots;
     RecArea ra;
@@ -724,8 +728,13 @@ template <int W> struct ChunkSink {
         st = OutState();
         oc = OutCtx{slots[j].pairs, slots[j].pcap, slots[j].ctr, j, false};
         join = j;
+        room = 0;
     }
-    __device__ __forceinline__ void append(bool has, T a, T b) { warp_append<W>(st, oc, has, a, b); }
+    __device__ __forceinline__ void append(bool has, T a, T b) {
+        warp_append<W>(st, oc, has, a, b);
+        open = (typename PairVec<W>::T *)oc.pairs + st.base;
+        set_room();
+    }
     // one append for all single-match items of a group
     template <int IT>
     __device__ __forceinline__ void append_group(const uint32_t *cnt, const T *first, const T *r) {
@@ -762,62 +771,70 @@ template <int W> struct ChunkSink {
         }
         st.pairs += tot;
     }
-    // one append for all single-match items of a group (at most 32 * IT pairs, so
-    // at most one new chunk): item-major positions, so that each store instruction
-    // writes consecutive slots; capacity tested once per group
     template <int IT>
     __device__ __forceinline__ void append_runs(const uint32_t *cnt, const T *first, const T *r) {
+        bool found[IT];
+#pragma unroll
+        for (int i = 0; i < IT; ++i) found[i] = cnt[i] == 1;
+        append_found<IT>(found, first, r);
+    }
+    // one append for all items of a group with a match (at most 32 * IT pairs, so at
+    // most one new chunk): item-major positions, so that each store instruction
+    // writes consecutive slots; capacity tested once per chunk
+    template <int IT>
+    __device__ __forceinline__ void append_found(const bool *found, const T *first, const T *r) {
+        using P = typename PairVec<W>::T;
         const unsigned lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
         unsigned m[IT], tot = 0;
 #pragma unroll
         for (int i = 0; i < IT; ++i) {
-            m[i] = __ballot_sync(0xffffffffu, cnt[i] == 1);
+            m[i] = __ballot_sync(0xffffffffu, found[i]);
             tot += __popc(m[i]);
         }
-        if (!tot) return;
-        const unsigned room = kChunkPairs - st.used;
+        if (tot <= room) {  // (warp-uniform) the open chunk has room, all of it inside the buffer
+            P *dst = open + st.used;
+#pragma unroll
+            for (int i = 0; i < IT; ++i) {
+                if (found[i]) {
+                    if constexpr (W == 4) dst[__popc(m[i] & lt)] = make_uint2(first[i], r[i]);
+                    else dst[__popc(m[i] & lt)] = make_ulonglong2(first[i], r[i]);
+                }
+                dst += __popc(m[i]);
+            }
+            st.used += tot;
+            st.pairs += tot;
+            room -= tot;
+            return;
+        }
+        const unsigned left = kChunkPairs - st.used;
         unsigned long long nb = 0;
-        if (tot > room) {
+        if (tot > left) {
             if (lane == 0) nb = atomicAdd(&oc.ctr->cursor, (unsigned long long)kChunkPairs);
             nb = __shfl_sync(0xffffffffu, nb, 0);
         }
         const unsigned long long c0 = st.base + st.used;
-        const bool safe = c0 + (tot < room ? tot : room) <= oc.pcap && (tot <= room || nb + (tot - room) <= oc.pcap);
         unsigned run = 0;
-        if (safe) {  // (warp-uniform) every position is inside the buffer
-            // pair idx of the group goes to c0 + idx in the open chunk, else to
-            // nb + (idx - room) in the new one: one base address per item (the
-            // second base is only used for idx >= room, so its wrap is harmless)
-            using P = typename std::conditional<W == 4, uint2, ulonglong2>::type;
-            const uint64_t a0 = (uint64_t)oc.pairs + c0 * sizeof(P);
-            const uint64_t a1 = (uint64_t)oc.pairs + (nb - room) * sizeof(P);
 #pragma unroll
-            for (int i = 0; i < IT; ++i) {
-                const unsigned idx = run + __popc(m[i] & lt);
-                P *dst = (P *)((idx < room ? a0 : a1) + (uint64_t)idx * sizeof(P));
-                if (cnt[i] == 1) {
-                    if constexpr (W == 4) *dst = make_uint2(first[i], r[i]);
-                    else *dst = make_ulonglong2(first[i], r[i]);
-                }
-                run += __popc(m[i]);
-            }
-        } else {
-#pragma unroll
-            for (int i = 0; i < IT; ++i) {
-                const unsigned idx = run + __popc(m[i] & lt);
-                const unsigned long long pos = idx < room ? c0 + idx : nb + (idx - room);
-                if (cnt[i] == 1 && pos < oc.pcap) PairOut<W>::put(oc.pairs, pos, first[i], r[i]);
-                run += __popc(m[i]);
-            }
+        for (int i = 0; i < IT; ++i) {
+            const unsigned idx = run + __popc(m[i] & lt);
+            const unsigned long long pos = idx < left ? c0 + idx : nb + (idx - left);
+            if (found[i] && pos < oc.pcap) PairOut<W>::put(oc.pairs, pos, first[i], r[i]);
+            run += __popc(m[i]);
         }
-        if (tot > room) {
+        if (tot > left) {
             st.base = nb;
-            st.used = tot - room;
+            st.used = tot - left;
             st.claimed = true;
         } else {
             st.used += tot;
         }
         st.pairs += tot;
+        open = (P *)oc.pairs + st.base;
+        set_room();
+    }
+    // pairs that fit the open chunk without a test of the buffer's end
+    __device__ __forceinline__ void set_room() {
+        room = st.claimed && st.base + kChunkPairs <= oc.pcap ? kChunkPairs - st.used : 0u;
     }
     __device__ __forceinline__ hj_counters *ctr() const { return oc.ctr; }
     __device__ __forceinline__ void end_task() {}
@@ -898,6 +915,13 @@ template <int W> struct WarpStageSink {
     __device__ __forceinline__ void append_runs(const uint32_t *cnt, const T *first, const T *r) {
         append_group<IT>(cnt, first, r);
     }
+    template <int IT>
+    __device__ __forceinline__ void append_found(const bool *found, const T *first, const T *r) {
+        uint32_t cnt[IT];
+#pragma unroll
+        for (int i = 0; i < IT; ++i) cnt[i] = found[i];
+        append_group<IT>(cnt, first, r);
+    }
     __device__ __forceinline__ hj_counters *ctr() const { return slots[join].ctr; }
     __device__ __forceinline__ void end_task() {}
     __device__ __forceinline__ void finish() { flush(); }
@@ -906,10 +930,9 @@ template <int W> struct WarpStageSink {
 // One group of IT probe items against the table, in phases so that the items'
 // shared-memory loads overlap: every item's home bucket (keys), then the match
 // masks and the first match's rid (one indexed load).  cnt[i] and first[i] cover
-// the home bucket only.  Inserts fill a bucket's slots in order and slots never
-// empty again, and an insert moves past a bucket only while it is full, so a run
-// goes on past the home bucket only if the bucket's last slot is taken AND its
-// overflow bit is set: bit i of the returned mask marks such an item (with at
+// the home bucket only.  Inserts fill a bucket's slots in order and move past it
+// only once it is full, so a run goes on past the home bucket only if the bucket's
+// last slot is taken AND more inserts tried it than it has slots: bit i of the returned mask marks such an item (with at
 // most one home match; an item with several takes the whole-run walk instead).
 // Items with live[i] false match nothing.
 template <int W, int IT>
@@ -947,11 +970,19 @@ constexpr uint32_t kMaxSmemWalk = 64;
 // run goes on past a full home bucket).
 constexpr uint32_t kWalkQ = 64;
 
-// Shared-memory layout of the join kernel: table slots (cap_max x slot bytes),
-// the overflow bitmap, then each warp's walk queue (kWalkQ keys, kWalkQ rids).
-__host__ __device__ constexpr uint32_t walkq_offset(uint32_t cap_max, uint32_t slot_bytes) {
-    return (cap_max * slot_bytes + (cap_max / 2 / 32 + 1) * 4 + 16 + 15) / 16 * 16;
+// Shared-memory layout of the join kernel: table slots (cap_max x slot bytes), the
+// buckets' counts (two bytes each; an aggregate table: its overflow bitmap),
+// then each warp's walk queue (kWalkQ keys, kWalkQ rids).
+__host__ __device__ constexpr uint32_t bucket_info_bytes(uint32_t cap, int width, bool agg) {
+    return agg ? (cap / 2 / 32 + 1) * 4 + 16 : cap * (uint32_t)width / 8;
 }
+__host__ __device__ constexpr uint32_t walkq_offset(uint32_t cap_max, uint32_t slot_bytes, int width, bool agg) {
+    return (cap_max * slot_bytes + bucket_info_bytes(cap_max, width, agg) + 15) / 16 * 16;
+}
+
+// Probe rows of the next task asked into L2 (64 KB of 16-byte vectors).
+constexpr uint32_t kAheadVecs = 4096;
+__device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 // The walks of n <= 32 queued items, one per lane: each lane follows its key's run
 // from the bucket after its home and emits every match found there.  A walk is
@@ -1004,17 +1035,12 @@ __device__ __forceinline__ void drain_walks(const SoaTab<W> &tab, const typename
 
 template <int W, int U, class Sink>
 __device__ __forceinline__ void probe_fast(const SoaTab<W> &tab, const typename Tup<W>::Vec *Sv, uint32_t nsv,
-                                           Sink &sink, unsigned warp, unsigned nwarps, unsigned lane,
-                                           typename Tup<W>::U *wqk, typename Tup<W>::U *wqr) {
+                                           Sink &sink, uint32_t g, uint32_t gstride, unsigned lane,
+                                           typename Tup<W>::U *wqk, typename Tup<W>::U *wqr, uint32_t qn) {
     using T = typename Tup<W>::U;
     using Vec = typename Tup<W>::Vec;
     constexpr int PV = Tup<W>::kPerVec, IT = U * PV;
-    // runs that go on past a full home bucket are queued and walked 32 at a time
-    constexpr bool kQueue = true;
-    const uint32_t gstride = nwarps * 32u * U;
     const unsigned lt = (1u << lane) - 1u;
-    uint32_t g = warp * 32u * U;
-    uint32_t qn = 0;  // queued walks (warp-uniform)
     Vec cur[U], nxt[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -1045,21 +1071,6 @@ __device__ __forceinline__ void probe_fast(const SoaTab<W> &tab, const typename 
         uint32_t cnt[IT];
         T first[IT];
         const uint32_t walk = probe_items<W, IT>(tab, k, live, cnt, first);
-        if constexpr (!kQueue) {
-            // walked at once: the run's further matches join the item's count (and
-            // an item with several then takes the whole-run walk below)
-            if (walk) {
-#pragma unroll
-                for (int i = 0; i < IT; ++i) {
-                    if (!((walk >> i) & 1u)) continue;
-                    const uint32_t h = part_bucket<W>(k[i], tab.nb);
-                    T f2 = 0;
-                    const uint32_t c2 = soa_lookup<W>(tab, k[i], h + 1 == tab.nb ? 0 : h + 1, &f2);
-                    if (cnt[i] == 0) first[i] = f2;
-                    cnt[i] += c2;
-                }
-            }
-        }
         sink.template append_runs<IT>(cnt, first, r);
         // several home matches (duplicate build keys): the whole warp walks each such run
         bool multi_any = false;
@@ -1079,7 +1090,7 @@ __device__ __forceinline__ void probe_fast(const SoaTab<W> &tab, const typename 
             }
         }
         // runs that go on past the home bucket: queued, walked 32 at a time
-        if (kQueue && __any_sync(0xffffffffu, walk != 0)) {
+        if (__any_sync(0xffffffffu, walk != 0)) {
 #pragma unroll
             for (int i = 0; i < IT; ++i) {
                 const bool w = (walk >> i) & 1u;
@@ -1101,10 +1112,123 @@ __device__ __forceinline__ void probe_fast(const SoaTab<W> &tab, const typename 
 #pragma unroll
         for (int u = 0; u < U; ++u) cur[u] = nxt[u];
     }
-    if (kQueue && qn) {
+    if (qn) {
         __syncwarp();
         drain_walks<W>(tab, wqk, wqr, qn, sink);
     }
+}
+
+// Whether no key is twice in the table: every thread of the CTA compares the keys
+// of its buckets, and of a bucket that overflowed with those its run goes on to.
+template <int W, int NT> __device__ __forceinline__ bool keys_repeat(const SoaTab<W> &t) {
+    using T = typename Tup<W>::U;
+    constexpr uint32_t G = SoaTab<W>::G;
+    bool dup = false;
+    for (uint32_t b = threadIdx.x; b < t.nb; b += NT) {
+        T k[G];
+        t.ld(b, 0, k);
+#pragma unroll
+        for (uint32_t i = 0; i < G; ++i)
+#pragma unroll
+            for (uint32_t j = i + 1; j < G; ++j) dup |= k[i] == k[j] && k[j] != t.empty;
+        uint32_t c = b;
+        for (uint32_t it = 1; it < t.nb && t.overflowed(c); ++it) {
+            c = c + 1 == t.nb ? 0 : c + 1;
+            T o[G];
+            t.ld(c, 0, o);
+#pragma unroll
+            for (uint32_t i = 0; i < G; ++i)
+#pragma unroll
+                for (uint32_t j = 0; j < G; ++j) dup |= k[i] == o[j] && o[j] != t.empty;
+        }
+    }
+    return dup;
+}
+
+// Probe of a table whose keys are all different, over whole groups of U vectors per
+// lane (the rest goes through probe_fast): a match in the home bucket ends the search,
+// so an item is its bucket's four (two) compares, a select, and one rid.  Only an item
+// without a match whose home bucket overflowed is queued (about 1 %, against 3 % when
+// keys may repeat).  What bounds it: instructions and the shared-memory pipe (a bucket
+// of random lanes takes 10.3 cycles per warp), each at 55 %, and the latency that 20
+// warps leave open.  A join of 2^22 with 2^25 4-byte tuples issues 84e6 warp
+// instructions, 128e6 through the general loop; 2^24 x 2^28 1020 -> 828 us.
+template <int W, int U, class Sink>
+__device__ __forceinline__ void probe_unique(const SoaTab<W> &tab, const typename Tup<W>::Vec *Sv, uint32_t nsv,
+                                             Sink &sink, unsigned warp, unsigned nwarps, unsigned lane,
+                                             typename Tup<W>::U *wqk, typename Tup<W>::U *wqr) {
+    using T = typename Tup<W>::U;
+    using Vec = typename Tup<W>::Vec;
+    constexpr int PV = Tup<W>::kPerVec, IT = U * PV;
+    constexpr uint32_t G = SoaTab<W>::G;
+    const uint32_t gstride = nwarps * 32u * U, whole = nsv / (32u * U) * (32u * U);
+    const unsigned lt = (1u << lane) - 1u;
+    uint32_t g = warp * 32u * U, qn = 0;
+    Vec nxt[U];
+    if (g < whole)
+#pragma unroll
+        for (int u = 0; u < U; ++u) nxt[u] = ld_stream(Sv + g + u * 32u + lane);
+    for (; g < whole; g += gstride) {
+        T k[IT], r[IT];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if constexpr (W == 4) {
+                k[2 * u] = nxt[u].x; r[2 * u] = nxt[u].y; k[2 * u + 1] = nxt[u].z; r[2 * u + 1] = nxt[u].w;
+            } else {
+                k[u] = nxt[u].x; r[u] = nxt[u].y;
+            }
+        }
+        // (the group in registers covers part of the loads' latency, L2 the rest)
+        const uint32_t pv = g + 3u * gstride + lane * 8u;
+        if (lane < 4u * U && pv < nsv) prefetch_l2(Sv + pv);
+        if (g + gstride < whole)
+#pragma unroll
+            for (int u = 0; u < U; ++u) nxt[u] = ld_stream(Sv + g + gstride + u * 32u + lane);
+        uint32_t home[IT];
+        T kb[IT][G], first[IT];
+#pragma unroll
+        for (int i = 0; i < IT; ++i) {
+            home[i] = part_bucket<W>(k[i], tab.nb);
+            tab.ld(home[i], 0, kb[i]);
+        }
+        bool found[IT], w[IT], anyw = false;
+#pragma unroll
+        for (int i = 0; i < IT; ++i) {
+            uint32_t sl = home[i] * G + (G - 1);
+            bool f = kb[i][G - 1] == k[i];
+#pragma unroll
+            for (int q = (int)G - 2; q >= 0; --q) {
+                const bool h = kb[i][q] == k[i];
+                sl = h ? home[i] * G + q : sl;
+                f |= h;
+            }
+            found[i] = f;
+            first[i] = tab.rptr[sl];
+            w[i] = !f && kb[i][G - 1] != tab.empty && tab.overflowed(home[i]);
+            anyw |= w[i];
+        }
+        sink.template append_found<IT>(found, first, r);
+        if (__any_sync(0xffffffffu, anyw)) {
+#pragma unroll
+            for (int i = 0; i < IT; ++i) {
+                const unsigned wm = __ballot_sync(0xffffffffu, w[i]);
+                if (!wm) continue;
+                if (w[i]) {
+                    const uint32_t pos = qn + (uint32_t)__popc(wm & lt);
+                    wqk[pos] = k[i];
+                    wqr[pos] = r[i];
+                }
+                qn += (uint32_t)__popc(wm);
+                if (qn >= 32) {
+                    __syncwarp();
+                    drain_walks<W>(tab, wqk + (qn - 32), wqr + (qn - 32), 32, sink);
+                    qn -= 32;
+                }
+            }
+        }
+    }
+    // the slice's last, partial group: a warp's turn if it is the next of its groups
+    probe_fast<W, 1>(tab, Sv, nsv, sink, g == whole ? whole : nsv, 32u, lane, wqk, wqr, qn);
 }
 
 // Bytes per slot of a partition's shared-memory aggregate table: the key, the
@@ -1150,12 +1274,14 @@ template <int W> struct AggSoa {
             v[0] = x.x; v[1] = x.y;
         }
     }
-    // Add m build tuples of key k (a = the sum of their A(rid), used with
-    // checksums).  The slot of k is the first slot of its run that holds k, else
-    // the first empty one, claimed by CAS: slots only ever go from empty to a key,
-    // so two inserts of the same key always meet in one slot.  False if every
-    // bucket is full.
-    __device__ __forceinline__ bool insert(T k, uint32_t m, uint64_t a) const {
+    // Add a build tuple of key k (a = A(rid), used with checksums).  The slot of k is
+    // the first slot of its run that holds k, else the first empty one, claimed by
+    // CAS: slots only ever go from empty to a key, so two inserts of the same key
+    // always meet in one slot.  The 64-bit sum takes two 32-bit adds, the carry out of
+    // the low one with the high one (exact modulo 2^64 whatever the order): the shared
+    // memory adds 32-bit words of equal keys by itself, while one 64-bit add is a
+    // loop of CAS that equal keys repeat.  False if every bucket is full.
+    __device__ __forceinline__ bool insert(T k, uint64_t a) const {
         uint32_t b = part_bucket<W>(k, nb);
         for (uint32_t it = 0; it < nb; ++it) {
             volatile T *kb = keys + b * G;
@@ -1174,8 +1300,12 @@ template <int W> struct AggSoa {
                     hit = emp;
                 }
                 if (hit < 0) break;  // full bucket without k
-                atomicAdd(&cnt[b * G + hit], m);
-                if (suma) atomicAdd(&suma[b * G + hit], (unsigned long long)a);
+                atomicAdd(&cnt[b * G + hit], 1u);
+                if (suma) {
+                    uint32_t *w = (uint32_t *)&suma[b * G + hit];
+                    const uint32_t lo = (uint32_t)a, old = atomicAdd(&w[0], lo);
+                    atomicAdd(&w[1], (uint32_t)(a >> 32) + (old + lo < lo ? 1u : 0u));
+                }
                 return true;
             }
             atomicOr(&ovf[b >> 5], 1u << (b & 31));
@@ -1203,17 +1333,22 @@ template <int W> struct AggSoa {
     }
 };
 
+// CTAs per SM of the join kernel's launch shapes.
+__host__ __device__ constexpr int join_ctas(int nt) { return nt > 512 ? 1 : 2; }
+
 template <int W, bool AGG, int NT, class Sink, bool FAST>
-__global__ void __launch_bounds__(NT, 2048 / NT / 2) partition_join_kernel(
-    const PartTask *tasks, uint64_t ntasks, const JoinSlot *slots, hj_counters *work, uint32_t cap_max, RecArea ra,
+__global__ void __launch_bounds__(NT, join_ctas(NT)) partition_join_kernel(
+    const PartTask *tasks, uint64_t ntasks, uint64_t lead, const JoinSlot *slots, hj_counters *work, uint32_t cap_max, RecArea ra,
     uint32_t *oversize, int chk, void *stage_base, uint32_t scap) {
     using T = typename Tup<W>::U;
     using Vec = typename Tup<W>::Vec;
     constexpr int PV = Tup<W>::kPerVec, U = 2, IT = U * PV;
-    constexpr uint32_t G = SoaTab<W>::G;
+    constexpr uint32_t G = SoaTab<W>::G, AG = AggSoa<W>::G;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_full;
-    __shared__ unsigned long long s_p;
+    __shared__ __align__(16) PartTask s_task[2];
+    __shared__ unsigned long long s_idx[2];
+    __shared__ int s_ahead;
     const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
 
     Sink sink;
@@ -1225,17 +1360,45 @@ __global__ void __launch_bounds__(NT, 2048 / NT / 2) partition_join_kernel(
         sink.scap = scap;
         sink.slots = slots;
     }
-    for (;;) {
-        if (threadIdx.x == 0) s_p = atomicAdd(&work->work, 1ull);
-        __syncthreads();
-        const uint64_t ti = s_p;
-        if (ti >= ntasks) break;
-        const PartTask tk = tasks[ti];
+    // While more than two of the first `lead` tasks per CTA remain, tasks are taken one ahead: during a
+    // task's build warp 0 reads the record of the next one (whose index it took at the
+    // end of the task before), and during its probe the next one's build rows and first
+    // probe rows are asked into L2.  The last tasks are taken as CTAs fall idle.
+    constexpr unsigned kTaskWords = sizeof(PartTask) / 4;
+    static_assert(kTaskWords <= 32, "a warp reads a task record");
+    constexpr unsigned long long kNone = ~0ull;
+    unsigned long long idx = kNone;  // warp 0, lane 0: the next task's index, if taken ahead
+    if (warp == 0) {
+        unsigned long long i = 0;
+        if (lane == 0) i = atomicAdd(&work->work, 1ull);
+        i = __shfl_sync(0xffffffffu, i, 0);
+        if (i < ntasks && lane < kTaskWords) ((uint32_t *)&s_task[0])[lane] = ((const uint32_t *)(tasks + i))[lane];
+        if (lane == 0) {
+            s_idx[0] = i;
+            if (i + 2 * gridDim.x < lead) idx = atomicAdd(&work->work, 1ull);
+        }
+    }
+    __syncthreads();
+    for (unsigned cur_task = 0;; cur_task ^= 1) {
+        if (s_idx[cur_task] >= ntasks) break;
+        const uint64_t ti = s_idx[cur_task];
+        const PartTask &tk = s_task[cur_task];
+        uint32_t rec = 0;  // warp 0: the next task's record, a word per lane
+        if (warp == 0) {
+            idx = __shfl_sync(0xffffffffu, idx, 0);
+            if (idx < ntasks && lane < kTaskWords) rec = ((const uint32_t *)(tasks + idx))[lane];
+        }
+        auto pass_record = [&]() {
+            if (warp != 0) return;
+            if (idx != kNone && lane < kTaskWords) ((uint32_t *)&s_task[cur_task ^ 1])[lane] = rec;
+            if (lane == 0) s_ahead = idx < ntasks;
+        };
         const uint32_t nrv = tk.nr / PV, nsv = tk.ns / PV;
         const Vec *Rv = (const Vec *)tk.R;
         const Vec *Sv = (const Vec *)tk.S;
         const uint64_t nr = tk.nr;  // build rows, padding included
         const PartFilter pf{tk.p, (int)tk.b1, (int)tk.b2, 1};
+        const T pk1 = (T)tk.pk1, pk2 = (T)tk.pk2;  // keys of padding rows, besides 0
         hj_counters *jc = slots[tk.join].ctr;
         sink.begin_task(tk.join);
         ProbeAcc acc;
@@ -1257,15 +1420,28 @@ __global__ void __launch_bounds__(NT, 2048 / NT / 2) partition_join_kernel(
                 }
             }
         }
-        uint32_t *ovf = (uint32_t *)(smem + (size_t)cap_max * (AGG ? agg_slot_bytes(W, chk) : 2 * W));
+        uint32_t *info = (uint32_t *)(smem + (size_t)cap_max * (AGG ? agg_slot_bytes(W, chk) : 2 * W));
         const T top = Tup<W>::kAllOnes;
         const T empty = pf.keep(hashw<W>(top)) ? (T)tk.ek1 : top;
-        const SoaTab<W> tab{cap / G, empty, ovf, (const T *)smem, (const T *)smem + cap};
-        const AggSoa<W> at = AggSoa<W>::at(smem, cap, empty, ovf, chk != 0);
+        const SoaTab<W> tab{cap / G, empty, (const uint16_t *)info, (const T *)smem, (const T *)smem + cap};
+        const AggSoa<W> at = AggSoa<W>::at(smem, cap, empty, info, chk != 0);
+        constexpr int RB = 2;  // build vectors per thread in flight
+        Vec rx[RB];
+        auto load_r = [&](uint32_t v0) {
+#pragma unroll
+            for (int u = 0; u < RB; ++u)
+                if (v0 + u * NT < nrv) rx[u] = ld_stream(Rv + v0 + u * NT);
+        };
+        if (!work_p) pass_record();
         if (work_p) {
-            T *kv = (T *)smem;  // key region: cap keys; the rid (or sum and count) regions follow
-            for (uint32_t i = threadIdx.x; i < cap; i += blockDim.x) kv[i] = empty;
-            for (uint32_t i = threadIdx.x; i < (cap / G + 31) / 32; i += blockDim.x) ovf[i] = 0;
+            if constexpr (!AGG) load_r(threadIdx.x);
+            // key region: cap keys (whole 128s); the rid (or sum and count) regions follow
+            uint4 e4;
+            if constexpr (W == 4) e4 = make_uint4(empty, empty, empty, empty);
+            else e4 = make_uint4((uint32_t)empty, (uint32_t)(empty >> 32), (uint32_t)empty, (uint32_t)(empty >> 32));
+            for (uint32_t i = threadIdx.x; i < cap * W / 16; i += NT) ((uint4 *)smem)[i] = e4;
+            const uint32_t info_words = AGG ? (cap / AG + 31) / 32 : cap / G / 2;
+            for (uint32_t i = threadIdx.x; i < info_words; i += NT) info[i] = 0;
             if (AGG) {
                 for (uint32_t i = threadIdx.x; i < cap; i += blockDim.x) {
                     at.cnt[i] = 0;
@@ -1278,92 +1454,97 @@ __global__ void __launch_bounds__(NT, 2048 / NT / 2) partition_join_kernel(
             __syncthreads();
             // build over R_p
             if constexpr (AGG) {
-                // lanes of a warp holding the same key insert once, their count and
-                // A(rid) sum together (a repeated key's slot takes one atomic per warp
-                // group instead of one per tuple); the loop is warp-uniform
-                for (uint32_t v0 = threadIdx.x & ~31u; v0 < nrv; v0 += blockDim.x) {
-                    const uint32_t v = v0 + lane;
-                    T k[2] = {0, 0}, r[2] = {0, 0};
-                    if (v < nrv) {
-                        const Vec x = ld_stream(Rv + v);
-                        if constexpr (W == 4) {
-                            k[0] = x.x; r[0] = x.y; k[1] = x.z; r[1] = x.w;
-                        } else {
-                            k[0] = x.x; r[0] = x.y;
-                        }
+                for (uint32_t v = threadIdx.x; v < nrv; v += NT) {
+                    const Vec x = ld_stream(Rv + v);
+                    T k[2], r[2];
+                    if constexpr (W == 4) {
+                        k[0] = x.x; r[0] = x.y; k[1] = x.z; r[1] = x.w;
+                    } else {
+                        k[0] = x.x; r[0] = x.y;
                     }
 #pragma unroll
                     for (int e = 0; e < PV; ++e) {
                         // a padding row carries 0 or a pass's second sentinel: only
                         // such keys are hashed to see whether the row is the partition's
-                        const bool in = v < nrv && !((k[e] == T(0) || k[e] == (T)tk.pk1 || k[e] == (T)tk.pk2) &&
-                                                     !pf.keep(hashw<W>(k[e])));
-                        const unsigned g = __match_any_sync(0xffffffffu, k[e]) & __ballot_sync(0xffffffffu, in);
-                        const uint64_t a = chk && in ? mix_a(r[e]) : 0;
-                        uint64_t asum = a;
-                        if (chk && __any_sync(0xffffffffu, in && __popc(g) > 1)) {
-                            // the group's sum of A(rid): every lane's value, kept by
-                            // the lanes of its group (whole-warp shuffles)
-                            asum = 0;
-#pragma unroll 8
-                            for (int q = 0; q < 32; ++q) {
-                                const uint64_t y = __shfl_sync(0xffffffffu, a, q);
-                                if ((g >> q) & 1u) asum += y;
-                            }
-                        }
-                        if (!in || (g & ((1u << lane) - 1u))) continue;  // the group's lowest lane inserts
-                        if (!at.insert(k[e], (uint32_t)__popc(g), asum)) s_full = 1;
+                        if ((k[e] == T(0) || k[e] == pk1 || k[e] == pk2) && !pf.keep(hashw<W>(k[e]))) continue;
+                        if (!at.insert(k[e], chk ? mix_a(r[e]) : 0)) s_full = 1;
                     }
                 }
-            } else
-            for (uint32_t v = threadIdx.x; v < nrv; v += blockDim.x) {
-                const Vec x = ld_stream(Rv + v);
-                T k[2], r[2];
-                if constexpr (W == 4) {
-                    k[0] = x.x; r[0] = x.y; k[1] = x.z; r[1] = x.w;
-                } else {
-                    k[0] = x.x; r[0] = x.y;
-                }
+            } else {
+                // An insert takes a count of its home bucket with one atomic add: the
+                // count before it is its slot there (load factor 1/3: one in twenty
+                // moves on).  The adds of a thread's four tuples are in flight together.
+                // A walk past kMaxSmemWalk buckets means a heavily repeated key: the
+                // partition goes to the key-list fallback.
+                T *kv = (T *)smem;
+                const uint32_t lim = tab.nb < kMaxSmemWalk ? tab.nb : kMaxSmemWalk;
+                auto tried = [&](uint32_t b) -> uint32_t {
+                    const uint32_t sh = (b & 1u) * 16u;
+                    return (atomicAdd(&info[b >> 1], 1u << sh) >> sh) & 0xFFFFu;
+                };
+                for (uint32_t v0 = threadIdx.x; v0 < nrv; v0 += RB * NT) {
+                    if (v0 != threadIdx.x) load_r(v0);
+                    constexpr int QV = RB, QT = QV * PV;  // vectors and tuples of a step
 #pragma unroll
-                for (int e = 0; e < PV; ++e) {
-                    // a padding row carries 0 or a pass's second sentinel: only
-                    // such keys are hashed to see whether the row is the partition's
-                    if ((k[e] == T(0) || k[e] == (T)tk.pk1 || k[e] == (T)tk.pk2) && !pf.keep(hashw<W>(k[e]))) continue;
-                    bool ok = false;
-                    {
-                        T *kv = (T *)smem;
-                        uint32_t bkt = part_bucket<W>(k[e], tab.nb);
-                        // a walk past kMaxSmemWalk buckets means a heavily repeated
-                        // key: the partition goes to the key-list fallback
-                        const uint32_t lim = tab.nb < kMaxSmemWalk ? tab.nb : kMaxSmemWalk;
-                        for (uint32_t it = 0; it < lim && !ok; ++it) {
-                            for (uint32_t q = 0; q < G; ++q) {
-                                T *slot = &kv[bkt * G + q];
-                                if (cas_key<W>(slot, empty, k[e]) == empty) {
-                                    slot[cap] = r[e];  // the same slot of the rid region
-                                    ok = true;
-                                    break;
-                                }
+                    for (int u0 = 0; u0 < RB; u0 += QV) {
+                        T k[QT], r[QT];
+                        uint32_t bkt[QT], q[QT];
+                        bool in[QT];
+#pragma unroll
+                        for (int i = 0; i < QT; ++i) {
+                            const Vec &x = rx[u0 + i / PV];
+                            if constexpr (W == 4) {
+                                k[i] = i % 2 ? x.z : x.x;
+                                r[i] = i % 2 ? x.w : x.y;
+                            } else {
+                                k[i] = x.x;
+                                r[i] = x.y;
                             }
-                            if (!ok) {  // moving past a full bucket: mark it
-                                atomicOr(&ovf[bkt >> 5], 1u << (bkt & 31));
-                                bkt = bkt + 1 == tab.nb ? 0 : bkt + 1;
+                            // a padding row carries 0 or a pass's second sentinel: only
+                            // such keys are hashed to see whether the row is the partition's
+                            in[i] = v0 + (u0 + i / PV) * NT < nrv &&
+                                    !((k[i] == T(0) || k[i] == pk1 || k[i] == pk2) &&
+                                      !pf.keep(hashw<W>(k[i])));
+                            bkt[i] = part_bucket<W>(k[i], tab.nb);
+                            q[i] = in[i] ? tried(bkt[i]) : 0u;
+                        }
+#pragma unroll
+                        for (int i = 0; i < QT; ++i) {
+                            if (!in[i]) continue;
+                            for (uint32_t it = 1; q[i] >= G && it < lim; ++it) {
+                                bkt[i] = bkt[i] + 1 == tab.nb ? 0 : bkt[i] + 1;
+                                q[i] = tried(bkt[i]);
+                            }
+                            if (q[i] < G) {
+                                T *slot = &kv[bkt[i] * G + q[i]];
+                                slot[0] = k[i];
+                                slot[cap] = r[i];  // the same slot of the rid region
+                            } else {
+                                s_full = 1;
                             }
                         }
                     }
-                    if (!ok) s_full = 1;
                 }
             }
+            pass_record();
             __syncthreads();
+            if (s_ahead) {  // the next task's rows into L2
+                const PartTask &nt = s_task[cur_task ^ 1];
+                const uint32_t rl = (nt.nr / PV + 7) / 8, sl = (min(nt.ns / PV, kAheadVecs) + 7) / 8;
+                for (uint32_t i = threadIdx.x; i < rl + sl; i += NT)
+                    prefetch_l2(i < rl ? (const char *)nt.R + (uint64_t)i * 128 : (const char *)nt.S + (uint64_t)(i - rl) * 128);
+            }
+            bool unique = false;
+            if constexpr (FAST) unique = nsv >= 2 * nrv && !s_full && !__syncthreads_or(keys_repeat<W, NT>(tab));
             if (s_full) {
                 if (threadIdx.x == 0) oversize[atomicAdd(&work->n_oversize, 1ull)] = (uint32_t)ti;
             } else {
                 if constexpr (FAST) {  // no aggregate, no checksum
-                    // one vector per thread and group (two 4-byte tuples, one 8-byte):
-                    // fewer live registers than U, which leaves the batched walks room
-                    constexpr int FU = 1;
-                    T *wq = (T *)(smem + walkq_offset(cap_max, 2 * W)) + (size_t)warp * 2 * kWalkQ;
-                    probe_fast<W, FU>(tab, Sv, nsv, sink, warp, nwarps, lane, wq, wq + kWalkQ);
+                    T *wq = (T *)(smem + walkq_offset(cap_max, 2 * W, W, false)) + (size_t)warp * 2 * kWalkQ;
+                    if (unique)
+                        probe_unique<W, 2>(tab, Sv, nsv, sink, warp, nwarps, lane, wq, wq + kWalkQ);
+                    else  // one vector per thread: the batched walks need the registers
+                        probe_fast<W, 1>(tab, Sv, nsv, sink, warp * 32u, nwarps * 32u, lane, wq, wq + kWalkQ, 0);
                 } else {
                 const uint32_t gstride = nwarps * 32 * U;
                 Vec cur[U], nxt[U];
@@ -1397,12 +1578,12 @@ __global__ void __launch_bounds__(NT, 2048 / NT / 2) partition_join_kernel(
                         // home buckets of all items first; no partition filter: a padding
                         // tuple's key hashes to another partition, so it matches no slot
                         uint32_t home[IT];
-                        T kb[IT][G];
+                        T kb[IT][AG];
 #pragma unroll
                         for (int i = 0; i < IT; ++i) {
                             home[i] = part_bucket<W>(k[i], at.nb);
 #pragma unroll
-                            for (uint32_t q = 0; q < G; ++q) kb[i][q] = at.empty;
+                            for (uint32_t q = 0; q < AG; ++q) kb[i][q] = at.empty;
                             if (val[i]) at.ld(home[i], kb[i]);
                         }
 #pragma unroll
@@ -1410,12 +1591,12 @@ __global__ void __launch_bounds__(NT, 2048 / NT / 2) partition_join_kernel(
                             uint32_t mm = 0;
                             bool e = false;
 #pragma unroll
-                            for (uint32_t q = 0; q < G; ++q) {
+                            for (uint32_t q = 0; q < AG; ++q) {
                                 mm |= (uint32_t)(kb[i][q] == k[i]) << q;
                                 e |= kb[i][q] == at.empty;
                             }
                             // (a lane past the slice's end holds a stale key: no slot)
-                            uint32_t sl = val[i] && mm ? home[i] * G + (uint32_t)(__ffs(mm) - 1) : ~0u;
+                            uint32_t sl = val[i] && mm ? home[i] * AG + (uint32_t)(__ffs(mm) - 1) : ~0u;
                             if (val[i] && !mm && !e && at.overflowed(home[i]))  // the run continues (rare)
                                 sl = at.find_from(k[i], home[i] + 1 == at.nb ? 0 : home[i] + 1);
                             if (sl != ~0u) {
@@ -1503,9 +1684,23 @@ __global__ void __launch_bounds__(NT, 2048 / NT / 2) partition_join_kernel(
                 }
             }
         }
-        flush_acc(jc, acc, AGG);
+        if constexpr (!FAST) flush_acc(jc, acc, AGG);
         if constexpr (!AGG) sink.end_task();
-        __syncthreads();  // every warp is done with this table and with s_p
+        if (warp == 0) {
+            unsigned long long n = idx;
+            if (idx == kNone) {
+                if (lane == 0) n = atomicAdd(&work->work, 1ull);
+                n = __shfl_sync(0xffffffffu, n, 0);
+                if (n < ntasks && lane < kTaskWords)
+                    ((uint32_t *)&s_task[cur_task ^ 1])[lane] = ((const uint32_t *)(tasks + n))[lane];
+            }
+            idx = kNone;
+            if (lane == 0) {
+                s_idx[cur_task ^ 1] = n;
+                if (n + 2 * gridDim.x < lead) idx = atomicAdd(&work->work, 1ull);
+            }
+        }
+        __syncthreads();  // every warp is done with this table and has the next task's record
     }
     if constexpr (!AGG) sink.finish();
 }
@@ -1599,9 +1794,12 @@ uint64_t empty_key2(int width, int b1, int b2) {
     return k;
 }
 
-// Join launch shape: two 512-thread CTAs per SM with tables up to 100 KiB, or one
-// 1024-thread CTA per SM with up to 200 KiB when the expected build partition
-// needs the room (load factor about 1/3 either way).
+// Join launch shape: two CTAs per SM with tables up to 100 KiB, or one of twice the
+// threads with up to 200 KiB when the expected build partition needs the room (load
+// factor about 1/3 either way).  The aggregate join runs 1024 threads per SM, the pair
+// join 640: its probe loop holds four tuples' buckets and needs 96 registers (with 64,
+// 1024 threads spill into an L1 that the tables leave no room: 2^24 x 2^28 1257 us
+// against 828, 896 threads 1181, 768 threads 1072, 576 threads 881).
 struct JoinCfg {
     int nt;
     uint64_t smem_limit;
@@ -1612,17 +1810,17 @@ static uint64_t join_slot_bytes(int width, int agg, int checksum) {
 static JoinCfg join_cfg(int width, int agg, int checksum, uint64_t expect_r) {
     const uint64_t slot = join_slot_bytes(width, agg, checksum);
     const uint64_t need = 3 * (expect_r + 6 * (uint64_t)__builtin_sqrt((double)expect_r + 1.0) + 64) * slot;
-    if (need <= (100ull << 10)) return JoinCfg{512, 100ull << 10};
-    return JoinCfg{1024, 200ull << 10};
+    if (need <= (100ull << 10)) return JoinCfg{agg ? 512 : 320, 100ull << 10};
+    return JoinCfg{agg ? 1024 : 640, 200ull << 10};
 }
 
 uint64_t partition_join_warps(hj_ctx *c) { return (uint64_t)num_sms(c) * 32; }
 uint64_t partition_join_ctas(hj_ctx *c, int width, int agg, uint64_t expect_r) {
-    return (uint64_t)num_sms(c) * (2048 / join_cfg(width, agg, 1, expect_r).nt / 2);
+    return (uint64_t)num_sms(c) * join_ctas(join_cfg(width, agg, 1, expect_r).nt);
 }
 
-hj_status partition_join(hj_ctx *c, int width, int agg, const PartTask *tasks, uint64_t ntasks, const JoinSlot *slots,
-                         uint64_t expect_r, int checksum, uint32_t *oversize, RecArea ra, void *stage,
+hj_status partition_join(hj_ctx *c, int width, int agg, const PartTask *tasks, uint64_t ntasks, uint64_t lead,
+                         const JoinSlot *slots, uint64_t expect_r, int checksum, uint32_t *oversize, RecArea ra, void *stage,
                          uint32_t scap) {
     if (ntasks == 0) return HJ_OK;
     const uint64_t slot_bytes = join_slot_bytes(width, agg, checksum);
@@ -1637,25 +1835,26 @@ hj_status partition_join(hj_ctx *c, int width, int agg, const PartTask *tasks, u
     // warp's walk queue, within what the shape's CTAs per SM can have (two
     // 512-thread CTAs share an SM)
     const uint64_t qbytes = (!agg && !checksum) ? (uint64_t)(cfg.nt / 32) * kWalkQ * 2 * width : 0;
-    const uint64_t total_max = cfg.nt == 512 ? (112ull << 10) : (222ull << 10);
+    const uint64_t total_max = join_ctas(cfg.nt) == 2 ? (112ull << 10) : (222ull << 10);
     const uint64_t budget = std::min<uint64_t>(cfg.smem_limit + qbytes, total_max) - qbytes;
-    uint64_t max_slots = (budget - bitmap_bytes) / slot_bytes / 128 * 128;
+    uint64_t max_slots = agg ? (budget - bitmap_bytes) / slot_bytes / 128 * 128
+                             : (budget - 16) * 8 / (8 * slot_bytes + (uint64_t)width) / 128 * 128;
     uint64_t cap_max = want < max_slots ? want : max_slots;
     if (cap_max < 128) cap_max = 128;
-    const size_t smem = (size_t)walkq_offset((uint32_t)cap_max, (uint32_t)slot_bytes) + (size_t)qbytes;
-    unsigned grid = (unsigned)num_sms(c) * (2048 / cfg.nt / 2);
+    const size_t smem = (size_t)walkq_offset((uint32_t)cap_max, (uint32_t)slot_bytes, width, agg != 0) + (size_t)qbytes;
+    unsigned grid = (unsigned)num_sms(c) * join_ctas(cfg.nt);
     if (grid > ntasks) grid = (unsigned)ntasks;
 #define HJ_PJ(WW, AA, NT, SK, FF)                                                                               \
     do {                                                                                                        \
         auto kern = partition_join_kernel<WW, AA, NT, SK<WW>, FF>;                                              \
         HJ_TRY(allow_max_smem(c, (const void *)kern));                                                         \
-        HJ_LAUNCH(c, "partition_join", kern, grid, NT, smem, tasks, ntasks, slots, c->d_ctr, (uint32_t)cap_max, \
+        HJ_LAUNCH(c, "partition_join", kern, grid, NT, smem, tasks, ntasks, lead, slots, c->d_ctr, (uint32_t)cap_max, \
                   ra, oversize, checksum, stage, scap);                                                         \
     } while (0)
 #define HJ_PJ_NT(WW, AA, SK, FF)                                \
     do {                                                        \
-        if (cfg.nt == 512) HJ_PJ(WW, AA, 512, SK, FF);           \
-        else HJ_PJ(WW, AA, 1024, SK, FF);                        \
+        if (join_ctas(cfg.nt) == 2) HJ_PJ(WW, AA, (AA ? 512 : 320), SK, FF); \
+        else HJ_PJ(WW, AA, (AA ? 1024 : 640), SK, FF);           \
     } while (0)
 #define HJ_PJ_F(WW, SK)                                         \
     do {                                                        \
