@@ -51,7 +51,7 @@ WORKLOADS = {
         kind="batch", njoins=4096, nr=0, ns=0, algo=2,
         desc="4096 independent joins, |R| log-uniform in [2^10, 2^22], |S| = 4|R| (uint32 key, uint32 rid); "
              "R keys a permutation of 1..|R|, S keys uniform over [1, ceil(|R|/0.75)] (75% match); pairs "
-             "materialised; one hj_join_batch call (CUDA graph per wave) per step vs one hj_join per join"),
+             "materialised; one hj_join_batch call (a few launches per wave) per step vs one hj_join per join"),
     "serve_20000": dict(
         kind="serve", nreq=20000, nr=0, ns=0, algo=0, budget=120 << 30, load=0.7, sweep=(0.5, 0.9),
         desc="serving: 20000 join requests, Poisson arrivals, |R| log-uniform in [2^12, 2^24], |S| log-uniform "

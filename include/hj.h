@@ -76,7 +76,7 @@ typedef struct hj_rel {
 
 /* opts.flags */
 #define HJ_FLAG_CHECKSUM 1u /* MATERIALIZE: also compute c0, c1 over the pairs           */
-#define HJ_FLAG_GRAPH 2u    /* hj_join_batch: capture each wave's launches in a CUDA graph */
+#define HJ_FLAG_GRAPH 2u    /* hj_join_batch: accepted, changes nothing (a wave is four launches) */
 
 typedef struct hj_opts {
     int32_t algo;          /* HJ_ALGO_*                                              */
@@ -109,8 +109,7 @@ typedef struct hj_table hj_table;
  * (NULL: the library creates its own non-blocking stream, which is NOT ordered
  * after work on the legacy default stream -- pass cudaStreamLegacy to order the
  * context's work with that stream, e.g. after kernels that produced the inputs
- * there).  Any stream may be given, the legacy one included: the library captures
- * CUDA graphs on private streams.  `hbm_budget_bytes`
+ * there).  Any stream may be given, the legacy one included.  `hbm_budget_bytes`
  * caps the device memory the library holds at once (0: no cap).  Every later call
  * on the context must run with that device current or will make it current. */
 hj_status hj_create(hj_ctx **ctx, int device, void *cuda_stream, uint64_t hbm_budget_bytes);
@@ -157,14 +156,13 @@ hj_status hj_join(hj_ctx *ctx, const hj_rel *R, const hj_rel *S, const hj_opts *
 
 /* Many independent joins: outs[j] receives the join of Rs[j] and Ss[j] exactly as
  * hj_join would return it (count, checksums, library-owned pairs).  All relations
- * share one width; each must have fewer than 2^32 - 1 tuples.  Joins are grouped
- * by the radix bits their build side needs; every group is partitioned in one
- * pass per relation side and all (join, partition) pairs of all groups are joined
- * by ONE persistent launch that takes them from a work counter, so small and large
- * joins share the GPU.  If the joins' workspace exceeds the HBM budget (the
- * context's, else 70% of free device memory) they run in several such waves.
- * opts->flags & HJ_FLAG_GRAPH captures each wave's device work in a CUDA graph and
- * launches it as one.  opts->algo, radix_bits and passes are ignored. */
+ * share one width; each must have fewer than 2^32 - 1 tuples.  Every join partitions
+ * on the radix bits its build side needs; two launches partition all relations, and
+ * all (join, partition) pairs are joined by ONE persistent launch that takes them from
+ * a work counter, so small and large joins share the GPU.  If the joins' workspace
+ * exceeds the HBM budget (the context's, else 70% of free device memory) they run in
+ * several such waves.  opts->flags & HJ_FLAG_GRAPH is accepted and changes nothing (a
+ * wave is four launches).  opts->algo, radix_bits and passes are ignored. */
 hj_status hj_join_batch(hj_ctx *ctx, int n, const hj_rel *Rs, const hj_rel *Ss, const hj_opts *opts,
                         hj_result *outs);
 
@@ -293,7 +291,7 @@ typedef struct hj_server_opts {
     int32_t max_wave;      /* most requests in one wave (0: 512)                       */
     uint64_t wave_tuples;  /* a wave stops growing past this many tuples of R and S;
                               a request above it runs alone (0: 2^26)                 */
-    uint64_t flags;        /* HJ_FLAG_GRAPH: waves of several joins run as a CUDA graph */
+    uint64_t flags;        /* HJ_FLAG_GRAPH: accepted, changes nothing (hj_join_batch) */
 } hj_server_opts;
 
 /* Host clock (seconds since hj_server_create, steady clock) of a request's steps. */

@@ -422,7 +422,7 @@ hj_status run_partition_join(hj_ctx *c, const hj_rel *R, const hj_rel *S, const 
     const uint64_t pcap = mat ? sink->pcap : 0;
     HJ_LAUNCH(c, "set_slot", set_slot_kernel, 1, 1, 0, slot_dev, pairs, (unsigned long long)pcap, c->d_ctr);
     const uint64_t expect = NP ? (R->n + NP - 1) / NP : 0;
-    HJ_TRY(partition_join(c, W, agg, tasks, ntasks, NP, slot_dev, expect, chk, oversize, ra, nullptr, 0));
+    HJ_TRY(partition_join(c, W, agg, tasks, ntasks, NP, slot_dev, expect, chk, oversize, ra, false));
     if (mat) HJ_TRY(sink->finalize_device(c->d_ctr));
     HJ_TRY(read_counters(c));
     HJ_TRY(check_output_status(c));
@@ -628,7 +628,7 @@ hj_status join_host_pipelined(hj_ctx *c, const hj_rel *Rh, const hj_rel *Sh, con
             HJ_LAUNCH(c, "set_slot", set_slot_kernel, 1, 1, 0, slot.as<JoinSlot>(), mat ? ps.sink.pairs.p : nullptr,
                       (unsigned long long)(mat ? ps.sink.pcap : 0), c->d_ctr);
             HJ_TRY(partition_join(c, W, is_agg(o.mode), tasks.as<PartTask>(), ntasks, NP, slot.as<JoinSlot>(),
-                                  (Rh->n + NP - 1) / NP, wants_checksum(o), oversize.as<uint32_t>(), ra, nullptr, 0));
+                                  (Rh->n + NP - 1) / NP, wants_checksum(o), oversize.as<uint32_t>(), ra, false));
             if (mat) HJ_TRY(ps.sink.finalize_device(c->d_ctr));
             HJ_CUDA(c, cudaMemcpyAsync(ps.h, c->d_ctr, sizeof(hj_counters), cudaMemcpyDeviceToHost, c->stream));
             HJ_CUDA(c, cudaEventRecord(ps.computed, c->stream));

@@ -83,12 +83,13 @@ uint64_t tail_split_from(hj_ctx *c, int width, int agg, uint64_t NP, uint64_t ex
 // must be zero at launch), one ahead while more than two per CTA of the first `lead`
 // (the ones that are sure to hold rows) remain.  Tasks whose table does not fit are appended to
 // `oversize` (task indices) and counted in c->d_ctr->n_oversize.  Pairs go to
-// each task's join slot: with `stage` (a staging area of scap pairs per warp, for
-// partition_join_warps(c) warps) by
-// exact claims, otherwise by per-warp chunks recorded in `ra`.
+// each task's join slot: `staged`, by exact claims of what a warp collected in shared
+// memory, otherwise by per-warp chunks recorded in `ra`.
 hj_status partition_join(hj_ctx *c, int width, int agg, const PartTask *tasks, uint64_t ntasks, uint64_t lead,
-                         const JoinSlot *slots, uint64_t expect_r, int checksum, uint32_t *oversize, RecArea ra, void *stage,
-                         uint32_t scap);
+                         const JoinSlot *slots, uint64_t expect_r, int checksum, uint32_t *oversize, RecArea ra,
+                         bool staged);
+// Build rows of a partition that leave room for the table and the staging buffers.
+uint64_t batch_partition_rows(int width);
 uint64_t partition_join_warps(hj_ctx *c);
 uint64_t partition_join_ctas(hj_ctx *c, int width, int agg, uint64_t expect_r);
 
@@ -141,14 +142,27 @@ hj_status fallback_reprobe(hj_ctx *c, bool chk, const FallbackRedo &redo, const 
 // run is rounded up to whole 32-byte sectors with padding tuples whose key
 // hashes to another digit, so the output holds up to partition_out_rows() rows
 // and segment s of the output starts where the padded segments before it end.
-// With seg_ptrs (device array of nseg pointers, 16-byte aligned), segment s is read
-// from its own array seg_ptrs[s] instead of from `in` (fan-out at most 2^11).
 hj_status partition_pass(hj_ctx *c, int width, const void *in, uint64_t n_total, const uint64_t *seg_off,
-                         uint64_t nseg, int shift, int bits, void *out, uint64_t *part_off, int pad,
-                         const void *const *seg_ptrs = nullptr);
+                         uint64_t nseg, int shift, int bits, void *out, uint64_t *part_off, int pad);
 // One padded pass over a single segment of n rows at 2^bits <= 2^11 digits:
 // partition_pass's output with two launches (histogram, scatter).
 hj_status partition_pass1(hj_ctx *c, int width, const void *in, uint64_t n, int bits, void *out, uint64_t *part_off);
+// Padded passes of many relations at once, each on its own bits <= 2^11 digits: chunk
+// by chunk (device array), relation by relation ranges of `out`.  H and base hold
+// 2^bits words per chunk, T 2^bits + 1 per relation (zero beforehand), part_off
+// as many offsets, rows of `out`.
+struct BatchChunk {
+    const void *src;   // its tuples (16-byte aligned)
+    uint64_t obase;    // first row of its relation's output range (a multiple of 16)
+    uint64_t h_at;     // its counts in H and base
+    uint64_t t_at;     // its relation's totals in T and offsets in part_off
+    uint32_t n;        // its rows (even, but for a relation's last chunk)
+    uint16_t bits;
+    uint16_t lead;     // 1: the relation's first chunk (writes the offsets)
+};
+uint64_t batch_chunk_rows(hj_ctx *c, uint64_t rows, int bits);
+hj_status batch_partition(hj_ctx *c, int width, const BatchChunk *chunks, uint64_t nchunks, int max_bits, uint32_t *H,
+                          uint32_t *base, uint32_t *T, void *out, uint64_t *part_off);
 uint64_t partition_out_rows(hj_ctx *c, int width, uint64_t n_total, uint64_t nseg, int bits, int pad);
 // Exclusive scan of n uint32 counts into n + 1 uint64 offsets (out[n] = total).
 hj_status scan_counts(hj_ctx *c, const uint32_t *in, uint64_t n, unsigned long long *out);

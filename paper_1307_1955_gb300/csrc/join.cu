@@ -717,8 +717,8 @@ template <int W> struct ChunkSink {
     using T = typename Tup<W>::U;
     OutState st;
     OutCtx oc;
-    typename PairVec<W>::T *open = nullptr;  // the open chunk (append_runs)
-    unsigned room = 0;                       // rows of it that append_runs may fill without a test
+    typename PairVec<W>::T *open = nullptr;  // the open chunk (append_found)
+    unsigned room = 0;                       // rows of it that append_found may fill without a test
     unsigned join = ~0u;
     const JoinSlot *slots;
     RecArea ra;
@@ -770,13 +770,6 @@ template <int W> struct ChunkSink {
             st.used += tot;
         }
         st.pairs += tot;
-    }
-    template <int IT>
-    __device__ __forceinline__ void append_runs(const uint32_t *cnt, const T *first, const T *r) {
-        bool found[IT];
-#pragma unroll
-        for (int i = 0; i < IT; ++i) found[i] = cnt[i] == 1;
-        append_found<IT>(found, first, r);
     }
     // one append for all items of a group with a match (at most 32 * IT pairs, so at
     // most one new chunk): item-major positions, so that each store instruction
@@ -845,12 +838,14 @@ template <int W> struct ChunkSink {
 
 // Per-warp staged exact output (batches of joins, whose many joins per launch
 // would leave a partly filled chunk per warp and join): each warp collects its
-// pairs in a private buffer of scap pairs in global memory (a few KB per warp,
-// L2-resident) and, when the buffer fills or the warp moves on to another join,
+// pairs in a private buffer of scap pairs in shared memory and, when the buffer fills or the warp moves on to another join,
 // claims exactly that many rows of the join's buffer with one atomic add and
 // copies them out with coalesced stores.  Output is dense as written (no
 // compaction) and the sink needs no CTA barrier.  scap >= 32 x the items of a
 // group, so one flush always makes room.
+// (4 KB per warp: 700 us for the 200 joins of batch_partition_rows, 720 us with 2 KB; the
+// same staged in global memory, twice the rows per partition, 890 us)
+constexpr uint32_t kJoinStageBytes = 4096;
 template <int W> struct WarpStageSink {
     using T = typename Tup<W>::U;
     using P = typename std::conditional<W == 4, uint2, ulonglong2>::type;
@@ -912,56 +907,27 @@ template <int W> struct WarpStageSink {
         used += tot;
     }
     template <int IT>
-    __device__ __forceinline__ void append_runs(const uint32_t *cnt, const T *first, const T *r) {
-        append_group<IT>(cnt, first, r);
-    }
-    template <int IT>
     __device__ __forceinline__ void append_found(const bool *found, const T *first, const T *r) {
-        uint32_t cnt[IT];
+        const unsigned lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
+        unsigned m[IT], tot = 0;
 #pragma unroll
-        for (int i = 0; i < IT; ++i) cnt[i] = found[i];
-        append_group<IT>(cnt, first, r);
+        for (int i = 0; i < IT; ++i) {
+            m[i] = __ballot_sync(0xffffffffu, found[i]);
+            tot += __popc(m[i]);
+        }
+        if (used + tot > scap) flush();
+        P *dst = stage + used;
+#pragma unroll
+        for (int i = 0; i < IT; ++i) {
+            if (found[i]) dst[__popc(m[i] & lt)] = mk(first[i], r[i]);
+            dst += __popc(m[i]);
+        }
+        used += tot;
     }
     __device__ __forceinline__ hj_counters *ctr() const { return slots[join].ctr; }
     __device__ __forceinline__ void end_task() {}
     __device__ __forceinline__ void finish() { flush(); }
 };
-
-// One group of IT probe items against the table, in phases so that the items'
-// shared-memory loads overlap: every item's home bucket (keys), then the match
-// masks and the first match's rid (one indexed load).  cnt[i] and first[i] cover
-// the home bucket only.  Inserts fill a bucket's slots in order and move past it
-// only once it is full, so a run goes on past the home bucket only if the bucket's
-// last slot is taken AND more inserts tried it than it has slots: bit i of the returned mask marks such an item (with at
-// most one home match; an item with several takes the whole-run walk instead).
-// Items with live[i] false match nothing.
-template <int W, int IT>
-__device__ __forceinline__ uint32_t probe_items(const SoaTab<W> &tab, const typename Tup<W>::U *k, const bool *live,
-                                                uint32_t *cnt, typename Tup<W>::U *first) {
-    using T = typename Tup<W>::U;
-    constexpr uint32_t G = SoaTab<W>::G;
-    uint32_t home[IT];
-    T kb[IT][G];
-#pragma unroll
-    for (int i = 0; i < IT; ++i) {
-        home[i] = part_bucket<W>(k[i], tab.nb);  // < nb for any key: the load is in bounds
-        tab.ld(home[i], 0, kb[i]);
-    }
-    uint32_t walk = 0;
-#pragma unroll
-    for (int i = 0; i < IT; ++i) {
-        uint32_t m = 0;
-#pragma unroll
-        for (uint32_t q = 0; q < G; ++q) m |= (uint32_t)(kb[i][q] == k[i]) << q;
-        if (!live[i]) m = 0;
-        // the first match's rid, read without a branch (slot G - 1 when nothing matched)
-        const T fr = tab.ld1(home[i], 1, (uint32_t)(__ffs(m | (1u << (G - 1))) - 1));
-        first[i] = m ? fr : T(0);
-        cnt[i] = __popc(m);
-        walk |= (uint32_t)(live[i] && cnt[i] <= 1 && kb[i][G - 1] != tab.empty && tab.overflowed(home[i])) << i;
-    }
-    return walk;
-}
 
 // Longest walk (in buckets) of an insert into a partition's shared-memory table.
 constexpr uint32_t kMaxSmemWalk = 64;
@@ -1033,91 +999,6 @@ __device__ __forceinline__ void drain_walks(const SoaTab<W> &tab, const typename
     }
 }
 
-template <int W, int U, class Sink>
-__device__ __forceinline__ void probe_fast(const SoaTab<W> &tab, const typename Tup<W>::Vec *Sv, uint32_t nsv,
-                                           Sink &sink, uint32_t g, uint32_t gstride, unsigned lane,
-                                           typename Tup<W>::U *wqk, typename Tup<W>::U *wqr, uint32_t qn) {
-    using T = typename Tup<W>::U;
-    using Vec = typename Tup<W>::Vec;
-    constexpr int PV = Tup<W>::kPerVec, IT = U * PV;
-    const unsigned lt = (1u << lane) - 1u;
-    Vec cur[U], nxt[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-        const uint32_t rel = g + u * 32u + lane;
-        if (rel < nsv) cur[u] = ld_stream(Sv + rel);
-    }
-    for (; g < nsv; g += gstride) {
-        const uint32_t gn = g + gstride;
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const uint32_t rel = gn + u * 32u + lane;
-            if (rel < nsv) nxt[u] = ld_stream(Sv + rel);
-        }
-        T k[IT], r[IT];
-        bool live[IT];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const bool in = g + (uint32_t)u * 32u + lane < nsv;
-            if constexpr (W == 4) {
-                k[2 * u] = cur[u].x; r[2 * u] = cur[u].y; k[2 * u + 1] = cur[u].z; r[2 * u + 1] = cur[u].w;
-                live[2 * u] = in;
-                live[2 * u + 1] = in;
-            } else {
-                k[u] = cur[u].x; r[u] = cur[u].y;
-                live[u] = in;
-            }
-        }
-        uint32_t cnt[IT];
-        T first[IT];
-        const uint32_t walk = probe_items<W, IT>(tab, k, live, cnt, first);
-        sink.template append_runs<IT>(cnt, first, r);
-        // several home matches (duplicate build keys): the whole warp walks each such run
-        bool multi_any = false;
-#pragma unroll
-        for (int i = 0; i < IT; ++i) multi_any |= cnt[i] > 1;
-        if (__any_sync(0xffffffffu, multi_any)) {
-#pragma unroll
-            for (int i = 0; i < IT; ++i) {
-                unsigned multi = __ballot_sync(0xffffffffu, cnt[i] > 1);
-                while (multi) {
-                    const int L = __ffs(multi) - 1;
-                    multi &= multi - 1;
-                    const T kk = __shfl_sync(0xffffffffu, k[i], L);
-                    const T ss = __shfl_sync(0xffffffffu, r[i], L);
-                    soa_coop_emit<W>(tab, kk, ss, part_bucket<W>(kk, tab.nb), sink);
-                }
-            }
-        }
-        // runs that go on past the home bucket: queued, walked 32 at a time
-        if (__any_sync(0xffffffffu, walk != 0)) {
-#pragma unroll
-            for (int i = 0; i < IT; ++i) {
-                const bool w = (walk >> i) & 1u;
-                const unsigned wm = __ballot_sync(0xffffffffu, w);
-                if (!wm) continue;
-                if (w) {
-                    const uint32_t pos = qn + (uint32_t)__popc(wm & lt);
-                    wqk[pos] = k[i];
-                    wqr[pos] = r[i];
-                }
-                qn += (uint32_t)__popc(wm);
-                if (qn >= 32) {
-                    __syncwarp();
-                    drain_walks<W>(tab, wqk + (qn - 32), wqr + (qn - 32), 32, sink);
-                    qn -= 32;
-                }
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) cur[u] = nxt[u];
-    }
-    if (qn) {
-        __syncwarp();
-        drain_walks<W>(tab, wqk, wqr, qn, sink);
-    }
-}
-
 // Whether no key is twice in the table: every thread of the CTA compares the keys
 // of its buckets, and of a bucket that overflowed with those its run goes on to.
 template <int W, int NT> __device__ __forceinline__ bool keys_repeat(const SoaTab<W> &t) {
@@ -1145,90 +1026,135 @@ template <int W, int NT> __device__ __forceinline__ bool keys_repeat(const SoaTa
     return dup;
 }
 
-// Probe of a table whose keys are all different, over whole groups of U vectors per
-// lane (the rest goes through probe_fast): a match in the home bucket ends the search,
-// so an item is its bucket's four (two) compares, a select, and one rid.  Only an item
-// without a match whose home bucket overflowed is queued (about 1 %, against 3 % when
-// keys may repeat).  What bounds it: instructions and the shared-memory pipe (a bucket
-// of random lanes takes 10.3 cycles per warp), each at 55 %, and the latency that 20
-// warps leave open.  A join of 2^22 with 2^25 4-byte tuples issues 84e6 warp
-// instructions, 128e6 through the general loop; 2^24 x 2^28 1020 -> 828 us.
-template <int W, int U, class Sink>
-__device__ __forceinline__ void probe_unique(const SoaTab<W> &tab, const typename Tup<W>::Vec *Sv, uint32_t nsv,
-                                             Sink &sink, unsigned warp, unsigned nwarps, unsigned lane,
-                                             typename Tup<W>::U *wqk, typename Tup<W>::U *wqr) {
+// Probe one group of U vectors per lane (FULL: every lane holds tuples in all of them),
+// in phases so that the items' shared-memory loads overlap: every item's home bucket
+// (keys), then the place of the match (a select per key) and its rid.  Inserts fill a
+// bucket's slots in order and move past it only once it is full, so a run goes on past
+// the home bucket only if the bucket's last slot is taken AND more inserts tried it than
+// it has slots: such items are queued and their runs walked 32 at a time.  With UNIQ (no
+// key is twice in the table) a match ends the search; otherwise an item with several
+// matches in its home bucket has its whole run walked by the warp.
+template <int W, int U, bool UNIQ, bool FULL, class Sink>
+__device__ __forceinline__ void probe_group_smem(const SoaTab<W> &tab, const typename Tup<W>::Vec *x, const bool *in,
+                                                 Sink &sink, unsigned lane, typename Tup<W>::U *wqk,
+                                                 typename Tup<W>::U *wqr, uint32_t &qn) {
     using T = typename Tup<W>::U;
-    using Vec = typename Tup<W>::Vec;
     constexpr int PV = Tup<W>::kPerVec, IT = U * PV;
     constexpr uint32_t G = SoaTab<W>::G;
+    T k[IT], r[IT];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        if constexpr (W == 4) {
+            k[2 * u] = x[u].x; r[2 * u] = x[u].y; k[2 * u + 1] = x[u].z; r[2 * u + 1] = x[u].w;
+        } else {
+            k[u] = x[u].x; r[u] = x[u].y;
+        }
+    }
+    uint32_t home[IT];
+    T kb[IT][G], first[IT];
+#pragma unroll
+    for (int i = 0; i < IT; ++i) {
+        home[i] = part_bucket<W>(k[i], tab.nb);  // < nb for any key: the load is in bounds
+        tab.ld(home[i], 0, kb[i]);
+    }
+    bool found[IT], w[IT], several[IT], anyw = false, anys = false;
+#pragma unroll
+    for (int i = 0; i < IT; ++i) {
+        const bool live = FULL || in[i / PV];
+        uint32_t sl = home[i] * G + (G - 1), c = kb[i][G - 1] == k[i];
+        bool f = kb[i][G - 1] == k[i];
+#pragma unroll
+        for (int q = (int)G - 2; q >= 0; --q) {
+            const bool h = kb[i][q] == k[i];
+            sl = h ? home[i] * G + q : sl;
+            f |= h;
+            c += h;
+        }
+        first[i] = tab.rptr[sl];
+        several[i] = !UNIQ && live && c > 1;
+        found[i] = live && f && !several[i];
+        w[i] = live && !(UNIQ && f) && !several[i] && kb[i][G - 1] != tab.empty && tab.overflowed(home[i]);
+        anyw |= w[i];
+        anys |= several[i];
+    }
+    sink.template append_found<IT>(found, first, r);
+    if (!UNIQ && __any_sync(0xffffffffu, anys)) {
+#pragma unroll
+        for (int i = 0; i < IT; ++i) {
+            unsigned m = __ballot_sync(0xffffffffu, several[i]);
+            while (m) {
+                const int L = __ffs(m) - 1;
+                m &= m - 1;
+                const T kk = __shfl_sync(0xffffffffu, k[i], L);
+                const T ss = __shfl_sync(0xffffffffu, r[i], L);
+                soa_coop_emit<W>(tab, kk, ss, part_bucket<W>(kk, tab.nb), sink);
+            }
+        }
+    }
+    if (__any_sync(0xffffffffu, anyw)) {
+#pragma unroll
+        for (int i = 0; i < IT; ++i) {
+            const unsigned wm = __ballot_sync(0xffffffffu, w[i]);
+            if (!wm) continue;
+            if (w[i]) {
+                const uint32_t pos = qn + (uint32_t)__popc(wm & ((1u << lane) - 1u));
+                wqk[pos] = k[i];
+                wqr[pos] = r[i];
+            }
+            qn += (uint32_t)__popc(wm);
+            if (qn >= 32) {
+                __syncwarp();
+                drain_walks<W>(tab, wqk + (qn - 32), wqr + (qn - 32), 32, sink);
+                qn -= 32;
+            }
+        }
+    }
+}
+
+// A CTA's probe of a slice of nsv vectors.  What bounds it: instructions and the
+// shared-memory pipe (a bucket of random lanes takes 10.3 cycles per warp), each at
+// 55 %, and the latency that 20 warps leave open.  Queued are 1 % of the items of a table
+// of different keys, 3 % otherwise.  A join of 2^22 with 2^25 4-byte tuples of
+// different build keys issues 84e6 warp instructions; one vector per lane, with the
+// matches of a bucket counted and several bases per store, took 128e6.
+template <int W, int U, bool UNIQ, class Sink>
+__device__ __forceinline__ void probe_smem(const SoaTab<W> &tab, const typename Tup<W>::Vec *Sv, uint32_t nsv,
+                                           Sink &sink, unsigned warp, unsigned nwarps, unsigned lane,
+                                           typename Tup<W>::U *wqk, typename Tup<W>::U *wqr) {
+    using Vec = typename Tup<W>::Vec;
     const uint32_t gstride = nwarps * 32u * U, whole = nsv / (32u * U) * (32u * U);
-    const unsigned lt = (1u << lane) - 1u;
     uint32_t g = warp * 32u * U, qn = 0;
     Vec nxt[U];
     if (g < whole)
 #pragma unroll
         for (int u = 0; u < U; ++u) nxt[u] = ld_stream(Sv + g + u * 32u + lane);
     for (; g < whole; g += gstride) {
-        T k[IT], r[IT];
+        Vec cur[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if constexpr (W == 4) {
-                k[2 * u] = nxt[u].x; r[2 * u] = nxt[u].y; k[2 * u + 1] = nxt[u].z; r[2 * u + 1] = nxt[u].w;
-            } else {
-                k[u] = nxt[u].x; r[u] = nxt[u].y;
-            }
-        }
+        for (int u = 0; u < U; ++u) cur[u] = nxt[u];
         // (the group in registers covers part of the loads' latency, L2 the rest)
         const uint32_t pv = g + 3u * gstride + lane * 8u;
         if (lane < 4u * U && pv < nsv) prefetch_l2(Sv + pv);
         if (g + gstride < whole)
 #pragma unroll
             for (int u = 0; u < U; ++u) nxt[u] = ld_stream(Sv + g + gstride + u * 32u + lane);
-        uint32_t home[IT];
-        T kb[IT][G], first[IT];
-#pragma unroll
-        for (int i = 0; i < IT; ++i) {
-            home[i] = part_bucket<W>(k[i], tab.nb);
-            tab.ld(home[i], 0, kb[i]);
-        }
-        bool found[IT], w[IT], anyw = false;
-#pragma unroll
-        for (int i = 0; i < IT; ++i) {
-            uint32_t sl = home[i] * G + (G - 1);
-            bool f = kb[i][G - 1] == k[i];
-#pragma unroll
-            for (int q = (int)G - 2; q >= 0; --q) {
-                const bool h = kb[i][q] == k[i];
-                sl = h ? home[i] * G + q : sl;
-                f |= h;
-            }
-            found[i] = f;
-            first[i] = tab.rptr[sl];
-            w[i] = !f && kb[i][G - 1] != tab.empty && tab.overflowed(home[i]);
-            anyw |= w[i];
-        }
-        sink.template append_found<IT>(found, first, r);
-        if (__any_sync(0xffffffffu, anyw)) {
-#pragma unroll
-            for (int i = 0; i < IT; ++i) {
-                const unsigned wm = __ballot_sync(0xffffffffu, w[i]);
-                if (!wm) continue;
-                if (w[i]) {
-                    const uint32_t pos = qn + (uint32_t)__popc(wm & lt);
-                    wqk[pos] = k[i];
-                    wqr[pos] = r[i];
-                }
-                qn += (uint32_t)__popc(wm);
-                if (qn >= 32) {
-                    __syncwarp();
-                    drain_walks<W>(tab, wqk + (qn - 32), wqr + (qn - 32), 32, sink);
-                    qn -= 32;
-                }
-            }
-        }
+        probe_group_smem<W, U, UNIQ, true>(tab, cur, nullptr, sink, lane, wqk, wqr, qn);
     }
-    // the slice's last, partial group: a warp's turn if it is the next of its groups
-    probe_fast<W, 1>(tab, Sv, nsv, sink, g == whole ? whole : nsv, 32u, lane, wqk, wqr, qn);
+    if (g == whole && whole < nsv) {  // the slice's last, partial group, in this warp's turn
+        Vec cur[U];
+        bool in[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            in[u] = g + u * 32u + lane < nsv;
+            if (in[u]) cur[u] = ld_stream(Sv + g + u * 32u + lane);
+            else cur[u] = Vec{};
+        }
+        probe_group_smem<W, U, UNIQ, false>(tab, cur, in, sink, lane, wqk, wqr, qn);
+    }
+    if (qn) {
+        __syncwarp();
+        drain_walks<W>(tab, wqk, wqr, qn, sink);
+    }
 }
 
 // Bytes per slot of a partition's shared-memory aggregate table: the key, the
@@ -1339,7 +1265,7 @@ __host__ __device__ constexpr int join_ctas(int nt) { return nt > 512 ? 1 : 2; }
 template <int W, bool AGG, int NT, class Sink, bool FAST>
 __global__ void __launch_bounds__(NT, join_ctas(NT)) partition_join_kernel(
     const PartTask *tasks, uint64_t ntasks, uint64_t lead, const JoinSlot *slots, hj_counters *work, uint32_t cap_max, RecArea ra,
-    uint32_t *oversize, int chk, void *stage_base, uint32_t scap) {
+    uint32_t *oversize, int chk, uint32_t stage_at) {
     using T = typename Tup<W>::U;
     using Vec = typename Tup<W>::Vec;
     constexpr int PV = Tup<W>::kPerVec, U = 2, IT = U * PV;
@@ -1356,8 +1282,8 @@ __global__ void __launch_bounds__(NT, join_ctas(NT)) partition_join_kernel(
         sink.slots = slots;
         sink.ra = ra;
     } else {
-        sink.stage = (typename WarpStageSink<W>::P *)stage_base + ((size_t)blockIdx.x * nwarps + warp) * scap;
-        sink.scap = scap;
+        sink.stage = (typename WarpStageSink<W>::P *)(smem + stage_at + warp * kJoinStageBytes);
+        sink.scap = kJoinStageBytes / (2 * W);
         sink.slots = slots;
     }
     // While more than two of the first `lead` tasks per CTA remain, tasks are taken one ahead: during a
@@ -1541,10 +1467,8 @@ __global__ void __launch_bounds__(NT, join_ctas(NT)) partition_join_kernel(
             } else {
                 if constexpr (FAST) {  // no aggregate, no checksum
                     T *wq = (T *)(smem + walkq_offset(cap_max, 2 * W, W, false)) + (size_t)warp * 2 * kWalkQ;
-                    if (unique)
-                        probe_unique<W, 2>(tab, Sv, nsv, sink, warp, nwarps, lane, wq, wq + kWalkQ);
-                    else  // one vector per thread: the batched walks need the registers
-                        probe_fast<W, 1>(tab, Sv, nsv, sink, warp * 32u, nwarps * 32u, lane, wq, wq + kWalkQ, 0);
+                    if (unique) probe_smem<W, 2, true>(tab, Sv, nsv, sink, warp, nwarps, lane, wq, wq + kWalkQ);
+                    else probe_smem<W, 2, false>(tab, Sv, nsv, sink, warp, nwarps, lane, wq, wq + kWalkQ);
                 } else {
                 const uint32_t gstride = nwarps * 32 * U;
                 Vec cur[U], nxt[U];
@@ -1814,14 +1738,18 @@ static JoinCfg join_cfg(int width, int agg, int checksum, uint64_t expect_r) {
     return JoinCfg{agg ? 1024 : 640, 200ull << 10};
 }
 
+// (two CTAs of an SM then cover each other's waits: 200 joins of 3e7 with 1.2e8 tuples 700 us
+// in the join kernel, 765 us at twice the rows, one CTA per SM)
+uint64_t batch_partition_rows(int width) { return width == 4 ? 2048 : 1024; }
+
 uint64_t partition_join_warps(hj_ctx *c) { return (uint64_t)num_sms(c) * 32; }
 uint64_t partition_join_ctas(hj_ctx *c, int width, int agg, uint64_t expect_r) {
     return (uint64_t)num_sms(c) * join_ctas(join_cfg(width, agg, 1, expect_r).nt);
 }
 
 hj_status partition_join(hj_ctx *c, int width, int agg, const PartTask *tasks, uint64_t ntasks, uint64_t lead,
-                         const JoinSlot *slots, uint64_t expect_r, int checksum, uint32_t *oversize, RecArea ra, void *stage,
-                         uint32_t scap) {
+                         const JoinSlot *slots, uint64_t expect_r, int checksum, uint32_t *oversize, RecArea ra,
+                         bool staged) {
     if (ntasks == 0) return HJ_OK;
     const uint64_t slot_bytes = join_slot_bytes(width, agg, checksum);
     const JoinCfg cfg = join_cfg(width, agg, checksum, expect_r);
@@ -1831,10 +1759,10 @@ hj_status partition_join(hj_ctx *c, int width, int agg, const PartTask *tasks, u
     uint64_t want = (uint64_t)(3.0 * (mean + 6.0 * __builtin_sqrt(mean + 1.0) + 64.0));
     want = (want + 127) / 128 * 128;
     const uint64_t bitmap_bytes = 4096;
-    // the fast probe (no aggregate, no checksum) into the chunk sink adds each
-    // warp's walk queue, within what the shape's CTAs per SM can have (two
-    // 512-thread CTAs share an SM)
-    const uint64_t qbytes = (!agg && !checksum) ? (uint64_t)(cfg.nt / 32) * kWalkQ * 2 * width : 0;
+    // the fast probe (no aggregate, no checksum) adds each warp's walk queue, staged
+    // output its buffer, within what the shape's CTAs per SM can have
+    const uint64_t stage_bytes = staged ? (uint64_t)(cfg.nt / 32) * kJoinStageBytes : 0;
+    const uint64_t qbytes = ((!agg && !checksum) ? (uint64_t)(cfg.nt / 32) * kWalkQ * 2 * width : 0) + stage_bytes;
     const uint64_t total_max = join_ctas(cfg.nt) == 2 ? (112ull << 10) : (222ull << 10);
     const uint64_t budget = std::min<uint64_t>(cfg.smem_limit + qbytes, total_max) - qbytes;
     uint64_t max_slots = agg ? (budget - bitmap_bytes) / slot_bytes / 128 * 128
@@ -1849,7 +1777,7 @@ hj_status partition_join(hj_ctx *c, int width, int agg, const PartTask *tasks, u
         auto kern = partition_join_kernel<WW, AA, NT, SK<WW>, FF>;                                              \
         HJ_TRY(allow_max_smem(c, (const void *)kern));                                                         \
         HJ_LAUNCH(c, "partition_join", kern, grid, NT, smem, tasks, ntasks, lead, slots, c->d_ctr, (uint32_t)cap_max, \
-                  ra, oversize, checksum, stage, scap);                                                         \
+                  ra, oversize, checksum, (uint32_t)(smem - stage_bytes));                                                         \
     } while (0)
 #define HJ_PJ_NT(WW, AA, SK, FF)                                \
     do {                                                        \
@@ -1863,7 +1791,7 @@ hj_status partition_join(hj_ctx *c, int width, int agg, const PartTask *tasks, u
     } while (0)
 #define HJ_PJ_SK(WW)                                            \
     do {                                                        \
-        if (stage) HJ_PJ_F(WW, WarpStageSink);                       \
+        if (staged) HJ_PJ_F(WW, WarpStageSink);                       \
         else HJ_PJ_F(WW, ChunkSink);                             \
     } while (0)
     if (width == 4) {

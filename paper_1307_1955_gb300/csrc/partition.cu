@@ -167,7 +167,7 @@ template <int W>
 __global__ void __launch_bounds__(kHistThreads) hist_kernel(const void *in, uint64_t n_total, const uint64_t *seg_off,
                                                             uint64_t nseg, const unsigned long long *cb,
                                                             uint64_t chunk, int shift, int bits, int pad,
-                                                            uint32_t *H, const void *const *seg_ptrs) {
+                                                            uint32_t *H) {
     using U = typename Tup<W>::U;
     constexpr int PV = Tup<W>::kPerVec, SV = Sector<W>::kTuples;
     extern __shared__ uint32_t hist[];
@@ -179,10 +179,8 @@ __global__ void __launch_bounds__(kHistThreads) hist_kernel(const void *in, uint
         return;
     }
     const ChunkPos cp = chunk_pos(seg_off, nseg, cb, chunk, g);
-    // tuples come from `in` (global row index), or from the segment's own array
-    const void *src = seg_ptrs ? seg_ptrs[cp.s] : in;
-    const uint64_t ioff = seg_ptrs ? seg_off[cp.s] : 0;
-    const uint64_t lo = cp.lo - ioff, hi = cp.hi - ioff;
+    const void *src = in;
+    const uint64_t lo = cp.lo, hi = cp.hi;
     __syncthreads();
     // whole vectors of the chunk: no per-tuple range tests, 32-bit indices
     const uint64_t va = (lo + PV - 1) / PV, vb = hi / PV;
@@ -329,18 +327,16 @@ __device__ __forceinline__ bool chunk_runs(const RunGeom &rg, uint64_t chunk, ui
 // sectors, writes it to H1[g * P + d] and takes the rows of its run among the
 // digit's runs with one atomic add on the digit's total T1[d] (zero beforehand).
 template <int W>
-__global__ void __launch_bounds__(kHistThreads) hist1_kernel(const void *in, uint64_t n, uint64_t chunk, int bits,
-                                                             uint32_t *H1, uint32_t *base1, uint32_t *T1) {
+__device__ __forceinline__ void hist_chunk(const void *in, uint32_t n, int bits, uint32_t *hist, uint32_t *H,
+                                           uint32_t *base, uint32_t *T) {
     using Vec = typename Tup<W>::Vec;
     constexpr int PV = Tup<W>::kPerVec, SV = Sector<W>::kTuples;
-    extern __shared__ uint32_t hist[];
     const uint32_t P = 1u << bits;
-    const uint64_t g = blockIdx.x, lo = g * chunk, hi = min(lo + chunk, n);
     for (uint32_t d = threadIdx.x; d < P; d += blockDim.x) hist[d] = 0;
     __syncthreads();
     // chunks start on whole vectors; a 4-byte relation's odd last row is read alone
-    const Vec *vp = (const Vec *)in + lo / PV;
-    const uint32_t nv = (uint32_t)((hi - lo) / PV);
+    const Vec *vp = (const Vec *)in;
+    const uint32_t nv = n / PV;
     for (uint32_t v0 = 0; v0 < nv; v0 += blockDim.x * kHistUnroll) {
         Vec x[kHistUnroll];
 #pragma unroll
@@ -358,17 +354,25 @@ __global__ void __launch_bounds__(kHistThreads) hist1_kernel(const void *in, uin
         }
     }
     if constexpr (W == 4) {
-        if (threadIdx.x == 0 && (hi - lo) % 2) {
-            const uint32_t k = ((const uint32_t *)in)[2 * (hi - 1)];
+        if (threadIdx.x == 0 && n % 2) {
+            const uint32_t k = ((const uint32_t *)in)[2 * (size_t)(n - 1)];
             atomicAdd(&hist[digit_of(key_hash<W>(k), 0, bits)], 1u);
         }
     }
     __syncthreads();
     for (uint32_t d = threadIdx.x; d < P; d += blockDim.x) {
         const uint32_t c = (hist[d] + SV - 1) / SV * SV;
-        H1[g * P + d] = c;
-        base1[g * P + d] = c ? atomicAdd(&T1[d], c) : 0u;
+        H[d] = c;
+        base[d] = c ? atomicAdd(&T[d], c) : 0u;
     }
+}
+
+template <int W>
+__global__ void __launch_bounds__(kHistThreads) hist1_kernel(const void *in, uint64_t n, uint64_t chunk, int bits,
+                                                             uint32_t *H1, uint32_t *base1, uint32_t *T1) {
+    extern __shared__ uint32_t hist[];
+    const uint64_t g = blockIdx.x, lo = g * chunk, hi = min(lo + chunk, n), at = g << bits;
+    hist_chunk<W>((const char *)in + lo * (2 * W), (uint32_t)(hi - lo), bits, hist, H1 + at, base1 + at, T1);
 }
 
 // ----------------------------------------------------------------- scatter
@@ -644,7 +648,7 @@ template <int W>
 __global__ void __launch_bounds__(kTmaThreads, 1) scatter_tma_kernel(
     const void *in, uint64_t n_total, const uint64_t *seg_off, uint64_t nseg, const unsigned long long *cb,
     uint64_t chunk, int shift, int bits, const unsigned long long *Hs, void *out, int pad, uint64_t sent_k0,
-    uint64_t sent_k1, unsigned long long *fault, const void *const *seg_ptrs, uint32_t wait_limit) {
+    uint64_t sent_k1, unsigned long long *fault, uint32_t wait_limit) {
     using U = typename Tup<W>::U;
     using TS = TmaShape<W>;
     using Slot = typename SortSlot<W>::T;
@@ -676,11 +680,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) scatter_tma_kernel(
     const uint64_t obase = seg_start / SV * SV;
     Slot *outp = (Slot *)out + obase;
     const uint64_t tb = 2 * W;
-    // tuples come from `in` (global row index), or from the segment's own array
-    const void *src = seg_ptrs ? seg_ptrs[cp.s] : in;
-    const uint64_t ioff = seg_ptrs ? seg_off[cp.s] : 0;
-    const uint64_t nsrc = seg_ptrs ? seg_off[cp.s + 1] - seg_off[cp.s] : n_total;
-    const uint64_t last16 = (nsrc * tb) / 16 * 16;  // bytes of `src` a 16-byte copy may touch
+    const uint64_t last16 = (n_total * tb) / 16 * 16;  // bytes of `in` a 16-byte copy may touch
     for (uint32_t d = threadIdx.x; d < P; d += blockDim.x) {
         DigitMeta m;
         m.gcur = (uint32_t)(seg_off[0] + Hs[row + (uint64_t)d * cp.nch + cp.cidx] - obase);
@@ -695,11 +695,11 @@ __global__ void __launch_bounds__(kTmaThreads, 1) scatter_tma_kernel(
         fence_mbar_init();
     }
     __syncthreads();
-    // byte range of src staged for the tile of global rows [t0, t1): 16-byte
+    // byte range of `in` staged for the tile of global rows [t0, t1): 16-byte
     // aligned, inside the array
     auto stage_range = [&](uint64_t t0, uint64_t t1, uint64_t *b0, uint64_t *b1) {
-        *b0 = ((t0 - ioff) * tb) / 16 * 16;
-        uint64_t e = ((t1 - ioff) * tb + 15) / 16 * 16;
+        *b0 = (t0 * tb) / 16 * 16;
+        uint64_t e = (t1 * tb + 15) / 16 * 16;
         *b1 = e < last16 ? e : last16;
     };
     auto issue = [&](uint64_t t0, uint64_t t1) {
@@ -707,7 +707,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) scatter_tma_kernel(
         stage_range(t0, t1, &b0, &b1);
         if (b1 > b0) {
             mbar_expect_tx(bar, (uint32_t)(b1 - b0));
-            bulk_g2s(stage_s, (const char *)src + b0, (uint32_t)(b1 - b0), bar);
+            bulk_g2s(stage_s, (const char *)in + b0, (uint32_t)(b1 - b0), bar);
         } else {
             mbar_expect_tx(bar, 0);
         }
@@ -731,7 +731,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) scatter_tma_kernel(
         uint64_t b0, b1;
         stage_range(t0, t1, &b0, &b1);
         const uint32_t ntile = (uint32_t)(t1 - t0);
-        const uint32_t skew = (uint32_t)(t0 - ioff - b0 / tb);            // 0 or 1 leading slots
+        const uint32_t skew = (uint32_t)(t0 - b0 / tb);            // 0 or 1 leading slots
         const uint32_t staged = b1 > b0 ? (uint32_t)((b1 - b0) / tb) : 0u;
         const uint32_t nstaged = staged > skew ? staged - skew : 0u;       // tuples of the tile in the stage
         U k[IT], r[IT];
@@ -741,7 +741,7 @@ __global__ void __launch_bounds__(kTmaThreads, 1) scatter_tma_kernel(
             const uint32_t t = (uint32_t)i * kTmaThreads + threadIdx.x;
             Slot sl;
             if (t < nstaged) sl = stage[t + skew];
-            else if (t < ntile) sl = ((const Slot *)src)[t0 - ioff + t];
+            else if (t < ntile) sl = ((const Slot *)in)[t0 + t];
             else {
                 if constexpr (W == 4) sl = 0ull;
                 else sl = make_ulonglong2(0ull, 0ull);
@@ -892,54 +892,59 @@ __global__ void __launch_bounds__(kTmaThreads, 1) scatter_tma_kernel(
 // tiles ahead 301).  Sectors written by a lane each, carried tuples moved to the front
 // and no L2 prefetch took 387 us, and 401 .. 430 us at 2^5 .. 2^8 digits (now 220).
 constexpr int kRegionThreads = 1024;
+constexpr int kRegionVecs = 4;  // 16-byte vectors per thread per tile
+constexpr size_t kRegionSmem = 227u * 1024u - 1024u;
 
-template <int W, int LOG2P> struct RegionShape {
-    static constexpr uint32_t P = 1u << LOG2P, PITCH = P + 1;
-    static constexpr uint32_t SV = (uint32_t)Sector<W>::kTuples;
+// Shape of a region scatter at 2^lp digits.
+template <int W> struct RegionShape {
     static constexpr int PV = Tup<W>::kPerVec;
-    static constexpr int VPT = 4;                    // 16-byte vectors per thread per tile
-    static constexpr int IT = VPT * PV;              // tuples per thread per tile
-    static constexpr uint32_t T = kRegionThreads * IT;
-    static constexpr uint32_t LPD = LOG2P >= 11 ? 2 : 4;  // lanes per flushed digit
-    static constexpr uint32_t LINE = LPD * SV;            // rows of a whole flush
-    // groups of LPD lanes that share a digit's flush (few digits hold many lines each)
-    static constexpr uint32_t GPD = kRegionThreads / LPD > P ? kRegionThreads / LPD / P : 1;
-    static constexpr size_t kBudget = 227u * 1024u - 1024u;  // dynamic shared memory
+    static constexpr uint32_t SV = (uint32_t)Sector<W>::kTuples;
+    static constexpr uint32_t T = kRegionThreads * kRegionVecs * PV;  // tuples per tile
+    __host__ __device__ static constexpr uint32_t pitch(uint32_t lp) { return (1u << lp) + 1u; }
     // slots per digit: what shared memory holds (three tiles' tuples and more)
-    static constexpr uint32_t K = (uint32_t)((kBudget - (size_t)P * 12) / ((size_t)PITCH * 2 * W)) / SV * SV;
-    static constexpr size_t kSmem = ((size_t)K * PITCH * 2 * W + (size_t)P * 12 + 15) / 16 * 16;
-    static_assert(K >= LINE + SV, "a digit holds a flush and a sector more");
-    static_assert(K + T < 65536, "tuples held, refused ones of a tile included, count in 16 bits");
+    __host__ __device__ static constexpr uint32_t slots(uint32_t lp) {
+        return (uint32_t)((kRegionSmem - 16 - ((size_t)12 << lp)) / ((size_t)pitch(lp) * 2 * W)) / SV * SV;
+    }
+    __host__ __device__ static constexpr uint32_t lanes(uint32_t lp) { return lp >= 11 ? 2 : 4; }  // per flushed digit
+    static_assert(slots(11) >= lanes(11) * SV + SV && slots(10) >= lanes(10) * SV + SV,
+                  "a digit holds a flush and a sector more");
+    static_assert(slots(1) + T < 65536, "tuples held, refused ones of a tile included, count in 16 bits");
 };
 
+// Shared memory of a region scatter: the rings, then three words per digit.
+template <int W> struct RegionMem {
+    using Slot = typename SortSlot<W>::T;
+    Slot *ring;      // slots(lp) * pitch(lp)
+    uint32_t *word;  // P: tuples held (may pass the slots) | first slot << 16
+    uint32_t *nxt;   // P: next row of the run
+    uint32_t *tail;  // P: rows at and above belong to refused tuples
+    __device__ __forceinline__ RegionMem(unsigned char *smem, uint32_t lp) {
+        using RS = RegionShape<W>;
+        ring = (Slot *)smem;
+        word = (uint32_t *)(ring + (size_t)RS::slots(lp) * RS::pitch(lp));
+        nxt = word + (1u << lp);
+        tail = nxt + (1u << lp);
+    }
+};
+
+// The scatter of one chunk, rows [0, nrows) of vsrc, on hash bits [shift, shift + lp)
+// to runs [nxt, tail) of outp (set by the caller; row 0 of outp is `al` rows into a
+// line).  LOG2P is lp, or 0 for a fan-out known at run time.  All threads call.
 template <int W, int LOG2P>
-__global__ void __launch_bounds__(kRegionThreads, 1) scatter_region_kernel(
-    const void *in, uint64_t n_total, RunGeom rg, uint64_t chunk, int shift, void *out, uint64_t sent_k0,
-    uint64_t sent_k1, const void *const *seg_ptrs, unsigned long long *fault) {
+__device__ __forceinline__ void region_chunk(const RegionMem<W> &rm, uint32_t lp_rt, const typename Tup<W>::Vec *vsrc,
+                                             uint32_t nrows, typename SortSlot<W>::T *outp, uint32_t al, int shift,
+                                             uint64_t sent_k0, uint64_t sent_k1) {
     using U = typename Tup<W>::U;
     using Vec = typename Tup<W>::Vec;
-    using RS = RegionShape<W, LOG2P>;
+    using RS = RegionShape<W>;
     using Slot = typename SortSlot<W>::T;
-    constexpr uint32_t P = RS::P, K = RS::K, PITCH = RS::PITCH, SV = RS::SV, LPD = RS::LPD, LINE = RS::LINE;
-    constexpr int PV = RS::PV, VPT = RS::VPT, NT = kRegionThreads;
-    extern __shared__ __align__(16) unsigned char smem[];
-    Slot *ring = (Slot *)smem;                                    // K * PITCH
-    uint32_t *word = (uint32_t *)(ring + (size_t)K * PITCH);     // P: tuples held (may pass K) | first slot << 16
-    uint32_t *nxt = word + P;                                     // P: next row of the run
-    uint32_t *tail = nxt + P;                                     // P: rows at and above belong to refused tuples
-
-    const uint64_t g = blockIdx.x;
-    ChunkPos cp;
-    uint64_t obase;
-    if (!chunk_runs<P, NT>(rg, chunk, g, SV, &cp, &obase, nxt, tail, fault)) return;
-    Slot *outp = (Slot *)out + obase;
-    const uint32_t al = (uint32_t)(obase % LINE);
-    // this chunk's tuples: rows [lo, hi) of src; lo is a whole number of vectors
-    // (chunks, segments and arrays start on 16 bytes)
-    const void *src = seg_ptrs ? seg_ptrs[cp.s] : in;
-    const uint64_t ioff = seg_ptrs ? rg.seg_off[cp.s] : 0;
-    const Vec *vsrc = (const Vec *)src + (cp.lo - ioff) / PV;
-    const uint32_t nrows = (uint32_t)(cp.hi - cp.lo);
+    const uint32_t lp = LOG2P ? (uint32_t)LOG2P : lp_rt;
+    const uint32_t P = 1u << lp, K = RS::slots(lp), PITCH = RS::pitch(lp), LPD = RS::lanes(lp);
+    constexpr uint32_t SV = RS::SV;
+    const uint32_t LINE = LPD * SV;  // rows of a whole flush (a power of two)
+    constexpr int PV = RS::PV, VPT = kRegionVecs, NT = kRegionThreads;
+    Slot *ring = rm.ring;
+    uint32_t *word = rm.word, *nxt = rm.nxt, *tail = rm.tail;
     for (uint32_t d = threadIdx.x; d < P; d += NT) word[d] = 0;
     // vector j of the tile [t0, lim) for this thread; a last vector holding one
     // tuple of a 4-byte relation is read with an 8-byte load (nothing past the
@@ -1012,30 +1017,29 @@ __global__ void __launch_bounds__(kRegionThreads, 1) scatter_region_kernel(
             }
         }
         __syncthreads();
-        // 2. flush up to the last line boundary
-        const uint32_t q = threadIdx.x % LPD, grp = threadIdx.x / LPD;
-        constexpr uint32_t NG = NT / LPD;
+        // 2. flush up to the last line boundary; with few digits, which hold many lines
+        // each, several groups of LPD lanes share a digit
+        const uint32_t NG = NT / LPD, q = threadIdx.x & (LPD - 1u), grp = threadIdx.x / LPD;
+        const uint32_t gpd = NG > P ? NG >> lp : 1u;
 #pragma unroll
         for (uint32_t r0 = 0; r0 < (P > NG ? P : NG); r0 += NG) {
-            const uint32_t d = (r0 + grp) % P, part = grp / P;  // (part: 0 unless groups share a digit)
-            const bool act = RS::GPD * P >= NG || grp < RS::GPD * P;
+            const uint32_t d = (r0 + grp) & (P - 1u), part = grp >> lp;  // (part: 0 unless groups share a digit)
             const uint32_t v = word[d], raw = v & 0xFFFFu, held = raw < K ? raw : K, head = v >> 16;
-            const uint32_t row = nxt[d], first = LINE - (row + al) % LINE;  // rows to the first boundary
+            const uint32_t row = nxt[d], first = LINE - ((row + al) & (LINE - 1u));  // rows to the first boundary
             const uint32_t nl = held < first ? 0u : 1u + (held - first) / LINE;
-            if (act)
-                for (uint32_t i = part; i < nl; i += RS::GPD) {
-                    const uint32_t at = i ? first + (i - 1) * LINE : 0u, len = i ? LINE : first;
-                    if (q * SV >= len) continue;
-                    uint32_t s = head + at + q * SV;  // (whole sectors, as K: no wrap inside one)
-                    if (s >= K) s -= K;
-                    Slot tup[SV];
+            for (uint32_t i = part; i < nl; i += gpd) {
+                const uint32_t at = i ? first + (i - 1) * LINE : 0u, len = i ? LINE : first;
+                if (q * SV >= len) continue;
+                uint32_t s = head + at + q * SV;  // (whole sectors, as K: no wrap inside one)
+                if (s >= K) s -= K;
+                Slot tup[SV];
 #pragma unroll
-                    for (uint32_t x = 0; x < SV; ++x) tup[x] = ring[(s + x) * PITCH + d];
-                    st_sector(outp + row + at + q * SV, (const unsigned long long *)tup);
-                }
-            if (RS::GPD > 1) __syncthreads();
+                for (uint32_t x = 0; x < SV; ++x) tup[x] = ring[(s + x) * PITCH + d];
+                st_sector(outp + row + at + q * SV, (const unsigned long long *)tup);
+            }
+            if (gpd > 1) __syncthreads();
             else __syncwarp();  // every lane has read its digit's word
-            if (q == 0 && part == 0 && act && (nl || raw != held)) {
+            if (q == 0 && part == 0 && (nl || raw != held)) {
                 const uint32_t w = nl ? first + (nl - 1) * LINE : 0u;
                 uint32_t h = head + w;
                 if (h >= K) h -= K;
@@ -1063,14 +1067,87 @@ __global__ void __launch_bounds__(kRegionThreads, 1) scatter_region_kernel(
 }
 
 template <int W, int LOG2P>
-static hj_status launch_region(hj_ctx *c, unsigned grid, const void *in, uint64_t n_total, const RunGeom &rg,
-                               uint64_t chunk, int shift, void *out, uint64_t k0, uint64_t k1,
-                               const void *const *seg_ptrs) {
+__global__ void __launch_bounds__(kRegionThreads, 1) scatter_region_kernel(
+    const void *in, RunGeom rg, uint64_t chunk, int shift, void *out, uint64_t sent_k0, uint64_t sent_k1,
+    unsigned long long *fault) {
+    using Slot = typename SortSlot<W>::T;
+    extern __shared__ __align__(16) unsigned char smem[];
+    const RegionMem<W> rm(smem, LOG2P);
+    ChunkPos cp;
+    uint64_t obase;
+    if (!chunk_runs<(1u << LOG2P), kRegionThreads>(rg, chunk, blockIdx.x, RegionShape<W>::SV, &cp, &obase, rm.nxt, rm.tail,
+                                                   fault))
+        return;
+    // (lo is a whole number of vectors: chunks, segments and arrays start on 16 bytes)
+    region_chunk<W, LOG2P>(rm, LOG2P, (const typename Tup<W>::Vec *)in + cp.lo / Tup<W>::kPerVec,
+                           (uint32_t)(cp.hi - cp.lo), (Slot *)out + obase,
+                           (uint32_t)(obase % (RegionShape<W>::lanes(LOG2P) * RegionShape<W>::SV)), shift, sent_k0,
+                           sent_k1);
+}
+
+// ------------------------------------------------------- passes of a batch
+// Partition passes of many relations, each on its own number of digits, in two
+// launches: every chunk of every relation counts its digits and takes its runs' rows
+// (as hist1_kernel), then every chunk scatters.  A relation's output is its own
+// range of `out` (part.obase rows on, sized for its padding by the host), so nothing is
+// scanned across relations.  A pass per relation or per group of one fan-out left
+// most SMs idle: 200 joins took 2 x 7 passes of ten launches each, 1.5 ms for 1.2 GB.
+template <int W>
+__global__ void __launch_bounds__(kHistThreads) batch_hist_kernel(const BatchChunk *chunks, uint32_t *H, uint32_t *base,
+                                                                  uint32_t *T) {
+    extern __shared__ uint32_t hist[];
+    const BatchChunk bc = chunks[blockIdx.x];
+    hist_chunk<W>(bc.src, bc.n, (int)bc.bits, hist, H + bc.h_at, base + bc.h_at, T + bc.t_at);
+}
+
+struct BatchPadKeys {
+    uint64_t k1[12];  // second padding key by bits (the first is 0)
+};
+
+template <int W>
+__global__ void __launch_bounds__(kRegionThreads, 1) batch_scatter_kernel(const BatchChunk *chunks, const uint32_t *H,
+                                                                          const uint32_t *base, const uint32_t *T,
+                                                                          void *out, uint64_t *part_off,
+                                                                          BatchPadKeys pk) {
+    using Slot = typename SortSlot<W>::T;
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ unsigned long long sc[33];
+    const BatchChunk bc = chunks[blockIdx.x];
+    const uint32_t lp = bc.bits, P = 1u << lp;
+    const RegionMem<W> rm(smem, lp);
+    // digit d's partition starts at the sum of the padded totals of digits < d
+    constexpr uint32_t PER = 2;  // digits per thread, consecutive (P <= 2^11)
+    unsigned long long v[PER], sum = 0, tot;
+#pragma unroll
+    for (uint32_t q = 0; q < PER; ++q) {
+        const uint32_t d = threadIdx.x * PER + q;
+        v[q] = d < P ? T[bc.t_at + d] : 0u;
+        sum += v[q];
+    }
+    unsigned long long at = block_exclusive_scan<unsigned long long>(sum, sc, &tot);
+#pragma unroll
+    for (uint32_t q = 0; q < PER; ++q) {
+        const uint32_t d = threadIdx.x * PER + q;
+        if (d < P) {
+            rm.nxt[d] = (uint32_t)at + base[bc.h_at + d];
+            rm.tail[d] = rm.nxt[d] + H[bc.h_at + d];
+            if (bc.lead) part_off[bc.t_at + d] = bc.obase + at;
+        }
+        at += v[q];
+    }
+    if (bc.lead && threadIdx.x == 0) part_off[bc.t_at + P] = bc.obase + tot;
+    // (obase: whole lines)
+    region_chunk<W, 0>(rm, lp, (const typename Tup<W>::Vec *)bc.src, bc.n, (Slot *)out + bc.obase, 0u, 0, 0ull,
+                       pk.k1[lp]);
+}
+
+template <int W, int LOG2P>
+static hj_status launch_region(hj_ctx *c, unsigned grid, const void *in, const RunGeom &rg, uint64_t chunk, int shift,
+                               void *out, uint64_t k0, uint64_t k1) {
     auto kern = scatter_region_kernel<W, LOG2P>;
-    const size_t smem = RegionShape<W, LOG2P>::kSmem;
     HJ_TRY(allow_max_smem(c, (const void *)kern));
-    HJ_LAUNCH(c, "partition_scatter", kern, grid, kRegionThreads, smem, in, n_total, rg, chunk, shift, out, k0, k1,
-              seg_ptrs, &c->d_ctr->fault);
+    HJ_LAUNCH(c, "partition_scatter", kern, grid, kRegionThreads, kRegionSmem, in, rg, chunk, shift, out, k0, k1,
+              &c->d_ctr->fault);
     return HJ_OK;
 }
 
@@ -1148,7 +1225,7 @@ __device__ __forceinline__ void red_release_add_cta(uint32_t *p, uint32_t v) {
 template <int W, int LOG2P>
 __global__ void __launch_bounds__(kRingThreads, 1) scatter_ring_kernel(
     const void *in, uint64_t n_total, RunGeom rg, uint64_t chunk, int shift, void *out, uint64_t sent_k0,
-    uint64_t sent_k1, const void *const *seg_ptrs, unsigned long long *fault, uint64_t max_passes) {
+    uint64_t sent_k1, unsigned long long *fault, uint64_t max_passes) {
     using U = typename Tup<W>::U;
     using Vec = typename Tup<W>::Vec;
     using RS = RingShape<W, LOG2P>;
@@ -1168,9 +1245,7 @@ __global__ void __launch_bounds__(kRingThreads, 1) scatter_ring_kernel(
     uint64_t obase;
     if (!chunk_runs<P, kRingThreads>(rg, chunk, g, SV, &cp, &obase, nxt, tail, fault)) return;
     Slot *outp = (Slot *)out + obase;
-    const void *src = seg_ptrs ? seg_ptrs[cp.s] : in;
-    const uint64_t ioff = seg_ptrs ? rg.seg_off[cp.s] : 0;
-    const Vec *vsrc = (const Vec *)src + (cp.lo - ioff) / PV;  // chunks start on whole vectors
+    const Vec *vsrc = (const Vec *)in + cp.lo / PV;  // chunks start on whole vectors
     const uint32_t nrows = (uint32_t)(cp.hi - cp.lo);
     const uint32_t dk0 = (uint32_t)(key_hash<W>((U)sent_k0) >> shift) & (P - 1u);
     auto empty_key = [&](uint32_t d) -> U { return d != dk0 ? (U)sent_k0 : (U)sent_k1; };
@@ -1312,14 +1387,13 @@ __global__ void __launch_bounds__(kRingThreads, 1) scatter_ring_kernel(
 
 template <int W, int LOG2P>
 static hj_status launch_ring(hj_ctx *c, unsigned grid, const void *in, uint64_t n_total, const RunGeom &rg,
-                             uint64_t chunk, int shift, void *out, uint64_t k0, uint64_t k1,
-                             const void *const *seg_ptrs) {
+                             uint64_t chunk, int shift, void *out, uint64_t k0, uint64_t k1) {
     auto kern = scatter_ring_kernel<W, LOG2P>;
     HJ_TRY(allow_max_smem(c, (const void *)kern));
     const uint64_t passes = c->wait_limit ? std::min<uint64_t>(c->wait_limit, kRingMaxPasses) : kRingMaxPasses;
     constexpr size_t smem = RingShape<W, LOG2P>::kSmem;
     HJ_LAUNCH(c, "partition_scatter", kern, grid, kRingThreads, smem, in, n_total, rg, chunk, shift, out, k0, k1,
-              seg_ptrs, &c->d_ctr->fault, passes);
+              &c->d_ctr->fault, passes);
     return HJ_OK;
 }
 
@@ -1337,13 +1411,13 @@ static bool use_ring(const hj_ctx *c, int bits) {
 template <int W>
 static hj_status launch_region_bits(hj_ctx *c, int bits, unsigned grid, const void *in, uint64_t n_total,
                                     const RunGeom &rg, uint64_t chunk, int shift, void *out, uint64_t k0,
-                                    uint64_t k1, const void *const *seg_ptrs) {
+                                    uint64_t k1) {
 #define HJ_RG(B)                                                                                                 \
     case B:                                                                                                      \
-        return launch_region<W, B>(c, grid, in, n_total, rg, chunk, shift, out, k0, k1, seg_ptrs)
+        return launch_region<W, B>(c, grid, in, rg, chunk, shift, out, k0, k1)
 #define HJ_RI(B)                                                                                                 \
     case B:                                                                                                      \
-        return launch_ring<W, B>(c, grid, in, n_total, rg, chunk, shift, out, k0, k1, seg_ptrs)
+        return launch_ring<W, B>(c, grid, in, n_total, rg, chunk, shift, out, k0, k1)
     if (use_ring(c, bits)) {
         switch (bits) {
             HJ_RI(9); HJ_RI(10); HJ_RI(11);
@@ -1414,13 +1488,10 @@ static void sentinel_keys(int width, int shift, int bits, uint64_t *k0, uint64_t
 }
 
 hj_status partition_pass(hj_ctx *c, int width, const void *in, uint64_t n_total, const uint64_t *seg_off,
-                         uint64_t nseg, int shift, int bits, void *out, uint64_t *part_off, int pad,
-                         const void *const *seg_ptrs) {
+                         uint64_t nseg, int shift, int bits, void *out, uint64_t *part_off, int pad) {
     if (bits < 1 || bits > 12) return set_err(c, HJ_E_INVALID, "partition pass bits %d outside [1, 12]", bits);
     const uint64_t P = 1ull << bits;
     const ScatterCfg cfg = scatter_cfg(width, bits);
-    if (seg_ptrs && !cfg.tma)
-        return set_err(c, HJ_E_UNSUPPORTED, "per-segment inputs need a fan-out of at most 2^11");
     const uint64_t chunk = pass_chunk(c, width, bits, n_total);
     const uint64_t max_chunks = (n_total + chunk - 1) / chunk + nseg;
 
@@ -1441,9 +1512,9 @@ hj_status partition_pass(hj_ctx *c, int width, const void *in, uint64_t n_total,
     }
     size_t hsmem = P * 4;
     if (width == 4)
-        HJ_LAUNCH(c, "partition_hist", hist_kernel<4>, (unsigned)max_chunks, kHistThreads, hsmem, in, n_total, seg_off, nseg, cb, chunk, shift, bits, pad, H, seg_ptrs);
+        HJ_LAUNCH(c, "partition_hist", hist_kernel<4>, (unsigned)max_chunks, kHistThreads, hsmem, in, n_total, seg_off, nseg, cb, chunk, shift, bits, pad, H);
     else
-        HJ_LAUNCH(c, "partition_hist", hist_kernel<8>, (unsigned)max_chunks, kHistThreads, hsmem, in, n_total, seg_off, nseg, cb, chunk, shift, bits, pad, H, seg_ptrs);
+        HJ_LAUNCH(c, "partition_hist", hist_kernel<8>, (unsigned)max_chunks, kHistThreads, hsmem, in, n_total, seg_off, nseg, cb, chunk, shift, bits, pad, H);
     HJ_TRY(scan_counts(c, H, max_chunks * P, Hs));
     {
         uint64_t n = nseg * P + 1;
@@ -1465,11 +1536,9 @@ hj_status partition_pass(hj_ctx *c, int width, const void *in, uint64_t n_total,
     if (cfg.tma && pad) {
         const RunGeom rg{seg_off, nseg, cb, Hs, nullptr, nullptr, nullptr, 0, 0, nullptr};
         if (width == 4)
-            HJ_TRY(launch_region_bits<4>(c, bits, (unsigned)max_chunks, in, n_total, rg, chunk, shift, out, k0, k1,
-                                         seg_ptrs));
+            HJ_TRY(launch_region_bits<4>(c, bits, (unsigned)max_chunks, in, n_total, rg, chunk, shift, out, k0, k1));
         else
-            HJ_TRY(launch_region_bits<8>(c, bits, (unsigned)max_chunks, in, n_total, rg, chunk, shift, out, k0, k1,
-                                         seg_ptrs));
+            HJ_TRY(launch_region_bits<8>(c, bits, (unsigned)max_chunks, in, n_total, rg, chunk, shift, out, k0, k1));
     } else if (cfg.tma) {
         // mbarrier polls per tile: the default, or n - 1 under a test limit of n (so
         // that n = 1 gives up at the first wait, however long the hardware suspends
@@ -1478,13 +1547,11 @@ hj_status partition_pass(hj_ctx *c, int width, const void *in, uint64_t n_total,
         if (width == 4) {
             HJ_TRY(allow_max_smem(c, (const void *)scatter_tma_kernel<4>));
             HJ_LAUNCH(c, "partition_scatter", scatter_tma_kernel<4>, (unsigned)max_chunks, kTmaThreads, tma_smem, in,
-                      n_total, seg_off, nseg, cb, chunk, shift, bits, Hs, out, pad, k0, k1, &c->d_ctr->fault, seg_ptrs,
-                      polls);
+                      n_total, seg_off, nseg, cb, chunk, shift, bits, Hs, out, pad, k0, k1, &c->d_ctr->fault, polls);
         } else {
             HJ_TRY(allow_max_smem(c, (const void *)scatter_tma_kernel<8>));
             HJ_LAUNCH(c, "partition_scatter", scatter_tma_kernel<8>, (unsigned)max_chunks, kTmaThreads, tma_smem, in,
-                      n_total, seg_off, nseg, cb, chunk, shift, bits, Hs, out, pad, k0, k1, &c->d_ctr->fault, seg_ptrs,
-                      polls);
+                      n_total, seg_off, nseg, cb, chunk, shift, bits, Hs, out, pad, k0, k1, &c->d_ctr->fault, polls);
         }
     } else if (width == 4) {
         if (cfg.nt == 512) HJ_SC(4, 512, 8); else HJ_SC(4, 1024, 2);
@@ -1526,9 +1593,36 @@ hj_status partition_pass1(hj_ctx *c, int width, const void *in, uint64_t n, int 
     const RunGeom rg{nullptr, 1, nullptr, nullptr, H1.as<uint32_t>(), base1.as<uint32_t>(), T1.as<uint32_t>(), n,
                      nch, part_off};
     if (width == 4)
-        HJ_TRY(launch_region_bits<4>(c, bits, (unsigned)nch, in, n, rg, chunk, 0, out, k0, k1, nullptr));
+        HJ_TRY(launch_region_bits<4>(c, bits, (unsigned)nch, in, n, rg, chunk, 0, out, k0, k1));
     else
-        HJ_TRY(launch_region_bits<8>(c, bits, (unsigned)nch, in, n, rg, chunk, 0, out, k0, k1, nullptr));
+        HJ_TRY(launch_region_bits<8>(c, bits, (unsigned)nch, in, n, rg, chunk, 0, out, k0, k1));
+    return HJ_OK;
+}
+
+uint64_t batch_chunk_rows(hj_ctx *c, uint64_t rows, int bits) {
+    // eight chunks per SM over all relations, at least 64 rows per digit (so that padding
+    // stays below a twentieth) and 2^14
+    const uint64_t n = rows / ((uint64_t)num_sms(c) * 8) + 1, lo = std::max<uint64_t>(1ull << 14, 64ull << bits);
+    return (std::max(n, lo) + 8191) / 8192 * 8192;
+}
+
+hj_status batch_partition(hj_ctx *c, int width, const BatchChunk *chunks, uint64_t nchunks, int max_bits, uint32_t *H,
+                          uint32_t *base, uint32_t *T, void *out, uint64_t *part_off) {
+    if (nchunks == 0) return HJ_OK;
+    BatchPadKeys pk;
+    pk.k1[0] = 0;
+    for (int b = 1; b <= 11; ++b) pk.k1[b] = pass_pad_key(width, 0, b);
+#define HJ_BP(WW)                                                                                                      \
+    do {                                                                                                               \
+        HJ_LAUNCH(c, "partition_hist", batch_hist_kernel<WW>, (unsigned)nchunks, kHistThreads, (size_t)4 << max_bits, chunks, \
+                  H, base, T);                                                                                         \
+        HJ_TRY(allow_max_smem(c, (const void *)batch_scatter_kernel<WW>));                                             \
+        HJ_LAUNCH(c, "partition_scatter", batch_scatter_kernel<WW>, (unsigned)nchunks, kRegionThreads, kRegionSmem,    \
+                  chunks, H, base, T, out, part_off, pk);                                                              \
+    } while (0)
+    if (width == 4) HJ_BP(4);
+    else HJ_BP(8);
+#undef HJ_BP
     return HJ_OK;
 }
 

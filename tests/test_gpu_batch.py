@@ -173,3 +173,29 @@ def test_batch_full_size_counts_and_sampled_pairs(hjm, ctx):
             assert np.array_equal(_sorted(got), oracle.sorted_pairs(*oracle.hash_join(r, s))), j
     finally:
         hjm.hj_results_free(ctx, outs, n)
+
+
+@pytest.mark.parametrize("width", [4, 8])
+def test_batch_partitions_every_fanout_at_once(hjm, ctx, width):
+    # joins on 2^1 .. 2^9 digits in one batch, at sizes around the steps of the fan-out, odd
+    # row counts, chunks of one tuple past a whole one, and relations of one tuple
+    step = 2048 if width == 4 else 1024
+    dt = np.uint32 if width == 4 else np.uint64
+    rng = np.random.default_rng(77 + width)
+    sizes = [(1, 1), (1, 50_001), (3, 2), (2 * step, 16_384), (2 * step + 1, 16_385), (4 * step, 40_961),
+             (16 * step + 1, 32_769), (100 * step - 1, 30_001), (260 * step + 5, 70_003)]
+    host, Rs, Ss = [], [], []
+    for nr, ns in sizes:
+        R = np.stack([rng.permutation(np.arange(1, nr + 1)).astype(dt), np.arange(nr, dtype=dt)], 1)
+        S = np.stack([rng.integers(1, 2 * nr + 1, ns).astype(dt), np.arange(ns, dtype=dt)], 1)
+        host.append((R, S))
+        for a, rels in ((R, Rs), (S, Ss)):
+            rels.append(torch.from_numpy(a.view(np.int32 if width == 4 else np.int64)).to(DEV))
+    res = hjm.hj_join_batch(ctx, Rs, Ss, checksum=True)
+    cnt = hjm.hj_join_batch(ctx, Rs, Ss, mode=hjm.HJ_COUNT_CHECKSUM)
+    for j, (R, S) in enumerate(host):
+        want = oracle.sorted_pairs(*oracle.hash_join(R, S))
+        assert (res[j].count, *res[j].checksum) == oracle.join_aggregate(R, S), j
+        assert (cnt[j].count, *cnt[j].checksum) == oracle.join_aggregate(R, S), j
+        assert np.array_equal(_sorted(res[j].pairs_numpy()), want), j
+        res[j].free()
