@@ -889,8 +889,8 @@ __global__ void __launch_bounds__(kTmaThreads, 1) scatter_tma_kernel(
 // pipe (a claim 3.7 and a slot store 6.2 cycles per warp, a flush about 5) and the two
 // barriers of a tile.  One tile in registers covers a third of the loads' latency:
 // the tile after it is asked into L2 (2^26 tuples at 2^11 digits 362 -> 282 us; three
-// tiles ahead 301).  Sectors written by a lane each, carried tuples moved to the front
-// and no L2 prefetch took 387 us, and 401 .. 430 us at 2^5 .. 2^8 digits (now 220).
+// tiles ahead 301), and its loads go out one vector at a time (269 us).  Sectors written by a lane each, carried tuples moved to the front
+// and no L2 prefetch took 387 us, and 401 .. 430 us at 2^5 .. 2^8 digits (now 208).
 constexpr int kRegionThreads = 1024;
 constexpr int kRegionVecs = 4;  // 16-byte vectors per thread per tile
 constexpr size_t kRegionSmem = 227u * 1024u - 1024u;
@@ -946,24 +946,16 @@ __device__ __forceinline__ void region_chunk(const RegionMem<W> &rm, uint32_t lp
     Slot *ring = rm.ring;
     uint32_t *word = rm.word, *nxt = rm.nxt, *tail = rm.tail;
     for (uint32_t d = threadIdx.x; d < P; d += NT) word[d] = 0;
-    // vector j of the tile [t0, lim) for this thread; a last vector holding one
+    // vector j of the tile from row t0 on for this thread; a last vector holding one
     // tuple of a 4-byte relation is read with an 8-byte load (nothing past the
     // array end)
-    auto load = [&](uint32_t t0, uint32_t lim, Vec *v) {
-        if (t0 + RS::T <= lim) {
-#pragma unroll
-            for (int j = 0; j < VPT; ++j) v[j] = ld_stream(vsrc + t0 / PV + (uint32_t)j * NT + threadIdx.x);
-            return;
-        }
-#pragma unroll
-        for (int j = 0; j < VPT; ++j) {
-            const uint32_t r0 = t0 + ((uint32_t)j * NT + threadIdx.x) * PV;
-            if (r0 + PV <= lim) v[j] = ld_stream(vsrc + r0 / PV);
-            else if (r0 < lim) {
-                if constexpr (W == 4) {
-                    const uint2 x = ((const uint2 *)vsrc)[r0];
-                    v[j] = make_uint4(x.x, x.y, 0u, 0u);
-                }
+    auto load = [&](uint32_t t0, int j, Vec &v) {
+        const uint32_t r0 = t0 + ((uint32_t)j * NT + threadIdx.x) * PV;
+        if (r0 + PV <= nrows) v = ld_stream(vsrc + r0 / PV);
+        else if (r0 < nrows) {
+            if constexpr (W == 4) {
+                const uint2 x = ((const uint2 *)vsrc)[r0];
+                v = make_uint4(x.x, x.y, 0u, 0u);
             }
         }
     };
@@ -976,11 +968,20 @@ __device__ __forceinline__ void region_chunk(const RegionMem<W> &rm, uint32_t lp
     auto tile_end = [&](uint32_t t0) { return t0 + RS::T < nrows ? t0 + RS::T : nrows; };
     Vec cur[VPT], nx[VPT];
     prefetch(RS::T);
-    if (nrows) load(0, tile_end(0), cur);
+#pragma unroll
+    for (int j = 0; j < VPT; ++j) load(0, j, cur[j]);
     __syncthreads();
     for (uint32_t t0 = 0, t1; t0 < nrows; t0 = t1) {
         t1 = tile_end(t0);
-        if (t1 < nrows) load(t1, tile_end(t1), nx);
+        // The next tile's loads go out one vector at a time for 4-byte tuples: what L1 has
+        // left beside the rings holds two of the four, and more hold up the shared-memory
+        // pipe.  (8-byte tuples, half as many to a tile, do not lean on that pipe: 2^26
+        // of them took 501 us spread and 492 at once.)
+        constexpr bool kSpread = W == 4;
+        load(t1, 0, nx[0]);
+        if (!kSpread)
+#pragma unroll
+            for (int j = 1; j < VPT; ++j) load(t1, j, nx[j]);
         prefetch(t0 + 2 * RS::T);
         const bool whole = t0 + RS::T <= nrows;
         // 1. insert, the claims of four tuples in flight together
@@ -1015,8 +1016,10 @@ __device__ __forceinline__ void region_chunk(const RegionMem<W> &rm, uint32_t lp
                 if (held < K) ring[s * PITCH + d[i]] = sl[i];
                 else outp[atomicSub(&tail[d[i]], 1u) - 1u] = sl[i];
             }
+            if (kSpread && j0 == 0) load(t1, 1, nx[1]);
         }
         __syncthreads();
+        if (kSpread) load(t1, 2, nx[2]);
         // 2. flush up to the last line boundary; with few digits, which hold many lines
         // each, several groups of LPD lanes share a digit
         const uint32_t NG = NT / LPD, q = threadIdx.x & (LPD - 1u), grp = threadIdx.x / LPD;
@@ -1046,6 +1049,7 @@ __device__ __forceinline__ void region_chunk(const RegionMem<W> &rm, uint32_t lp
                 word[d] = (held - w) | (h << 16);
                 nxt[d] = row + w;
             }
+            if (kSpread && r0 == 0) load(t1, 3, nx[3]);
         }
         __syncthreads();
 #pragma unroll
@@ -1400,7 +1404,7 @@ static hj_status launch_ring(hj_ctx *c, unsigned grid, const void *in, uint64_t 
 // Which padded-pass scatter runs: the region scatter, unless the context asks for the
 // ring (hj_debug_scatter) or limits the waits, which only the ring has
 // (hj_debug_wait_limit).  Region against ring, per launch: 2^26 uniform 4-byte tuples
-// at 2^9 / 2^10 / 2^11 digits 0.22 / 0.26 / 0.28 ms against 0.39 / 0.34 / 0.33, 2^24
+// at 2^9 / 2^10 / 2^11 digits 0.22 / 0.25 / 0.27 ms against 0.39 / 0.34 / 0.33, 2^24
 // 73 / 84 / 90 us against 119 / 109 / 110; 2^25 8-byte tuples 0.21 / 0.24 / 0.27 ms
 // against 0.32 / 0.31 / 0.32, 2^22 45 / 50 / 56 us against 69 / 61 / 64.
 static bool use_ring(const hj_ctx *c, int bits) {
