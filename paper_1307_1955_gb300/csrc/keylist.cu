@@ -13,9 +13,9 @@
 //   2. an exclusive scan of the counts gives each key the offset of its rid list;
 //   3. a second pass over R places every rid in its key's list (a per-key fill
 //      position claimed by atomicAdd; the order inside a list is free).
-// In steps 1 and 3 the lanes of a warp holding one key act as one, and keys that
-// fill several lanes are also gathered per CTA tile in shared memory: a heavy
-// hitter's count and fill position take one global atomic per tile.
+// In steps 1 and 3 a CTA keeps a short list of keys that it met several times in one
+// warp (heavy hitters), and the lanes of a warp that hold a listed key act as one: its
+// count takes one global atomic per CTA, its fill position one per tile.
 // A probe finds its key's one slot and emits the key's rid list with its own rid:
 // lists of fewer than 32 pairs flattened across the warp (pair p of their
 // concatenation written by lane p mod 32); a list of up to kCoopPairs by the
@@ -184,19 +184,17 @@ hj_status scan_entries(hj_ctx *c, Src src, Dst dst, uint64_t n, uint64_t *total_
 }
 
 // --------------------------------------------------------------- build
-// Lanes of a warp holding the same kept key act as one: the lowest takes the
-// group's count in one atomic (a heavy hitter has many copies in every warp, and
-// one atomic per copy on one address would serialise the build).
 __device__ __forceinline__ unsigned lanes_lt() { return (1u << (threadIdx.x & 31)) - 1u; }
 
 constexpr uint64_t kGuessWalk = 64;
-// Keys that fill several lanes of a warp group (the heavy hitters that make a
-// partition need a key-list table) are also gathered per tile of a CTA: up to
-// kHot of them in shared memory, each then taking one global atomic per tile
-// instead of one per warp group.
+// Heavy hitters a CTA lists: up to kHot keys that filled several lanes of a warp, found
+// in every kLookEvery-th of its tiles (comparing all lanes' keys costs 62 cycles per
+// warp, comparing with the listed ones a few).  Lanes of a warp that hold a listed key
+// add to its entry in shared memory together.
 constexpr int kHot = 8;
+constexpr uint32_t kLookEvery = 8;
 
-// Entry of key k among the tile's gathered keys (a free one taken), or -1.
+// Entry of key k among the listed keys (a free one taken), or -1.
 template <int W> __device__ __forceinline__ int hot_entry(typename Tup<W>::U *hk, typename Tup<W>::U k) {
     using U = typename Tup<W>::U;
 #pragma unroll 1
@@ -221,7 +219,8 @@ __device__ __forceinline__ unsigned kl_add(AggSlot<W> *slots, uint64_t cap, type
     const uint64_t walk = guess && cap > kGuessWalk ? kGuessWalk : cap;
     uint64_t b = bucket_of<W>(h, cap);
     for (uint64_t it = 0; it < walk; ++it) {
-        const U old = cas_key<W>((U *)&slots[b].key, Tup<W>::kAllOnes, k);
+        U old = *(volatile U *)&slots[b].key;
+        if (old == Tup<W>::kAllOnes) old = cas_key<W>((U *)&slots[b].key, Tup<W>::kAllOnes, k);
         if (old == Tup<W>::kAllOnes || old == k) {
             add_cnt(&slots[b].cnt, (decltype(slots[b].cnt))m);
             return old == Tup<W>::kAllOnes;
@@ -233,18 +232,42 @@ __device__ __forceinline__ unsigned kl_add(AggSlot<W> *slots, uint64_t cap, type
     return 0;
 }
 
+// The listed key that a lane holds (k, if `on`), or -1; *mask gets the lanes that hold
+// it.  All lanes call; entries fill in order, all ones mark the end.
+template <int W>
+__device__ __forceinline__ int listed_key(const typename Tup<W>::U *hk, typename Tup<W>::U k, bool on, unsigned *mask) {
+    using U = typename Tup<W>::U;
+    int at = -1;
+    unsigned left = __ballot_sync(0xffffffffu, on);
+#pragma unroll 1
+    for (int j = 0; j < kHot && left; ++j) {
+        // (lane 0's view, so that the warp leaves together: entries are being added)
+        const U h = __shfl_sync(0xffffffffu, ((const volatile U *)hk)[j], 0);
+        if (h == Tup<W>::kAllOnes) break;
+        const unsigned m = __ballot_sync(0xffffffffu, on && k == h);
+        if (on && k == h) {
+            at = j;
+            *mask = m;
+        }
+        left &= ~m;
+    }
+    return at;
+}
+
 // Step 1: every kept key in the table, its count added.  Each key inserted counts
 // in *nkeys; with a first table sized for fewer distinct keys than rows
-// (key_limit = half its slots) the CTAs stop once they pass the limit, walks end
-// after kGuessWalk slots (at load <= 1/2 a longer one gives the table up too),
-// and the host builds again at full size.
+// (key_limit = half its slots) the CTAs stop after the tile in which they pass the
+// limit, walks end after kGuessWalk slots (at load <= 1/2 a longer one gives the table
+// up too), and the host builds again at full size.  What bounds it: one pass over R
+// (4.2e6 rows of which all but 6e3 hold one key 107 us with every lane group looking at
+// *nkeys, matching all lanes and adding per tile).
 template <int W>
 __global__ void __launch_bounds__(256) kl_count(const void *R, uint64_t n, AggSlot<W> *slots, uint64_t cap,
                                                 TableSide *side, hj_counters *ctr, PartFilter pf,
                                                 unsigned long long *nkeys, uint64_t key_limit) {
     using U = typename Tup<W>::U;
     constexpr int PV = Tup<W>::kPerVec;
-    __shared__ U hk[kHot];        // the tile's gathered keys (all ones: free)
+    __shared__ U hk[kHot];        // listed keys (all ones: free)
     __shared__ unsigned hc[kHot];  // and their counts
     __shared__ int stop;
     const unsigned lane = threadIdx.x & 31;
@@ -257,7 +280,8 @@ __global__ void __launch_bounds__(256) kl_count(const void *R, uint64_t n, AggSl
     }
     if (threadIdx.x == 0) stop = 0;
     __syncthreads();
-    for (uint64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {  // block-uniform
+    uint32_t round = 0;
+    for (uint64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++round) {  // block-uniform
         const uint64_t v = tile * blockDim.x + threadIdx.x;
         U k[2] = {0, 0}, r[2] = {0, 0};
         if (v < nv) kl_load<W>(R, v, n, k, r);
@@ -265,15 +289,19 @@ __global__ void __launch_bounds__(256) kl_count(const void *R, uint64_t n, AggSl
 #pragma unroll
         for (int e = 0; e < PV; ++e) {
             const uint64_t h = key_hash<W>(k[e]);
-            const bool ok = v < nv && v * PV + e < n && pf.keep(h);
-            const unsigned g = __match_any_sync(0xffffffffu, k[e]) & __ballot_sync(0xffffffffu, ok);
-            if (!ok || (g & lanes_lt())) continue;  // the group's lowest lane counts for it
-            const unsigned m = __popc(g);
-            if (k[e] == Tup<W>::kAllOnes) {
-                atomicAdd(&side->agg_cnt, (unsigned long long)m);
-                continue;
+            const bool ok = v < nv && v * PV + e < n && pf.keep(h), ones = k[e] == Tup<W>::kAllOnes;
+            const unsigned om = __ballot_sync(0xffffffffu, ok && ones);
+            if (om && lane == (unsigned)(__ffs(om) - 1)) atomicAdd(&side->agg_cnt, (unsigned long long)__popc(om));
+            unsigned hm = 0;
+            const int at = listed_key<W>(hk, k[e], ok && !ones, &hm);
+            if (at >= 0 && !(hm & lanes_lt())) atomicAdd(&hc[at], (unsigned)__popc(hm));
+            const bool rest = ok && !ones && at < 0;
+            unsigned m = 1;  // tuples this lane counts
+            if (round % kLookEvery == 0) {
+                const unsigned g = __match_any_sync(0xffffffffu, k[e]) & __ballot_sync(0xffffffffu, rest);
+                m = rest && !(g & lanes_lt()) ? __popc(g) : 0;  // the group's lowest lane, for all
             }
-            if (guess && *(volatile unsigned long long *)nkeys > key_limit) continue;  // given up
+            if (!rest || !m) continue;
             if (m > 1) {
                 const int j = hot_entry<W>(hk, k[e]);
                 if (j >= 0) {
@@ -286,26 +314,23 @@ __global__ void __launch_bounds__(256) kl_count(const void *R, uint64_t n, AggSl
         if (guess) {  // (the warp is converged again here)
             const unsigned tot = __reduce_add_sync(0xffffffffu, fresh);
             if (lane == 0 && tot) atomicAdd(nkeys, (unsigned long long)tot);
+            if (threadIdx.x == 0) stop = *(volatile unsigned long long *)nkeys > key_limit;
+            __syncthreads();
+            if (stop) return;  // given up: the host builds again
+            __syncthreads();   // (read before the next tile sets it)
         }
-        __syncthreads();
-        if (threadIdx.x < kHot) {  // the gathered keys: one add each
-            const U hkey = hk[threadIdx.x];
-            if (hkey != Tup<W>::kAllOnes) {
-                if (kl_add<W>(slots, cap, hkey, key_hash<W>(hkey), hc[threadIdx.x], guess, nkeys, ctr) && guess)
-                    atomicAdd(nkeys, 1ull);
-                hk[threadIdx.x] = Tup<W>::kAllOnes;
-                hc[threadIdx.x] = 0;
-            }
-        }
-        if (threadIdx.x == 0) stop = guess && *(volatile unsigned long long *)nkeys > key_limit;
-        __syncthreads();
-        if (stop) break;
+    }
+    __syncthreads();
+    if (threadIdx.x < kHot) {  // the listed keys: one add each
+        const U hkey = hk[threadIdx.x];
+        if (hkey != Tup<W>::kAllOnes && hc[threadIdx.x])
+            if (kl_add<W>(slots, cap, hkey, key_hash<W>(hkey), hc[threadIdx.x], guess, nkeys, ctr) && guess)
+                atomicAdd(nkeys, 1ull);
     }
 }
 
-// Step 3: every kept R tuple's rid into its key's list: a warp group's places
-// [at, at + popc(g)) claimed by its leader on the key's fill position, a gathered
-// key's places claimed once per tile.
+// Step 3: every kept R tuple's rid into its key's list: places claimed on the key's
+// fill position, a listed key's once per tile.
 template <int W>
 __global__ void __launch_bounds__(256) kl_scatter(const void *R, uint64_t n, AggSlot<W> *slots, uint64_t cap,
                                                   TableSide *side, typename Tup<W>::U *rids, hj_counters *ctr,
@@ -314,7 +339,7 @@ __global__ void __launch_bounds__(256) kl_scatter(const void *R, uint64_t n, Agg
     constexpr int PV = Tup<W>::kPerVec;
     __shared__ U hk[kHot];
     __shared__ unsigned hc[kHot];
-    __shared__ unsigned long long hb[kHot];  // first place of a gathered key's tuples (~0: none)
+    __shared__ unsigned long long hb[kHot];  // first place of a listed key's tuples (~0: none)
     const unsigned lane = threadIdx.x & 31;
     const uint64_t nv = (n + PV - 1) / PV;
     const uint64_t tiles = (nv + blockDim.x - 1) / blockDim.x;
@@ -323,30 +348,38 @@ __global__ void __launch_bounds__(256) kl_scatter(const void *R, uint64_t n, Agg
         hc[threadIdx.x] = 0;
     }
     __syncthreads();
-    for (uint64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {  // block-uniform
+    uint32_t round = 0;
+    for (uint64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x, ++round) {  // block-uniform
         const uint64_t v = tile * blockDim.x + threadIdx.x;
         U k[2] = {0, 0}, r[2] = {0, 0};
         if (v < nv) kl_load<W>(R, v, n, k, r);
-        int hj[2] = {-1, -1};      // gathered entry of item e
+        int hj[2] = {-1, -1};      // listed entry of item e
         unsigned hr[2] = {0, 0};   // and its place among the entry's tuples
 #pragma unroll
         for (int e = 0; e < PV; ++e) {
             const uint64_t h = key_hash<W>(k[e]);
-            const bool ok = v < nv && v * PV + e < n && pf.keep(h);
-            const unsigned g = __match_any_sync(0xffffffffu, k[e]) & __ballot_sync(0xffffffffu, ok);
+            const bool ok = v < nv && v * PV + e < n && pf.keep(h), ones = k[e] == Tup<W>::kAllOnes;
+            // a listed key's lanes take their places together, the lowest for all
+            unsigned g = 0;
+            int j = listed_key<W>(hk, k[e], ok && !ones, &g);
+            const bool known = j >= 0;
+            if (!known) g = ok ? 1u << lane : 0u;
+            if (round % kLookEvery == 0) {
+                const unsigned same = __match_any_sync(0xffffffffu, k[e]) & __ballot_sync(0xffffffffu, ok && !known);
+                if (!known) g = ok ? same : 0u;
+            }
             const int leader = g ? __ffs(g) - 1 : 0;
             // the leader claims the group's places: [at, at + popc(g)) of the key's
             // list, or of the all-ones keys' list counted down from the array's end,
-            // or of the key's gathered tuples in this tile
+            // or of the key's listed tuples in this tile
             uint64_t at = 0;
             bool fail = false;
-            int j = -1;
             if (ok && lane == (unsigned)leader) {
                 const uint64_t m = __popc(g);
-                if (k[e] == Tup<W>::kAllOnes) {
+                if (ones) {
                     at = atomicAdd(&side->n_allones, (unsigned long long)m);
                 } else {
-                    if (m > 1) j = hot_entry<W>(hk, k[e]);
+                    if (!known && m > 1) j = hot_entry<W>(hk, k[e]);
                     if (j >= 0) {
                         at = atomicAdd(&hc[j], (unsigned)m);
                     } else {
@@ -371,16 +404,16 @@ __global__ void __launch_bounds__(256) kl_scatter(const void *R, uint64_t n, Agg
             if (j >= 0) {
                 hj[e] = j;
                 hr[e] = (unsigned)(at + rank);
-            } else if (k[e] == Tup<W>::kAllOnes) {
+            } else if (ones) {
                 rids[n - 1 - (at + rank)] = r[e];
             } else {
                 rids[at + rank] = r[e];
             }
         }
         __syncthreads();
-        if (threadIdx.x < kHot) {  // the gathered keys: their places in one claim each
+        if (threadIdx.x < kHot) {  // the listed keys: their places in one claim each
             const U hkey = hk[threadIdx.x];
-            if (hkey != Tup<W>::kAllOnes) {
+            if (hkey != Tup<W>::kAllOnes && hc[threadIdx.x]) {
                 const uint64_t b = kl_find<W>(slots, cap, hkey, key_hash<W>(hkey));
                 const unsigned m = hc[threadIdx.x];
                 if (b == cap) {
@@ -392,7 +425,6 @@ __global__ void __launch_bounds__(256) kl_scatter(const void *R, uint64_t n, Agg
                 } else {
                     hb[threadIdx.x] = slots[b].suma + atomicAdd(&slots[b].pad, (unsigned long long)m);
                 }
-                hk[threadIdx.x] = Tup<W>::kAllOnes;
                 hc[threadIdx.x] = 0;
             }
         }
