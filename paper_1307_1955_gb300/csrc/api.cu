@@ -387,8 +387,39 @@ hj_status probe_into(hj_ctx *c, const hj_table *t, const hj_rel *S, const hj_opt
     return HJ_OK;
 }
 
+// SHJ of a build side that fits shared memory: one launch, no table in global memory.
+// *done is false when a heavily repeated build key needs the key-list table.
+hj_status join_small(hj_ctx *c, const hj_rel *R, const hj_rel *S, const hj_opts &o, hj_result *res, bool *done) {
+    *done = false;
+    PairSink sink(c, R->width);
+    uint64_t cap = std::max<uint64_t>(o.out_capacity ? o.out_capacity : S->n, 1);
+    for (int attempt = 0; attempt < 2; ++attempt) {
+        HJ_TRY(sink.reset(cap));
+        HJ_TRY(zero_counters(c));
+        HJ_TRY(small_join(c, R->width, R->tuples, R->n, S->tuples, S->n, sink.pairs.p, sink.pcap, c->d_ctr));
+        HJ_TRY(read_counters(c));
+        if (c->h_ctr->status & kStatusLongRun) return HJ_OK;
+        if (c->h_ctr->count <= sink.pcap) break;
+        cap = c->h_ctr->count;  // more pairs than the capacity: again at the exact size
+        if (attempt == 1) return set_err(c, HJ_E_CUDA, "pair capacity still too small after resizing");
+    }
+    fill_result(c, res, R->width, HJ_ALGO_SHJ, 0, 0);
+    res->pairs = sink.pairs.release();
+    res->pairs_cap = sink.pcap;
+    *done = true;
+    return HJ_OK;
+}
+
 hj_status join_shj(hj_ctx *c, const hj_rel *R, const hj_rel *S, const hj_opts &o, hj_result *res) {
     TableGuard tg{c};
+    if (o.mode == HJ_MATERIALIZE && !wants_checksum(o) && R->n <= small_join_rows(R->width)) {
+        bool done = false;
+        HJ_TRY(join_small(c, R, S, o, res, &done));
+        if (done) return HJ_OK;
+        HJ_TRY(zero_counters(c));
+        HJ_TRY(keylist_build(c, R->width, R->tuples, R->n, PartFilter{0, 0, 0, 0}, &tg.t));
+        return probe_into(c, tg.t, S, o, res, true);
+    }
     HJ_TRY(table_create(c, R->width, is_agg(o.mode), R->n, &tg.t, true));
     HJ_TRY(table_build(c, tg.t, R->tuples, R->n, PartFilter{0, 0, 0, 0}));
     bool long_run = false;

@@ -34,6 +34,13 @@ hj_status table_build(hj_ctx *c, hj_table *t, const void *R, uint64_t n, PartFil
 hj_status table_probe(hj_ctx *c, const hj_table *t, const void *S, uint64_t n, void *pairs, uint64_t pcap,
                       int checksum, PartFilter pf, hj_counters *ctr);
 
+// Pairs of S with a build relation of at most small_join_rows(width) tuples, whose table
+// every CTA keeps in shared memory: exact claims of ctr->count, as table_probe; a
+// heavily repeated build key sets kStatusLongRun instead.
+uint64_t small_join_rows(int width);
+hj_status small_join(hj_ctx *c, int width, const void *R, uint64_t nr, const void *S, uint64_t ns, void *pairs,
+                     uint64_t pcap, hj_counters *ctr);
+
 // A partition pair for the shared-memory join: padded partitions (every row
 // range starts on a 32-byte sector, its row count is a multiple of the sector's
 // tuples), their partition index p under pass bits (b1, b2) -- rows hashing

@@ -1033,11 +1033,16 @@ template <int W, int NT> __device__ __forceinline__ bool keys_repeat(const SoaTa
 // the home bucket only if the bucket's last slot is taken AND more inserts tried it than
 // it has slots: such items are queued and their runs walked 32 at a time.  With UNIQ (no
 // key is twice in the table) a match ends the search; otherwise an item with several
-// matches in its home bucket has its whole run walked by the warp.
-template <int W, int U, bool UNIQ, bool FULL, class Sink>
+// matches in its home bucket has its whole run walked by the warp.  With MARK the marker
+// of empty slots may be a key: its build rids are the `side` list.
+template <int W> struct SideList {
+    const typename Tup<W>::U *rids = nullptr;
+    uint32_t n = 0;
+};
+template <int W, int U, bool UNIQ, bool FULL, bool MARK, class Sink>
 __device__ __forceinline__ void probe_group_smem(const SoaTab<W> &tab, const typename Tup<W>::Vec *x, const bool *in,
                                                  Sink &sink, unsigned lane, typename Tup<W>::U *wqk,
-                                                 typename Tup<W>::U *wqr, uint32_t &qn) {
+                                                 typename Tup<W>::U *wqr, uint32_t &qn, const SideList<W> &side) {
     using T = typename Tup<W>::U;
     constexpr int PV = Tup<W>::kPerVec, IT = U * PV;
     constexpr uint32_t G = SoaTab<W>::G;
@@ -1060,7 +1065,7 @@ __device__ __forceinline__ void probe_group_smem(const SoaTab<W> &tab, const typ
     bool found[IT], w[IT], several[IT], anyw = false, anys = false;
 #pragma unroll
     for (int i = 0; i < IT; ++i) {
-        const bool live = FULL || in[i / PV];
+        const bool live = (FULL || in[i]) && !(MARK && k[i] == tab.empty);
         uint32_t sl = home[i] * G + (G - 1), c = kb[i][G - 1] == k[i];
         bool f = kb[i][G - 1] == k[i];
 #pragma unroll
@@ -1091,6 +1096,21 @@ __device__ __forceinline__ void probe_group_smem(const SoaTab<W> &tab, const typ
             }
         }
     }
+    if (MARK && side.n) {
+#pragma unroll
+        for (int i = 0; i < IT; ++i) {
+            unsigned m = __ballot_sync(0xffffffffu, (FULL || in[i]) && k[i] == tab.empty);
+            while (m) {
+                const int L = __ffs(m) - 1;
+                m &= m - 1;
+                const T ss = __shfl_sync(0xffffffffu, r[i], L);
+                for (uint32_t j = 0; j < side.n; j += 32) {
+                    const bool has = j + lane < side.n;
+                    sink.append(has, has ? side.rids[j + lane] : T(0), ss);
+                }
+            }
+        }
+    }
     if (__any_sync(0xffffffffu, anyw)) {
 #pragma unroll
         for (int i = 0; i < IT; ++i) {
@@ -1117,10 +1137,12 @@ __device__ __forceinline__ void probe_group_smem(const SoaTab<W> &tab, const typ
 // of different keys, 3 % otherwise.  A join of 2^22 with 2^25 4-byte tuples of
 // different build keys issues 84e6 warp instructions; one vector per lane, with the
 // matches of a bucket counted and several bases per store, took 128e6.
-template <int W, int U, bool UNIQ, class Sink>
+template <int W, int U, bool UNIQ, bool MARK = false, class Sink>
 __device__ __forceinline__ void probe_smem(const SoaTab<W> &tab, const typename Tup<W>::Vec *Sv, uint32_t nsv,
                                            Sink &sink, unsigned warp, unsigned nwarps, unsigned lane,
-                                           typename Tup<W>::U *wqk, typename Tup<W>::U *wqr) {
+                                           typename Tup<W>::U *wqk, typename Tup<W>::U *wqr,
+                                           const SideList<W> &side = SideList<W>()) {
+    constexpr int PV = Tup<W>::kPerVec;
     using Vec = typename Tup<W>::Vec;
     const uint32_t gstride = nwarps * 32u * U, whole = nsv / (32u * U) * (32u * U);
     uint32_t g = warp * 32u * U, qn = 0;
@@ -1138,18 +1160,20 @@ __device__ __forceinline__ void probe_smem(const SoaTab<W> &tab, const typename 
         if (g + gstride < whole)
 #pragma unroll
             for (int u = 0; u < U; ++u) nxt[u] = ld_stream(Sv + g + gstride + u * 32u + lane);
-        probe_group_smem<W, U, UNIQ, true>(tab, cur, nullptr, sink, lane, wqk, wqr, qn);
+        probe_group_smem<W, U, UNIQ, true, MARK>(tab, cur, nullptr, sink, lane, wqk, wqr, qn, side);
     }
     if (g == whole && whole < nsv) {  // the slice's last, partial group, in this warp's turn
         Vec cur[U];
-        bool in[U];
+        bool in[U * PV];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            in[u] = g + u * 32u + lane < nsv;
-            if (in[u]) cur[u] = ld_stream(Sv + g + u * 32u + lane);
+            const bool on = g + u * 32u + lane < nsv;
+            if (on) cur[u] = ld_stream(Sv + g + u * 32u + lane);
             else cur[u] = Vec{};
+#pragma unroll
+            for (int e = 0; e < PV; ++e) in[u * PV + e] = on;
         }
-        probe_group_smem<W, U, UNIQ, false>(tab, cur, in, sink, lane, wqk, wqr, qn);
+        probe_group_smem<W, U, UNIQ, false, MARK>(tab, cur, in, sink, lane, wqk, wqr, qn, side);
     }
     if (qn) {
         __syncwarp();
@@ -1627,6 +1651,188 @@ __global__ void __launch_bounds__(NT, join_ctas(NT)) partition_join_kernel(
         __syncthreads();  // every warp is done with this table and has the next task's record
     }
     if constexpr (!AGG) sink.finish();
+}
+
+// ========================================================= small build sides
+//
+// A build relation that fits shared memory whole needs neither a table in global
+// memory nor partitions: every CTA builds its own table of all of R (its rows come from
+// L2 after the first CTA) and probes its share of S, in one launch instead of three.  What
+// bounds it is the build's latency, then a probe's shared-memory work instead of its L2
+// sectors: 4097 x 10007 tuples 39.4 -> 32.8 us, 2500 x 2^23 111 -> 56 us.  All ones mark
+// empty slots; R's tuples of that key, which no slot can hold, go to a short list.
+constexpr uint32_t kSideRids = 64;
+template <int W, int NT>
+__global__ void __launch_bounds__(NT, join_ctas(NT)) small_join_kernel(const void *R, uint32_t nr, const void *S,
+                                                                       uint64_t ns, uint64_t slice, uint32_t cap,
+                                                                       void *pairs, uint64_t pcap, hj_counters *ctr,
+                                                                       uint32_t stage_at, uint32_t stage_bytes) {
+    using T = typename Tup<W>::U;
+    using Vec = typename Tup<W>::Vec;
+    constexpr int PV = Tup<W>::kPerVec;
+    constexpr uint32_t G = SoaTab<W>::G;
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ JoinSlot s_slot;
+    __shared__ T s_side[kSideRids];
+    __shared__ uint32_t s_nside;
+    __shared__ int s_full;
+    const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t nrv = nr / PV;  // whole vectors
+    const T ones = Tup<W>::kAllOnes;
+    uint32_t *info = (uint32_t *)(smem + (size_t)cap * 2 * W);
+    const SoaTab<W> tab{cap / G, ones, (const uint16_t *)info, (const T *)smem, (const T *)smem + cap};
+    constexpr int RB = 2;
+    Vec rx[RB];
+    auto load_r = [&](uint32_t v0) {
+#pragma unroll
+        for (int u = 0; u < RB; ++u) {
+            const uint32_t v = v0 + u * NT;
+            if (v < nrv) rx[u] = ld_stream((const Vec *)R + v);
+            else if (W == 4 && v * PV < nr) {
+                if constexpr (W == 4) {
+                    const uint2 y = ((const uint2 *)R)[2 * v];
+                    rx[u] = make_uint4(y.x, y.y, 0u, 0u);
+                }
+            }
+        }
+    };
+    load_r(threadIdx.x);
+    // the build rows that follow and the first probe rows into L2 meanwhile
+    for (uint32_t i = RB * NT / 8 + threadIdx.x; i * 8u < nrv; i += NT) prefetch_l2((const Vec *)R + i * 8u);
+    const uint64_t nsv = ns / PV, s0 = min(blockIdx.x * slice, nsv), s1 = min(s0 + slice, nsv);
+    const Vec *Sv = (const Vec *)S + s0;
+    for (uint32_t i = threadIdx.x; i < kAheadVecs / 8 && s0 + i * 8u < s1; i += NT) prefetch_l2(Sv + i * 8u);
+    const uint4 e4 = make_uint4(~0u, ~0u, ~0u, ~0u);
+    for (uint32_t i = threadIdx.x; i < cap * W / 16; i += NT) ((uint4 *)smem)[i] = e4;
+    for (uint32_t i = threadIdx.x; i < cap / G / 2; i += NT) info[i] = 0;
+    if (threadIdx.x == 0) {
+        s_full = 0;
+        s_nside = 0;
+        s_slot = JoinSlot{pairs, pcap, ctr, 0};
+    }
+    __syncthreads();
+    T *kv = (T *)smem;
+    const uint32_t lim = min(tab.nb, kMaxSmemWalk);
+    auto tried = [&](uint32_t b) -> uint32_t {
+        const uint32_t sh = (b & 1u) * 16u;
+        return (atomicAdd(&info[b >> 1], 1u << sh) >> sh) & 0xFFFFu;
+    };
+    for (uint32_t v0 = threadIdx.x; v0 * PV < nr; v0 += RB * NT) {
+        if (v0 != threadIdx.x) load_r(v0);
+        T k[RB * PV], r[RB * PV];
+        uint32_t bkt[RB * PV], q[RB * PV];
+        bool in[RB * PV];
+#pragma unroll
+        for (int i = 0; i < RB * PV; ++i) {
+            const Vec &x = rx[i / PV];
+            if constexpr (W == 4) {
+                k[i] = i % 2 ? x.z : x.x;
+                r[i] = i % 2 ? x.w : x.y;
+            } else {
+                k[i] = x.x;
+                r[i] = x.y;
+            }
+            in[i] = (v0 + (i / PV) * NT) * PV + i % PV < nr;
+            if (in[i] && k[i] == ones) {
+                const uint32_t at = atomicAdd(&s_nside, 1u);
+                if (at < kSideRids) s_side[at] = r[i];
+                else s_full = 1;
+                in[i] = false;
+            }
+            bkt[i] = part_bucket<W>(k[i], tab.nb);
+            q[i] = in[i] ? tried(bkt[i]) : 0u;
+        }
+#pragma unroll
+        for (int i = 0; i < RB * PV; ++i) {
+            if (!in[i]) continue;
+            for (uint32_t it = 1; q[i] >= G && it < lim; ++it) {
+                bkt[i] = bkt[i] + 1 == tab.nb ? 0 : bkt[i] + 1;
+                q[i] = tried(bkt[i]);
+            }
+            if (q[i] < G) {
+                T *slot = &kv[bkt[i] * G + q[i]];
+                slot[0] = k[i];
+                slot[cap] = r[i];
+            } else {
+                s_full = 1;  // a heavily repeated key
+            }
+        }
+    }
+    __syncthreads();
+    if (s_full) {  // (the same in every CTA)
+        if (threadIdx.x == 0) atomicOr(&ctr->status, (unsigned long long)kStatusLongRun);
+        return;
+    }
+    const SideList<W> side{s_side, s_nside};
+    const bool unique = s1 - s0 >= 2 * (uint64_t)nrv && !__syncthreads_or(keys_repeat<W, NT>(tab));
+    WarpStageSink<W> sink;
+    sink.stage = (typename WarpStageSink<W>::P *)(smem + stage_at + warp * stage_bytes);
+    sink.scap = stage_bytes / (2 * W);
+    sink.slots = &s_slot;
+    sink.begin_task(0);
+    T *wq = (T *)(smem + walkq_offset(cap, 2 * W, W, false)) + (size_t)warp * 2 * kWalkQ;
+    // (slices are below 2^32 vectors: a relation is)
+    if (unique)
+        probe_smem<W, 2, true, true>(tab, Sv, (uint32_t)(s1 - s0), sink, warp, NT / 32, lane, wq, wq + kWalkQ, side);
+    else
+        probe_smem<W, 2, false, true>(tab, Sv, (uint32_t)(s1 - s0), sink, warp, NT / 32, lane, wq, wq + kWalkQ, side);
+    if constexpr (W == 4) {  // an odd last tuple
+        if (ns % 2 && blockIdx.x + 1 == gridDim.x && warp == 0) {
+            Vec x[1];
+            const uint2 y = ((const uint2 *)S)[ns - 1];
+            x[0] = make_uint4(y.x, y.y, 0u, 0u);
+            const bool in[2] = {lane == 0, false};
+            uint32_t qn = 0;
+            probe_group_smem<W, 1, false, false, true>(tab, x, in, sink, lane, wq, wq + kWalkQ, qn, side);
+            if (qn) {
+                __syncwarp();
+                drain_walks<W>(tab, wq, wq + kWalkQ, qn, sink);
+            }
+        }
+    }
+    sink.finish();
+}
+
+// (what a table of two and a half slots per tuple holds in a CTA's shared memory)
+uint64_t small_join_rows(int width) { return width == 4 ? 8192 : 4096; }
+
+hj_status small_join(hj_ctx *c, int width, const void *R, uint64_t nr, const void *S, uint64_t ns, void *pairs,
+                     uint64_t pcap, hj_counters *ctr) {
+    if (!nr || !ns) return HJ_OK;
+    const uint64_t pv = width == 4 ? 2 : 1;
+    auto slots_for = [&](int nt, uint64_t stage) {
+        const uint64_t total = (join_ctas(nt) == 2 ? (112ull << 10) : (222ull << 10)) - 32,
+                       fixed = (uint64_t)(nt / 32) * (kWalkQ * 2 * width + stage);
+        return (total - fixed) * 8 / (17 * (uint64_t)width) / 128 * 128;
+    };
+    // Three slots per tuple, two and a half where that keeps two CTAs on an SM; a probe side
+    // that one wide CTA per SM covers is bound by the time to build the table, which
+    // twice the threads halve.
+    const uint64_t nsv = ns / pv, sms = (uint64_t)num_sms(c);
+    const uint64_t want = std::max<uint64_t>((3 * nr + 127) / 128 * 128, 128);
+    const bool two = nsv > sms * 1280 && nr * 5 / 2 <= slots_for(320, 2048);
+    const int nt = two ? 320 : 640;
+    const uint64_t stage = want <= slots_for(nt, 4096) ? 4096 : 2048, cap = std::min(want, slots_for(nt, stage));
+    const uint64_t queue_at = walkq_offset((uint32_t)cap, (uint32_t)(2 * width), width, false),
+                   stage_at = queue_at + (uint64_t)(nt / 32) * kWalkQ * 2 * width,
+                   smem = stage_at + (uint64_t)(nt / 32) * stage;
+    const uint64_t grid = std::max<uint64_t>(std::min<uint64_t>(sms * join_ctas(nt), (nsv + 2 * nt - 1) / (2 * nt)), 1);
+    const uint64_t slice = std::max<uint64_t>(((nsv + grid - 1) / grid + 63) / 64 * 64, 64);
+    const unsigned g = (unsigned)std::max<uint64_t>((nsv + slice - 1) / slice, 1);
+#define HJ_SM(WW, NT)                                                                                              \
+    do {                                                                                                           \
+        auto kern = small_join_kernel<WW, NT>;                                                                     \
+        HJ_TRY(allow_max_smem(c, (const void *)kern));                                                             \
+        HJ_LAUNCH(c, "small_join", kern, g, NT, smem, R, (uint32_t)nr, S, ns, slice, (uint32_t)cap, pairs, pcap, ctr, \
+                  (uint32_t)stage_at, (uint32_t)stage);                                                            \
+    } while (0)
+    if (width == 4) {
+        if (two) HJ_SM(4, 320); else HJ_SM(4, 640);
+    } else {
+        if (two) HJ_SM(8, 320); else HJ_SM(8, 640);
+    }
+#undef HJ_SM
+    return HJ_OK;
 }
 
 // Tasks of one join partitioned into NP padded partitions: task p covers rows
