@@ -15,8 +15,9 @@
 //   * a GPU overlaps the two within a kernel, so a step costs max(C_i, M_i), plus
 //     a launch latency per kernel;
 //   * the SHJ table's random accesses cost nothing extra while the table stays in
-//     L2 and one sector per access from HBM once it does not (the "leap" of the
-//     paper's end-to-end results once the table outgrows the cache, Sec. 5.5).
+//     L2, and one sector from HBM for the share of them that falls outside it (the
+//     "leap" of the paper's end-to-end results once the table outgrows the cache,
+//     Sec. 5.5); a build side that fits shared memory whole has no such table.
 // hj_tune then times the model's best few plans on the caller's relations and
 // caches the fastest for the relations' size class on the context; hj_join with
 // HJ_ALGO_AUTO uses a cached plan when one exists, else the model's choice.
@@ -32,27 +33,34 @@ namespace hj {
 namespace {
 
 // Effective thread instructions per item of each kernel at the sustained issue
-// rate below: ncu's smsp__inst_executed x 32 / items, scaled so that the model's
-// time equals the kernel's measured time on GB300 (4-byte tuples: the 2^24 x 2^28
-// join at 11 radix bits -- scatter 1.302 ms, join 1.019 ms -- and the build-heavy
-// 2^24 x 2^24 join -- join 0.229 ms, which with the first fixes the probe and build
-// costs --, 12 bits in one and two passes, and SHJ at 2^20 and 2^24 build tuples).
+// rate below, set so that the model's time equals the kernel's measured time on GB300
+// (4-byte tuples; where it says so, 8-byte tuples take twice as many): scatters of 2^26
+// (2^25) tuples, the joins of 2^24 x 2^24 and 2^24 x 2^28 at 11 radix bits (u64 3e6 x 2e7
+// at 10), SHJ of 2^18 .. 2^24 build tuples with 1, 8 and 64 times as many.
 // hj_tune measures the real thing on the caller's relations.
-constexpr double kIptHist = 22.0;            // per input tuple (bandwidth-bound)
-constexpr double kIptScatterRing = 101.0;    // per input tuple, ring scatter (2^10 and 2^11 digits)
-constexpr double kIptScatterRegion = 131.0;  // per input tuple, region scatter at 2^8 and 2^9 digits
-constexpr double kIptScatterRegionLow = 115.0;  // per input tuple, region scatter at <= 2^7 digits (measured per pass of 6 + 6 bits)
-constexpr double kIptScatterWide = 293.0;    // per input tuple, fan-out 2^12
-constexpr double kIptJoinProbe = 70.0;       // per S tuple, shared-memory table
-constexpr double kIptJoinBuild = 232.0;      // per R tuple, shared-memory table (latency-bound build)
-constexpr double kIptShjBuild = 40.0;     // per R tuple, global table
-constexpr double kIptShjProbe = 60.0;     // per S tuple, global table
-constexpr double kIssueFraction = 0.55;   // sustained share of the issue slots
-constexpr double kCopyFraction = 0.83;    // share of nominal HBM bandwidth a copy reaches
-constexpr double kRandomFraction = 0.2;   // share for 32-byte random sectors (table probes)
-constexpr double kLaunchS = 4e-6;         // per kernel launch
-constexpr double kShjFixedS = 55e-6;      // per SHJ call: table fill, allocations, one host synchronisation
-constexpr double kPhjFixedS = 50e-6;      // per PHJ call: allocations, launch gaps, one host synchronisation
+constexpr double kIptHist = 22.0;          // per input tuple (bandwidth-bound)
+constexpr double kIptScatter = 66.0;       // per input tuple, at most 2^9 digits (x 2 for 8 bytes)
+constexpr double kIptScatter10 = 80.0;     // 2^10 digits (x 2)
+constexpr double kIptScatter11 = 87.0;     // 2^11 digits (x 2)
+constexpr double kIptScatterNext = 35.0;   // added by a second pass (many segments, launches)
+constexpr double kIptScatterWide = 266.0;  // per input tuple, fan-out 2^12
+constexpr double kIptJoinProbe = 55.0;     // per S tuple, shared-memory table (x 2)
+constexpr double kIptJoinBuild = 184.0;    // per R tuple, shared-memory table (x 2)
+constexpr double kIptShjBuild = 240.0;     // per R tuple, global table in L2
+constexpr double kIptShjBuildAgg4 = 480.0;   // aggregate table (three atomics per tuple)
+constexpr double kIptShjBuildAgg8 = 1400.0;
+constexpr double kIptShjProbe4 = 140.0;    // per S tuple, global table in L2
+constexpr double kIptShjProbe8 = 172.0;    // 8-byte tuples
+constexpr double kIptShjAgg8 = 270.0;      // 8-byte tuples, aggregate table (32-byte slots)
+constexpr double kIptSmallProbe = 64.0;    // per S tuple, whole build side in shared memory (x 1.6)
+constexpr double kIssueFraction = 0.55;    // sustained share of the issue slots
+constexpr double kCopyFraction = 0.83;     // share of nominal HBM bandwidth a copy reaches
+constexpr double kRandomFraction = 0.2;    // share for 32-byte random sectors (table probes)
+constexpr double kL2Table = 0.75;          // share of L2 that a table may take before probes miss
+constexpr double kLaunchS = 4e-6;          // per kernel launch
+constexpr double kSmallFixedS = 32e-6;     // per SHJ call with the build side in shared memory
+constexpr double kShjFixedS = 35e-6;       // per SHJ call: allocations, one host synchronisation
+constexpr double kPhjFixedS = 50e-6;       // per PHJ call: allocations, launch gaps, one host synchronisation
 
 }  // namespace
 
@@ -89,30 +97,38 @@ double predict_seconds(const CostModel &m, int width, bool agg, bool mat, uint64
     const double t = 2.0 * width, o = 2.0 * width, ir = issue_rate(m), b = bw(m);
     const double n = (double)nR + (double)nS, M = mat ? (double)nS : 0.0;  // one match per probe tuple
     double s[4] = {0, 0, 0, 0};  // hist, scatter, join / build, probe
-    if (algo == HJ_ALGO_SHJ) {
-        const double cap = std::exp2(std::ceil(std::log2(2.0 * nR + 1.0)));
-        const double slot = agg ? (width == 4 ? 16.0 : 32.0) : t;
-        const bool in_l2 = cap * slot <= 0.5 * m.l2_bytes;
+    if (algo == HJ_ALGO_SHJ && mat && nR <= small_join_rows(width)) {
+        s[3] = std::max((t * nS + o * M) / b, nS * kIptSmallProbe * (width == 4 ? 1.0 : 1.6) / ir) + kSmallFixedS;
+    } else if (algo == HJ_ALGO_SHJ) {
+        // the table: a power of two at least twice R, or (pairs, up to twice L2) four
+        // slots per tuple; probes of what does not stay in L2 read a sector from HBM
+        const double slot = agg ? (width == 4 ? 16.0 : 32.0) : t, four = 4.0 * nR * slot;
+        const double table = !agg && four <= 256.0 * (1 << 20) ? four
+                                                               : std::exp2(std::ceil(std::log2(2.0 * nR + 1.0))) * slot;
+        const double miss = std::max(0.0, 1.0 - kL2Table * m.l2_bytes / std::max(table, 1.0));
         const double rnd = b * kRandomFraction;
-        s[2] = std::max(t * nR / b + cap * slot / b + (in_l2 ? 0.0 : 64.0 * nR / rnd), nR * kIptShjBuild / ir);
-        s[3] = std::max((t * nS + o * M) / b + (in_l2 ? 0.0 : 32.0 * nS / rnd), nS * kIptShjProbe / ir);
+        const double probe = width == 4 ? kIptShjProbe4 : agg ? kIptShjAgg8 : kIptShjProbe8;
+        const double build = !agg ? kIptShjBuild : width == 4 ? kIptShjBuildAgg4 : kIptShjBuildAgg8;
+        s[2] = std::max(t * nR / b, nR * build / ir) + table / b + miss * 64.0 * nR / rnd;
+        s[3] = std::max((t * nS + o * M) / b, nS * probe / ir) + miss * 32.0 * nS / rnd;
         s[3] += 5 * kLaunchS + kShjFixedS;
     } else {
         const int b1 = passes == 2 ? bits - bits / 2 : bits, b2 = passes == 2 ? bits / 2 : 0;
+        const double wide = width == 4 ? 1.0 : 2.0;
         for (int p = 0; p < passes; ++p) {
             const int bp = p == 0 ? b1 : b2;
-            const double ipt = bp >= 10 && bp <= 11 ? kIptScatterRing
-                               : bp <= 7               ? kIptScatterRegionLow
-                               : bp <= 9               ? kIptScatterRegion
-                                                       : kIptScatterWide;
+            const double ipt = bp <= 9    ? kIptScatter * wide
+                               : bp == 10 ? kIptScatter10 * wide
+                               : bp == 11 ? kIptScatter11 * wide
+                                          : kIptScatterWide;
             // a first pass at <= 2^11 digits is two launches per relation (histogram
             // and scatter place the runs themselves), any other pass eight
             s[0] += std::max(t * n / b, n * kIptHist / ir) + (p == 0 && bp <= 11 ? 2 * 2 : 2 * 8) * kLaunchS;
-            s[1] += std::max(2.0 * t * n / b, n * ipt / ir);
+            s[1] += std::max(2.0 * t * n / b, n * (ipt + (p ? kIptScatterNext * wide : 0.0)) / ir);
         }
         // fewer partition pairs than join CTAs leave SMs idle
         const double busy = std::min(1.0, std::exp2(bits) / (2.0 * m.sms));
-        s[2] = std::max((t * n + o * M) / b, (nS * kIptJoinProbe + nR * kIptJoinBuild) / ir) / busy + 6 * kLaunchS +
+        s[2] = std::max((t * n + o * M) / b, (nS * kIptJoinProbe + nR * kIptJoinBuild) * wide / ir) / busy + 6 * kLaunchS +
                kPhjFixedS;
         // the (chunk, digit) count matrix: written, scanned and read once per pass
         s[0] += passes * 24.0 * m.sms * std::exp2(std::max(b1, b2)) / b;
