@@ -288,7 +288,7 @@ hj_status partition_rel(hj_ctx *c, const hj_rel *in, int b1, int b2, int pad, De
     HJ_TRY(A.alloc(rows1 * tb + 64));
     HJ_TRY(off1.alloc(((1ull << b1) + 1) * 8));
     if (pad && b1 <= 11) {  // the first pass is one segment: the fused form
-        HJ_TRY(partition_pass1(c, in->width, in->tuples, n, b1, A.p, off1.as<uint64_t>()));
+        HJ_TRY(partition_pass1(c, in->width, b1, Pass1{in->tuples, n, A.p, off1.as<uint64_t>()}));
     } else {
         HJ_TRY(device_pair(c, 0ull, n, seg));
         HJ_TRY(partition_pass(c, in->width, in->tuples, n, seg.as<uint64_t>(), 1, 0, b1, A.p, off1.as<uint64_t>(),
@@ -314,6 +314,27 @@ hj_status partition_rel(hj_ctx *c, const hj_rel *in, int b1, int b2, int pad, De
     offsets.p = off2.release();
     *rows = rows2;
     return HJ_OK;
+}
+
+// Both relations of a join; in one pass at most 2^11 digits wide, by the same launches
+// (unless the context has a memory budget: one relation's scratch at a time then).
+hj_status partition_both(hj_ctx *c, const hj_rel *R, const hj_rel *S, int b1, int b2, DevBuf &Rp, DevBuf &roff,
+                         uint64_t *r_rows, DevBuf &Sp, DevBuf &soff, uint64_t *s_rows) {
+    const int W = R->width;
+    const uint64_t rr = partition_out_rows(c, W, R->n, 1, b1, 1), sr = partition_out_rows(c, W, S->n, 1, b1, 1);
+    if (b2 || b1 > 11 || c->budget || rr >= 0xFFFFFFFFull || sr >= 0xFFFFFFFFull) {
+        HJ_TRY(partition_rel(c, R, b1, b2, 1, Rp, roff, r_rows));
+        return partition_rel(c, S, b1, b2, 1, Sp, soff, s_rows);
+    }
+    const uint64_t tb = tuple_bytes(W), ob = ((1ull << b1) + 1) * 8;
+    HJ_TRY(Rp.alloc(rr * tb + 64));
+    HJ_TRY(roff.alloc(ob));
+    HJ_TRY(Sp.alloc(sr * tb + 64));
+    HJ_TRY(soff.alloc(ob));
+    *r_rows = rr;
+    *s_rows = sr;
+    return partition_pass1(c, W, b1, Pass1{R->tuples, R->n, Rp.p, roff.as<uint64_t>()},
+                           Pass1{S->tuples, S->n, Sp.p, soff.as<uint64_t>()});
 }
 
 void fill_result(hj_ctx *c, hj_result *res, int width, int algo, int bits, int passes) {
@@ -496,8 +517,7 @@ hj_status join_phj(hj_ctx *c, const hj_rel *R, const hj_rel *S, const hj_opts &o
     DevBuf Rp(c), Sp(c), roff(c), soff(c), oversize(c), tasks(c), slot(c);
     PairSink sink(c, R->width);
     uint64_t r_rows = 0, s_rows = 0;
-    HJ_TRY(partition_rel(c, R, b1, b2, 1, Rp, roff, &r_rows));
-    HJ_TRY(partition_rel(c, S, b1, b2, 1, Sp, soff, &s_rows));
+    HJ_TRY(partition_both(c, R, S, b1, b2, Rp, roff, &r_rows, Sp, soff, &s_rows));
     const uint64_t tail = tail_split_from(c, R->width, is_agg(o.mode), NP, NP ? (R->n + NP - 1) / NP : 0);
     const uint64_t slice = task_slice_rows(R->width, S->n, NP),
                    ntasks = max_tasks(NP, s_rows, slice) + (NP - tail);

@@ -151,9 +151,15 @@ hj_status fallback_reprobe(hj_ctx *c, bool chk, const FallbackRedo &redo, const 
 // and segment s of the output starts where the padded segments before it end.
 hj_status partition_pass(hj_ctx *c, int width, const void *in, uint64_t n_total, const uint64_t *seg_off,
                          uint64_t nseg, int shift, int bits, void *out, uint64_t *part_off, int pad);
-// One padded pass over a single segment of n rows at 2^bits <= 2^11 digits:
-// partition_pass's output with two launches (histogram, scatter).
-hj_status partition_pass1(hj_ctx *c, int width, const void *in, uint64_t n, int bits, void *out, uint64_t *part_off);
+// One padded pass over a single segment at 2^bits <= 2^11 digits, of one relation or of
+// two at once (y empty): partition_pass's output with two launches (histogram, scatter).
+struct Pass1 {
+    const void *in = nullptr;
+    uint64_t n = 0;
+    void *out = nullptr;
+    uint64_t *part_off = nullptr;
+};
+hj_status partition_pass1(hj_ctx *c, int width, int bits, const Pass1 &x, const Pass1 &y = Pass1());
 // Padded passes of many relations at once, each on its own bits <= 2^11 digits: chunk
 // by chunk (device array), relation by relation ranges of `out`.  H and base hold
 // 2^bits words per chunk, T 2^bits + 1 per relation (zero beforehand), part_off

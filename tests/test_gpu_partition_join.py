@@ -90,3 +90,13 @@ def test_many_tasks_and_a_buffer_that_ends_inside_a_chunk(hjm, ctx, cap):
     r = _rel(rng.permutation(np.arange(1, 30_001)), 4)
     s = _rel(rng.integers(1, 45_001, 90_003), 4)
     _check(hjm, ctx, r, s, radix_bits=11, out_capacity=cap)
+
+
+@pytest.mark.parametrize("nr,ns", [(50_001, 3), (3, 50_001), (70_001, 70_000), (100, 0), (0, 100), (1, 1)])
+@pytest.mark.parametrize("width,bits", [(4, 3), (4, 11), (8, 10)])
+def test_both_relations_in_one_pass(hjm, ctx, width, bits, nr, ns):
+    # one histogram and one scatter launch take the chunks of both, the larger first
+    rng = np.random.default_rng(nr + ns)
+    r = _rel(rng.permutation(np.arange(1, nr + 1)), width)
+    s = _rel(rng.integers(1, 2 * nr + 2, ns), width)
+    _check(hjm, ctx, r, s, radix_bits=bits)
