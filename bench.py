@@ -683,7 +683,7 @@ def batch_cpu_sample(Rs, Ss, target_s: float):
 
 def run_batch(args, wl, ws, rank, local):
     """Config of many uneven joins: hj_join_batch (one persistent join launch per wave,
-    CUDA graph) against one hj_join call per join, on the same resident inputs."""
+    four launches) against one hj_join call per join, on the same resident inputs."""
     import torch
     import torch.distributed as dist
 
