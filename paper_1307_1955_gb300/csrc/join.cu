@@ -1364,7 +1364,7 @@ __global__ void __launch_bounds__(NT, join_ctas(NT)) partition_join_kernel(
                 // about three slots per build row (load factor 1/3), whole buckets
                 const uint64_t want = (3 * nr + 127) / 128 * 128;
                 cap = want < cap_max ? (uint32_t)want : cap_max;
-                if (nr >= cap - cap / 4) {  // load factor above 3/4: leave to the fallback
+                if (nr >= cap - cap / 5) {  // load factor above 4/5: leave to the fallback
                     if (threadIdx.x == 0) oversize[atomicAdd(&work->n_oversize, 1ull)] = (uint32_t)ti;
                     work_p = false;
                 }
@@ -1925,11 +1925,14 @@ uint64_t empty_key2(int width, int b1, int b2) {
 }
 
 // Join launch shape: two CTAs per SM with tables up to 100 KiB, or one of twice the
-// threads with up to 200 KiB when the expected build partition needs the room (load
-// factor about 1/3 either way).  The aggregate join runs 1024 threads per SM, the pair
-// join 640: its probe loop holds four tuples' buckets and needs 96 registers (with 64,
-// 1024 threads spill into an L1 that the tables leave no room: 2^24 x 2^28 1257 us
-// against 828, 896 threads 1181, 768 threads 1072, 576 threads 881).
+// threads with up to 209 KiB (aggregates: 200 KiB) when the expected build partition needs
+// the room (load factor about 1/3 either way).  The buckets' counts are part of the 209 KiB:
+// 25088 4-byte slots, so that partitions of 18e3 build rows keep off the fallback (2^9
+// partitions of 17800 / 18300 / 19000 rows, |S| = 2 |R|: 657 / 747 / 860 us; with 200 KiB
+// and a load of at most 3/4 1762 / 4080 / 4220 us).  The aggregate join runs 1024 threads
+// per SM, the pair join 640: its probe loop holds four tuples' buckets and needs 96
+// registers (with 64, 1024 threads spill into an L1 that the tables leave no room: 2^24 x
+// 2^28 1257 us against 828, 896 threads 1181, 768 threads 1072, 576 threads 881).
 struct JoinCfg {
     int nt;
     uint64_t smem_limit;
@@ -1941,7 +1944,7 @@ static JoinCfg join_cfg(int width, int agg, int checksum, uint64_t expect_r) {
     const uint64_t slot = join_slot_bytes(width, agg, checksum);
     const uint64_t need = 3 * (expect_r + 6 * (uint64_t)__builtin_sqrt((double)expect_r + 1.0) + 64) * slot;
     if (need <= (100ull << 10)) return JoinCfg{agg ? 512 : 320, 100ull << 10};
-    return JoinCfg{agg ? 1024 : 640, 200ull << 10};
+    return JoinCfg{agg ? 1024 : 640, agg ? 200ull << 10 : 209ull << 10};
 }
 
 // (two CTAs of an SM then cover each other's waits: 200 joins of 3e7 with 1.2e8 tuples 700 us

@@ -1,7 +1,7 @@
 """The shared-memory join of partition pairs, against the CPU oracle: the probe loop
 for tables whose keys are all different and the general one, chosen per partition by
 comparing the table's keys (also those that moved past a full bucket), at slice sizes
-around whole groups; more tasks than two per CTA, so that some are taken ahead; a pair
+around whole groups; the largest build partitions that the table takes; more tasks than two per CTA, so that some are taken ahead; a pair
 buffer that ends inside a warp's chunk.  Integer results: every comparison is exact."""
 import numpy as np
 import pytest
@@ -100,3 +100,23 @@ def test_both_relations_in_one_pass(hjm, ctx, width, bits, nr, ns):
     r = _rel(rng.permutation(np.arange(1, nr + 1)), width)
     s = _rel(rng.integers(1, 2 * nr + 2, ns), width)
     _check(hjm, ctx, r, s, radix_bits=bits)
+
+
+@pytest.mark.parametrize("width,per", [(4, 18_000), (4, 19_400), (8, 8_900), (8, 9_400)])
+def test_largest_partitions_stay_in_shared_memory(hjm, ctx, width, per):
+    # 25088 4-byte or 12160 8-byte slots at a load of at most 4/5 take partitions of up to 20070
+    # or 9728 rows (the largest of these 8 hold 19593 and 9577, and less than 60 of padding)
+    rng = np.random.default_rng(per)
+    r = _rel(rng.permutation(np.arange(1, 8 * per + 1)), width)
+    s = _rel(rng.integers(1, 16 * per, 100_003), width)
+    hjm.prof_reset(ctx)
+    hjm.prof_enable(ctx, True)
+    try:
+        res = hjm.hj_join(ctx, _gpu(r), _gpu(s), algo=hjm.HJ_ALGO_PHJ, radix_bits=3, passes=1)
+        launched = set(hjm.prof_read(ctx))
+    finally:
+        hjm.prof_enable(ctx, False)
+    got = res.pairs_numpy().astype(np.uint64)
+    res.free()
+    assert np.array_equal(oracle.sorted_pairs(got[:, 0], got[:, 1]), oracle.sorted_pairs(*oracle.hash_join(r, s)))
+    assert "partition_join" in launched and "fallback_tasks" not in launched
