@@ -928,6 +928,8 @@ template <int W> struct WarpStageSink {
     __device__ __forceinline__ void end_task() {}
     __device__ __forceinline__ void finish() { flush(); }
 };
+// The same with the buffers in global memory (they stay in L2).
+template <int W> struct GlobalStageSink : WarpStageSink<W> {};
 
 // Longest walk (in buckets) of an insert into a partition's shared-memory table.
 constexpr uint32_t kMaxSmemWalk = 64;
@@ -1289,7 +1291,7 @@ __host__ __device__ constexpr int join_ctas(int nt) { return nt > 512 ? 1 : 2; }
 template <int W, bool AGG, int NT, class Sink, bool FAST>
 __global__ void __launch_bounds__(NT, join_ctas(NT)) partition_join_kernel(
     const PartTask *tasks, uint64_t ntasks, uint64_t lead, const JoinSlot *slots, hj_counters *work, uint32_t cap_max, RecArea ra,
-    uint32_t *oversize, int chk, uint32_t stage_at) {
+    uint32_t *oversize, int chk, uint32_t stage_at, void *stage) {
     using T = typename Tup<W>::U;
     using Vec = typename Tup<W>::Vec;
     constexpr int PV = Tup<W>::kPerVec, U = 2, IT = U * PV;
@@ -1306,7 +1308,11 @@ __global__ void __launch_bounds__(NT, join_ctas(NT)) partition_join_kernel(
         sink.slots = slots;
         sink.ra = ra;
     } else {
-        sink.stage = (typename WarpStageSink<W>::P *)(smem + stage_at + warp * kJoinStageBytes);
+        using P = typename WarpStageSink<W>::P;
+        if constexpr (std::is_same<Sink, GlobalStageSink<W>>::value)
+            sink.stage = (P *)((char *)stage + ((size_t)blockIdx.x * nwarps + warp) * kJoinStageBytes);
+        else
+            sink.stage = (P *)(smem + stage_at + warp * kJoinStageBytes);
         sink.scap = kJoinStageBytes / (2 * W);
         sink.slots = slots;
     }
@@ -1968,40 +1974,55 @@ hj_status partition_join(hj_ctx *c, int width, int agg, const PartTask *tasks, u
     uint64_t want = (uint64_t)(3.0 * (mean + 6.0 * __builtin_sqrt(mean + 1.0) + 64.0));
     want = (want + 127) / 128 * 128;
     const uint64_t bitmap_bytes = 4096;
-    // the fast probe (no aggregate, no checksum) adds each warp's walk queue, staged
-    // output its buffer, within what the shape's CTAs per SM can have
-    const uint64_t stage_bytes = staged ? (uint64_t)(cfg.nt / 32) * kJoinStageBytes : 0;
-    const uint64_t qbytes = ((!agg && !checksum) ? (uint64_t)(cfg.nt / 32) * kWalkQ * 2 * width : 0) + stage_bytes;
-    const uint64_t total_max = join_ctas(cfg.nt) == 2 ? (112ull << 10) : (222ull << 10);
-    const uint64_t budget = std::min<uint64_t>(cfg.smem_limit + qbytes, total_max) - qbytes;
-    uint64_t max_slots = agg ? (budget - bitmap_bytes) / slot_bytes / 128 * 128
-                             : (budget - 16) * 8 / (8 * slot_bytes + (uint64_t)width) / 128 * 128;
+    // the fast probe (no aggregate, no checksum) adds each warp's walk queue, output
+    // staged in shared memory its buffer, within what the shape's CTAs per SM can have
+    const uint64_t warps = (uint64_t)(cfg.nt / 32), total_max = join_ctas(cfg.nt) == 2 ? (112ull << 10) : (222ull << 10);
+    const uint64_t queues = !agg && !checksum ? warps * kWalkQ * 2 * width : 0;
+    auto slots_beside = [&](uint64_t extra) {
+        const uint64_t budget = std::min<uint64_t>(cfg.smem_limit + extra, total_max) - extra;
+        return agg ? (budget - bitmap_bytes) / slot_bytes / 128 * 128
+                   : (budget - 16) * 8 / (8 * slot_bytes + (uint64_t)width) / 128 * 128;
+    };
+    uint64_t stage_bytes = staged ? warps * kJoinStageBytes : 0;
+    // Staging takes up to 80 KB that a large build partition needs: past a load of 0.46 the
+    // buffers go to global memory (u32 14e6 / 2^24 / 18e6 / 22e6 build rows on 2^11
+    // partitions 641 / 746 / 797 / 1258 us in shared memory, 678 / 727 / 743 / 953 us in
+    // global; u64 6e6 / 7e6 / 8e6 / 10e6 786 / 866 / 1170 / 1893 and 811 / 858 / 1099 / 1217)
+    // and the tables hold as many rows as those of a single join.
+    const bool in_global = staged && join_ctas(cfg.nt) == 1 && mean > 0.46 * (double)slots_beside(queues + stage_bytes);
+    if (in_global) stage_bytes = 0;
+    const uint64_t max_slots = slots_beside(queues + stage_bytes);
     uint64_t cap_max = want < max_slots ? want : max_slots;
     if (cap_max < 128) cap_max = 128;
-    const size_t smem = (size_t)walkq_offset((uint32_t)cap_max, (uint32_t)slot_bytes, width, agg != 0) + (size_t)qbytes;
+    const size_t smem = (size_t)walkq_offset((uint32_t)cap_max, (uint32_t)slot_bytes, width, agg != 0) +
+                        (size_t)(queues + stage_bytes);
     unsigned grid = (unsigned)num_sms(c) * join_ctas(cfg.nt);
     if (grid > ntasks) grid = (unsigned)ntasks;
-#define HJ_PJ(WW, AA, NT, SK, FF)                                                                               \
-    do {                                                                                                        \
-        auto kern = partition_join_kernel<WW, AA, NT, SK<WW>, FF>;                                              \
-        HJ_TRY(allow_max_smem(c, (const void *)kern));                                                         \
+    DevBuf gstage(c);  // (freed in stream order after the launch)
+    if (in_global) HJ_TRY(gstage.alloc((uint64_t)grid * warps * kJoinStageBytes));
+#define HJ_PJ(WW, AA, NT, SK, FF)                                                                                     \
+    do {                                                                                                              \
+        auto kern = partition_join_kernel<WW, AA, NT, SK<WW>, FF>;                                                    \
+        HJ_TRY(allow_max_smem(c, (const void *)kern));                                                                \
         HJ_LAUNCH(c, "partition_join", kern, grid, NT, smem, tasks, ntasks, lead, slots, c->d_ctr, (uint32_t)cap_max, \
-                  ra, oversize, checksum, (uint32_t)(smem - stage_bytes));                                                         \
+                  ra, oversize, checksum, (uint32_t)(smem - stage_bytes), gstage.p);                                  \
     } while (0)
-#define HJ_PJ_NT(WW, AA, SK, FF)                                \
-    do {                                                        \
+#define HJ_PJ_NT(WW, AA, SK, FF)                                             \
+    do {                                                                     \
         if (join_ctas(cfg.nt) == 2) HJ_PJ(WW, AA, (AA ? 512 : 320), SK, FF); \
-        else HJ_PJ(WW, AA, (AA ? 1024 : 640), SK, FF);           \
+        else HJ_PJ(WW, AA, (AA ? 1024 : 640), SK, FF);                       \
     } while (0)
-#define HJ_PJ_F(WW, SK)                                         \
-    do {                                                        \
+#define HJ_PJ_F(WW, SK)                                          \
+    do {                                                         \
         if (checksum) HJ_PJ_NT(WW, false, SK, false);            \
         else HJ_PJ_NT(WW, false, SK, true);                      \
     } while (0)
-#define HJ_PJ_SK(WW)                                            \
-    do {                                                        \
-        if (staged) HJ_PJ_F(WW, WarpStageSink);                       \
-        else HJ_PJ_F(WW, ChunkSink);                             \
+#define HJ_PJ_SK(WW)                                                             \
+    do {                                                                         \
+        if (!staged) HJ_PJ_F(WW, ChunkSink);                                     \
+        else if (!in_global) HJ_PJ_F(WW, WarpStageSink);                         \
+        else if (checksum) HJ_PJ(WW, false, 640, GlobalStageSink, false);        \
+        else HJ_PJ(WW, false, 640, GlobalStageSink, true);                       \
     } while (0)
     if (width == 4) {
         if (agg) HJ_PJ_NT(4, true, ChunkSink, false); else HJ_PJ_SK(4);

@@ -199,3 +199,39 @@ def test_batch_partitions_every_fanout_at_once(hjm, ctx, width):
         assert (cnt[j].count, *cnt[j].checksum) == oracle.join_aggregate(R, S), j
         assert np.array_equal(_sorted(res[j].pairs_numpy()), want), j
         res[j].free()
+
+
+@pytest.mark.parametrize("width,nr", [(4, 25_000_000), (8, 12_000_000)])
+def test_batch_with_a_large_build_side_joins_in_shared_memory(hjm, ctx, width, nr):
+    # partitions of 12207 (8-byte: 5859) build rows on 2^11 digits leave no shared memory for
+    # the warps' pairs, which are then collected in global memory, not for the fallback
+    n2 = 5000
+    dt = torch.int32 if width == 4 else torch.int64
+    g = torch.Generator(device=DEV).manual_seed(nr)
+    Rs, Ss = [], []
+    for n, m in ((n2, 3 * n2), (nr, 300_001), (n2 // 2, 7)):
+        rk = torch.randperm(n, device=DEV, generator=g) + 1
+        sk = torch.randint(1, 2 * n, (m,), device=DEV, generator=g)
+        for k, rels in ((rk, Rs), (sk, Ss)):
+            rels.append(torch.stack([k.to(dt), torch.arange(len(k), dtype=dt, device=DEV)], 1))
+    for checksum in (False, True):
+        hjm.prof_reset(ctx)
+        hjm.prof_enable(ctx, True)
+        try:
+            res = hjm.hj_join_batch(ctx, Rs, Ss, checksum=checksum)
+            launched = set(hjm.prof_read(ctx))
+        finally:
+            hjm.prof_enable(ctx, False)
+        assert "partition_join" in launched and "fallback_tasks" not in launched
+        for r, R, S in zip(res, Rs, Ss):
+            # every key of R is its own row's: row of R by key, -1 where there is none
+            at = torch.full((2 * len(R) + 1,), -1, dtype=dt, device=DEV)
+            at[R[:, 0].long()] = R[:, 1]
+            hit = at[S[:, 0].long()] >= 0
+            want = torch.stack([at[S[:, 0].long()][hit], S[:, 1][hit]], 1).cpu().numpy()
+            got = r.pairs_numpy()
+            assert r.count == len(want)
+            assert np.array_equal(_sorted(got), _sorted(want.view(got.dtype)))
+            if checksum and len(R) < nr:
+                assert (r.count, *r.checksum) == oracle.join_aggregate(W.to_numpy_u(R), W.to_numpy_u(S))
+            r.free()
