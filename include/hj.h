@@ -465,6 +465,10 @@ hj_status hj_debug_outcore(hj_ctx *ctx, int mode);
  * with reset != 0, which then restarts the count from the bytes held now.  0 for
  * a NULL context. */
 uint64_t hj_debug_peak_bytes(hj_ctx *ctx, int reset);
+/* Test hook: the slots of the pair table that hj_build and SHJ make for n_build tuples
+ * of `width`-byte fields, on a context with or without a memory budget (no GPU
+ * needed).  0 for another width. */
+uint64_t hj_debug_table_slots(int width, uint64_t n_build, int budget);
 
 #ifdef __cplusplus
 }

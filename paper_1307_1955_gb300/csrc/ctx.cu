@@ -7,6 +7,7 @@
 
 #include "common.cuh"
 #include "ctx.cuh"
+#include "engine.cuh"
 
 namespace hj {
 
@@ -366,6 +367,10 @@ hj_status hj_debug_wait_limit(hj_ctx *c, uint64_t n) {
 }
 
 /* Measurement hook: force the region or the ring scatter (HJ_SCATTER_*). */
+uint64_t hj_debug_table_slots(int width, uint64_t n_build, int budget) {
+    return width == HJ_U32 || width == HJ_U64 ? hj::table_slots(width, 0, n_build, budget != 0) : 0;
+}
+
 hj_status hj_debug_scatter(hj_ctx *c, int kind) {
     if (!c || kind < HJ_SCATTER_AUTO || kind > HJ_SCATTER_RING) return HJ_E_INVALID;
     c->scatter_kind = kind;

@@ -15,6 +15,8 @@ struct RecArea;  // emit.cuh
 // Global-memory table (SHJ, Alg. 1): allocate + initialise (with zero_ctr the
 // context's counters too), build, probe.
 hj_status table_create(hj_ctx *c, int width, int agg, uint64_t n_build, hj_table **out, bool zero_ctr = false);
+// The slots it allocates: more than n_build; of a pair table below 2^32 buckets.
+uint64_t table_slots(int width, int agg, uint64_t n_build, bool budget);
 void table_destroy(hj_ctx *c, hj_table *t);
 // Key-list table (keylist.cu): aggregate-table slots over the kept tuples of
 // R[0, n) plus the rid lists (t->rids, every key's rids contiguous at the offset

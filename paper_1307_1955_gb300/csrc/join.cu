@@ -455,16 +455,24 @@ __global__ void __launch_bounds__(256) pair_table_init(ulonglong2 *slots, uint64
     if (ctr && i0 < offsetof(hj_counters, fault) / 8) ((unsigned long long *)ctr)[i0] = 0;
 }
 
-hj_status table_create(hj_ctx *c, int width, int agg, uint64_t n_build, hj_table **out, bool zero_ctr) {
-    *out = nullptr;
+uint64_t table_slots(int width, int agg, uint64_t n_build, bool budget) {
     // Capacity: a power of two at least twice the build size (load factor <= 0.5).  A
     // pair table takes four slots per tuple (2 % of 4-byte buckets are then full, 5 %
     // at three: 2^24 probes of 2^18 tuples 106 us against 123 us) unless the context
     // has a memory budget, which keeps the smaller size it always had.
     uint64_t cap = 64;
     while (cap < 2 * n_build + 1) cap <<= 1;
-    uint64_t slot_bytes = agg ? (width == 4 ? sizeof(AggSlot<4>) : sizeof(AggSlot<8>)) : 2ull * width;
-    if (!agg && !c->budget && 4 * n_build * slot_bytes <= kFastTableBytes) cap = std::max<uint64_t>(64, 4 * n_build);
+    if (agg) return cap;
+    if (!budget && 4 * n_build * 2 * width <= kFastTableBytes) cap = std::max<uint64_t>(64, 4 * n_build);
+    // (a bucket's number is 32 bits; the last power of two of 8-byte tuples would have one more)
+    const uint64_t g = width == 4 ? kBucketSlots<4> : kBucketSlots<8>;
+    return std::min<uint64_t>(cap, 0xFFFFFFFFull * g);
+}
+
+hj_status table_create(hj_ctx *c, int width, int agg, uint64_t n_build, hj_table **out, bool zero_ctr) {
+    *out = nullptr;
+    const uint64_t slot_bytes = agg ? (width == 4 ? sizeof(AggSlot<4>) : sizeof(AggSlot<8>)) : 2ull * width;
+    const uint64_t cap = table_slots(width, agg, n_build, c->budget != 0);
     DevBuf slots(c), side(c);
     HJ_TRY(slots.alloc(cap * slot_bytes));
     HJ_TRY(side.alloc(sizeof(TableSide)));

@@ -62,6 +62,22 @@ def test_debug_hooks_reject_a_null_context_without_a_gpu(lib):
         assert f(*args) == 1, name  # HJ_E_INVALID
 
 
+@pytest.mark.parametrize("budget", [0, 1])
+@pytest.mark.parametrize("width,group", [(4, 4), (8, 2)])
+def test_pair_table_has_a_32_bit_number_of_buckets(lib, width, group, budget):
+    # for every build side that is accepted (below 2^32 - 1 tuples): more slots than tuples, at
+    # a load of at most a half but for the last bucket, and a bucket number of 32 bits
+    f = lib.hj_debug_table_slots
+    f.restype = ctypes.c_uint64
+    f.argtypes = [ctypes.c_int, ctypes.c_uint64, ctypes.c_int]
+    for n in (0, 1, 16, 17, 1000, 1 << 20, (1 << 22) + 1, 1 << 30, (1 << 31) - 1, 1 << 31, (1 << 31) + 1, (1 << 32) - 2):
+        slots = f(width, n, budget)
+        assert slots % group == 0 and slots >= 64
+        assert slots // group < 1 << 32, n
+        assert slots >= 2 * n and slots > n
+    assert f(5, 10, 0) == 0
+
+
 def test_server_calls_reject_null_handles_without_a_gpu(lib):
     for name, args in (("hj_server_create", (None, None, None)), ("hj_server_submit", (None, None, None, 0, None)),
                        ("hj_server_poll", (None, 1, None, None)), ("hj_server_destroy", (None,)),
