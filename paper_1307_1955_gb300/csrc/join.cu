@@ -942,6 +942,13 @@ template <int W> struct GlobalStageSink : WarpStageSink<W> {};
 // Longest walk (in buckets) of an insert into a partition's shared-memory table.
 constexpr uint32_t kMaxSmemWalk = 64;
 
+// When no more walks than this are left of 32 after three buckets, the warp takes one after
+// the other, 32 slots at a time, in place of all at once, a bucket at a time (each key of R
+// 16 times: 3580 us without this, 3330 with).  Before that the walks left are short ones,
+// which end sooner together (taken one by one from the first bucket on: 2^24 x 2^28 tuples
+// of different keys 2330 -> 2500 us).
+constexpr int kLongWalks = 2;
+
 // Entries per warp of the queue of pending run walks (probe keys and rids whose
 // run goes on past a full home bucket).
 constexpr uint32_t kWalkQ = 64;
@@ -961,10 +968,10 @@ constexpr uint32_t kAheadVecs = 4096;
 __device__ __forceinline__ void prefetch_l2(const void *p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 // The walks of n <= 32 queued items, one per lane: each lane follows its key's run
-// from the bucket after its home and emits every match found there.  A walk is
-// rare (a few per cent of probes), so walking them one lane at a time as they
-// come would cost a whole warp pass each; batched, 32 walks cost about one.
-template <int W, class Sink>
+// from the bucket after its home and emits every match found there, a bucket per step.
+// Walking them one lane at a time as they come would cost a whole warp pass each;
+// batched, 32 walks of like length cost about one.
+template <int W, bool UNIQ, class Sink>
 __device__ __forceinline__ void drain_walks(const SoaTab<W> &tab, const typename Tup<W>::U *qk,
                                             const typename Tup<W>::U *qr, uint32_t n, Sink &sink) {
     using T = typename Tup<W>::U;
@@ -979,32 +986,42 @@ __device__ __forceinline__ void drain_walks(const SoaTab<W> &tab, const typename
         const uint32_t h = part_bucket<W>(kk, tab.nb);
         b = h + 1 == tab.nb ? 0 : h + 1;
     }
-    for (uint32_t it = 0; it < tab.nb; ++it) {
-        if (!__any_sync(0xffffffffu, active)) break;
+#pragma unroll 1
+    for (uint32_t it = 1; it < tab.nb; ++it) {
+        unsigned on = __ballot_sync(0xffffffffu, active);
+        if (!on || (it > 3 && __popc(on) <= kLongWalks)) {  // the long runs that are left: 32 slots at a time
+            while (on) {
+                const int L = __ffs(on) - 1;
+                on &= on - 1;
+                soa_coop_emit<W>(tab, __shfl_sync(0xffffffffu, kk, L), __shfl_sync(0xffffffffu, rr, L),
+                                 __shfl_sync(0xffffffffu, b, L), sink);
+            }
+            break;
+        }
+        T key[G];
+        tab.ld(b, 0, key);  // (a bucket of the table whatever the lane)
         uint32_t m = 0;
-        bool e = false;
-        if (active) {
-            T key[G];
-            tab.ld(b, 0, key);
 #pragma unroll
-            for (uint32_t q = 0; q < G; ++q) {
-                m |= (uint32_t)(key[q] == kk) << q;
-                e |= key[q] == tab.empty;
+        for (uint32_t q = 0; q < G; ++q) m |= (uint32_t)(active && key[q] == kk) << q;
+        const bool any = m != 0;
+        if (__any_sync(0xffffffffu, any)) {
+            if (UNIQ) {
+                sink.append(any, any ? tab.ld1(b, 1, (uint32_t)(__ffs(m) - 1)) : T(0), rr);
+                active = active && !any;
+            } else {
+                T rid[G], sr[G];
+                bool hit[G];
+                tab.ld(b, 1, rid);
+#pragma unroll
+                for (uint32_t q = 0; q < G; ++q) {
+                    hit[q] = (m >> q) & 1u;
+                    sr[q] = rr;
+                }
+                sink.template append_found<G>(hit, rid, sr);
             }
         }
-        // the matches of this bucket, one append per round (several only for
-        // duplicate build keys)
-        for (uint32_t q = 0; q < G; ++q) {
-            const bool hm = m != 0;
-            if (!__any_sync(0xffffffffu, hm)) break;
-            T v = 0;
-            if (hm) {
-                v = tab.ld1(b, 1, (uint32_t)(__ffs(m) - 1));
-                m &= m - 1;
-            }
-            sink.append(hm, v, rr);
-        }
-        active = active && !e && tab.overflowed(b);
+        // (slots fill in order: an empty one is the last)
+        active = active && key[G - 1] != tab.empty && tab.overflowed(b);
         b = b + 1 == tab.nb ? 0 : b + 1;
     }
 }
@@ -1042,9 +1059,12 @@ template <int W, int NT> __device__ __forceinline__ bool keys_repeat(const SoaTa
 // bucket's slots in order and move past it only once it is full, so a run goes on past
 // the home bucket only if the bucket's last slot is taken AND more inserts tried it than
 // it has slots: such items are queued and their runs walked 32 at a time.  With UNIQ (no
-// key is twice in the table) a match ends the search; otherwise an item with several
-// matches in its home bucket has its whole run walked by the warp.  With MARK the marker
-// of empty slots may be a key: its build rids are the `side` list.
+// key is twice in the table) a match ends the search; otherwise the further matches of the
+// home buckets go out one per item and step.  (A warp that walked one such item after the
+// other lived from many warps, 32 of them; with 20, |R| = 2^22 4-byte tuples of each key
+// twice / 4 / 16 times with 2^24: 3640 / 3860 / 5860 us, like this 575 / 937 / 3330; each key
+// four times with 8 bytes 4260 and 1665.)  With MARK the marker of empty slots may be a key:
+// its build rids are the `side` list.
 template <int W> struct SideList {
     const typename Tup<W>::U *rids = nullptr;
     uint32_t n = 0;
@@ -1072,40 +1092,38 @@ __device__ __forceinline__ void probe_group_smem(const SoaTab<W> &tab, const typ
         home[i] = part_bucket<W>(k[i], tab.nb);  // < nb for any key: the load is in bounds
         tab.ld(home[i], 0, kb[i]);
     }
-    bool found[IT], w[IT], several[IT], anyw = false, anys = false;
+    bool found[IT], w[IT], anyw = false;
+    uint32_t more = 0;  // further matches in the home buckets: G bits per item
 #pragma unroll
     for (int i = 0; i < IT; ++i) {
         const bool live = (FULL || in[i]) && !(MARK && k[i] == tab.empty);
-        uint32_t sl = home[i] * G + (G - 1), c = kb[i][G - 1] == k[i];
+        uint32_t sl = home[i] * G + (G - 1), m = (uint32_t)(kb[i][G - 1] == k[i]) << (G - 1);
         bool f = kb[i][G - 1] == k[i];
 #pragma unroll
         for (int q = (int)G - 2; q >= 0; --q) {
             const bool h = kb[i][q] == k[i];
             sl = h ? home[i] * G + q : sl;
             f |= h;
-            c += h;
+            m |= (uint32_t)h << q;
         }
         first[i] = tab.rptr[sl];
-        several[i] = !UNIQ && live && c > 1;
-        found[i] = live && f && !several[i];
-        w[i] = live && !(UNIQ && f) && !several[i] && kb[i][G - 1] != tab.empty && tab.overflowed(home[i]);
+        found[i] = live && f;
+        if (!UNIQ && live) more |= (m & (m - 1u)) << (i * G);
+        w[i] = live && !(UNIQ && f) && kb[i][G - 1] != tab.empty && tab.overflowed(home[i]);
         anyw |= w[i];
-        anys |= several[i];
     }
     sink.template append_found<IT>(found, first, r);
-    if (!UNIQ && __any_sync(0xffffffffu, anys)) {
+    if (!UNIQ)
+        while (__any_sync(0xffffffffu, more != 0)) {  // (at most G - 1 times)
 #pragma unroll
-        for (int i = 0; i < IT; ++i) {
-            unsigned m = __ballot_sync(0xffffffffu, several[i]);
-            while (m) {
-                const int L = __ffs(m) - 1;
-                m &= m - 1;
-                const T kk = __shfl_sync(0xffffffffu, k[i], L);
-                const T ss = __shfl_sync(0xffffffffu, r[i], L);
-                soa_coop_emit<W>(tab, kk, ss, part_bucket<W>(kk, tab.nb), sink);
+            for (int i = 0; i < IT; ++i) {
+                const uint32_t m = (more >> (i * G)) & ((1u << G) - 1u);
+                found[i] = m != 0;
+                if (m) first[i] = tab.ld1(home[i], 1, (uint32_t)(__ffs(m) - 1));
+                more &= ~((m & (0u - m)) << (i * G));
             }
+            sink.template append_found<IT>(found, first, r);
         }
-    }
     if (MARK && side.n) {
 #pragma unroll
         for (int i = 0; i < IT; ++i) {
@@ -1134,7 +1152,7 @@ __device__ __forceinline__ void probe_group_smem(const SoaTab<W> &tab, const typ
             qn += (uint32_t)__popc(wm);
             if (qn >= 32) {
                 __syncwarp();
-                drain_walks<W>(tab, wqk + (qn - 32), wqr + (qn - 32), 32, sink);
+                drain_walks<W, UNIQ>(tab, wqk + (qn - 32), wqr + (qn - 32), 32, sink);
                 qn -= 32;
             }
         }
@@ -1187,7 +1205,7 @@ __device__ __forceinline__ void probe_smem(const SoaTab<W> &tab, const typename 
     }
     if (qn) {
         __syncwarp();
-        drain_walks<W>(tab, wqk, wqr, qn, sink);
+        drain_walks<W, UNIQ>(tab, wqk, wqr, qn, sink);
     }
 }
 
@@ -1800,7 +1818,7 @@ __global__ void __launch_bounds__(NT, join_ctas(NT)) small_join_kernel(const voi
             probe_group_smem<W, 1, false, false, true>(tab, x, in, sink, lane, wq, wq + kWalkQ, qn, side);
             if (qn) {
                 __syncwarp();
-                drain_walks<W>(tab, wq, wq + kWalkQ, qn, sink);
+                drain_walks<W, false>(tab, wq, wq + kWalkQ, qn, sink);
             }
         }
     }

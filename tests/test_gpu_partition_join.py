@@ -1,8 +1,9 @@
 """The shared-memory join of partition pairs, against the CPU oracle: the probe loop
 for tables whose keys are all different and the general one, chosen per partition by
-comparing the table's keys (also those that moved past a full bucket), at slice sizes
-around whole groups; the largest build partitions that the table takes; more tasks than two per CTA, so that some are taken ahead; a pair
-buffer that ends inside a warp's chunk.  Integer results: every comparison is exact."""
+comparing the table's keys (also those that moved past a full bucket); runs of repeated
+keys; slice sizes around whole groups; the largest build partitions that the table takes;
+more tasks than two per CTA, so that some are taken ahead; a pair buffer that ends inside
+a warp's chunk.  Integer results: every comparison is exact."""
 import numpy as np
 import pytest
 import torch
@@ -71,6 +72,21 @@ def test_unique_and_repeated_keys(hjm, ctx, width, dups, per):
         keys = (keys + 1) // 2
     sk = rng.integers(1, 2 * n + 1, 4 * n + 77)
     _check(hjm, ctx, _rel(keys, width), _rel(sk, width), radix_bits=1)
+
+
+@pytest.mark.parametrize("copies", [3, 4, 5, 9, 33, 100, 300])
+@pytest.mark.parametrize("width", [4, 8])
+def test_runs_of_repeated_keys(hjm, ctx, width, copies):
+    # every key of R `copies` times, beside keys of one, two and twice as many rows: matches
+    # that fill the home bucket, runs over many buckets, all walked together or one after the
+    # other (the longest pass the insert's limit and take the key-list table)
+    rng = np.random.default_rng(copies + width)
+    k = 1200 // copies + 1
+    keys = np.concatenate([np.repeat(np.arange(1, k + 1), copies), np.repeat(np.arange(k + 1, k + 4), 2 * copies),
+                           np.arange(2000, 2400), np.repeat(np.arange(3000, 3100), 2)])
+    sk = rng.integers(1, 3200, 9001)
+    sk[:4000] = rng.integers(1, k + 4, 4000)
+    _check(hjm, ctx, _rel(rng.permutation(keys), width), _rel(sk, width), radix_bits=1)
 
 
 @pytest.mark.parametrize("ns", [1280, 1281, 1279, 2559, 2600, 5120 + 3])
