@@ -629,62 +629,6 @@ template <int W> struct SoaTab {
     }
 };
 
-// Lookup of key k: number of build matches and the rid of the first one.
-template <int W>
-__device__ __forceinline__ uint32_t soa_lookup(const SoaTab<W> &t, typename Tup<W>::U k, uint32_t home,
-                                               typename Tup<W>::U *first) {
-    using T = typename Tup<W>::U;
-    constexpr uint32_t G = SoaTab<W>::G;
-    uint32_t c = 0, bkt = home;
-    for (uint32_t it = 0; it < t.nb; ++it) {
-        T key[G];
-        t.ld(bkt, 0, key);
-        uint32_t m = 0;
-        bool e = false;
-#pragma unroll
-        for (uint32_t q = 0; q < G; ++q) {
-            m |= (uint32_t)(key[q] == k) << q;
-            e |= key[q] == t.empty;
-        }
-        if (m) {
-            T rid[G];
-            t.ld(bkt, 1, rid);
-            if (c == 0) {
-                T f = rid[G - 1];
-#pragma unroll
-                for (int q = (int)G - 2; q >= 0; --q)
-                    if ((m >> q) & 1u) f = rid[q];
-                *first = f;
-            }
-            c += __popc(m);
-        }
-        if (e || !t.overflowed(bkt)) break;
-        bkt = bkt + 1 == t.nb ? 0 : bkt + 1;
-    }
-    return c;
-}
-
-// Visit every build rid of key k (slow path for checksums).
-template <int W, class F>
-__device__ __forceinline__ void soa_visit(const SoaTab<W> &t, typename Tup<W>::U k, uint32_t home, F &&f) {
-    using T = typename Tup<W>::U;
-    constexpr uint32_t G = SoaTab<W>::G;
-    uint32_t bkt = home;
-    for (uint32_t it = 0; it < t.nb; ++it) {
-        T key[G], rid[G];
-        t.ld(bkt, 0, key);
-        t.ld(bkt, 1, rid);
-        bool e = false;
-#pragma unroll
-        for (uint32_t q = 0; q < G; ++q) {
-            if (key[q] == k) f(rid[q]);
-            e |= key[q] == t.empty;
-        }
-        if (e || !t.overflowed(bkt)) break;
-        bkt = bkt + 1 == t.nb ? 0 : bkt + 1;
-    }
-}
-
 // The whole warp emits every build match of key kk (probe rid ss): a window of
 // 32 slots (32 / G buckets) per step, up to the first bucket that ends the run.
 template <int W, class Sink>
@@ -723,6 +667,7 @@ __device__ __forceinline__ void soa_coop_emit(const SoaTab<W> &t, typename Tup<W
 // The join's pair count is the claim cursor (ctr->count).
 template <int W> struct ChunkSink {
     using T = typename Tup<W>::U;
+    static constexpr bool kCheck = false;
     OutState st;
     OutCtx oc;
     typename PairVec<W>::T *open = nullptr;  // the open chunk (append_found)
@@ -742,42 +687,6 @@ template <int W> struct ChunkSink {
         warp_append<W>(st, oc, has, a, b);
         open = (typename PairVec<W>::T *)oc.pairs + st.base;
         set_room();
-    }
-    // one append for all single-match items of a group
-    template <int IT>
-    __device__ __forceinline__ void append_group(const uint32_t *cnt, const T *first, const T *r) {
-        const unsigned lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
-        unsigned m[IT], tot = 0;
-#pragma unroll
-        for (int i = 0; i < IT; ++i) {
-            m[i] = __ballot_sync(0xffffffffu, cnt[i] == 1);
-            tot += __popc(m[i]);
-        }
-        if (!tot) return;
-        const unsigned room = kChunkPairs - st.used;
-        unsigned long long nbase = 0;
-        if (tot > room) {
-            if (lane == 0) nbase = atomicAdd(&oc.ctr->cursor, (unsigned long long)kChunkPairs);
-            nbase = __shfl_sync(0xffffffffu, nbase, 0);
-        }
-        unsigned run = 0;
-#pragma unroll
-        for (int i = 0; i < IT; ++i) {
-            if (cnt[i] == 1) {
-                const unsigned rank = run + __popc(m[i] & lt);
-                const unsigned long long pos = rank < room ? st.base + st.used + rank : nbase + (rank - room);
-                if (pos < oc.pcap) PairOut<W>::put(oc.pairs, pos, first[i], r[i]);
-            }
-            run += __popc(m[i]);
-        }
-        if (tot > room) {
-            st.base = nbase;
-            st.used = tot - room;
-            st.claimed = true;
-        } else {
-            st.used += tot;
-        }
-        st.pairs += tot;
     }
     // one append for all items of a group with a match (at most 32 * IT pairs, so at
     // most one new chunk): item-major positions, so that each store instruction
@@ -837,8 +746,6 @@ template <int W> struct ChunkSink {
     __device__ __forceinline__ void set_room() {
         room = st.claimed && st.base + kChunkPairs <= oc.pcap ? kChunkPairs - st.used : 0u;
     }
-    __device__ __forceinline__ hj_counters *ctr() const { return oc.ctr; }
-    __device__ __forceinline__ void end_task() {}
     __device__ __forceinline__ void finish() {
         if (join != ~0u) warp_finish(st, oc, ra);
     }
@@ -856,6 +763,7 @@ template <int W> struct ChunkSink {
 constexpr uint32_t kJoinStageBytes = 4096;
 template <int W> struct WarpStageSink {
     using T = typename Tup<W>::U;
+    static constexpr bool kCheck = false;
     using P = typename std::conditional<W == 4, uint2, ulonglong2>::type;
     P *stage = nullptr;  // this warp's buffer
     uint32_t scap = 0;
@@ -896,25 +804,6 @@ template <int W> struct WarpStageSink {
         used += k;
     }
     template <int IT>
-    __device__ __forceinline__ void append_group(const uint32_t *cnt, const T *first, const T *r) {
-        const unsigned lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
-        unsigned m[IT], tot = 0;
-#pragma unroll
-        for (int i = 0; i < IT; ++i) {
-            m[i] = __ballot_sync(0xffffffffu, cnt[i] == 1);
-            tot += __popc(m[i]);
-        }
-        if (!tot) return;
-        if (used + tot > scap) flush();
-        unsigned run = used;
-#pragma unroll
-        for (int i = 0; i < IT; ++i) {
-            if (cnt[i] == 1) stage[run + __popc(m[i] & lt)] = mk(first[i], r[i]);
-            run += __popc(m[i]);
-        }
-        used += tot;
-    }
-    template <int IT>
     __device__ __forceinline__ void append_found(const bool *found, const T *first, const T *r) {
         const unsigned lane = threadIdx.x & 31, lt = (1u << lane) - 1u;
         unsigned m[IT], tot = 0;
@@ -932,12 +821,29 @@ template <int W> struct WarpStageSink {
         }
         used += tot;
     }
-    __device__ __forceinline__ hj_counters *ctr() const { return slots[join].ctr; }
-    __device__ __forceinline__ void end_task() {}
     __device__ __forceinline__ void finish() { flush(); }
 };
 // The same with the buffers in global memory (they stay in L2).
 template <int W> struct GlobalStageSink : WarpStageSink<W> {};
+
+// Any of them with the checksums of the pairs it takes.
+template <int W, class Base> struct CheckSink : Base {
+    using T = typename Tup<W>::U;
+    static constexpr bool kCheck = true;
+    ProbeAcc acc;
+    __device__ __forceinline__ void append(bool has, T a, T b) {
+        add_check<W, true>(acc, has, a, b);
+        Base::append(has, a, b);
+    }
+    template <int IT> __device__ __forceinline__ void append_found(const bool *found, const T *first, const T *r) {
+#pragma unroll
+        for (int i = 0; i < IT; ++i) add_check<W, true>(acc, found[i], first[i], r[i]);
+        Base::template append_found<IT>(found, first, r);
+    }
+};
+template <int W> using ChunkCheckSink = CheckSink<W, ChunkSink<W>>;
+template <int W> using WarpStageCheckSink = CheckSink<W, WarpStageSink<W>>;
+template <int W> using GlobalStageCheckSink = CheckSink<W, GlobalStageSink<W>>;
 
 // Longest walk (in buckets) of an insert into a partition's shared-memory table.
 constexpr uint32_t kMaxSmemWalk = 64;
@@ -1311,16 +1217,92 @@ template <int W> struct AggSoa {
     }
 };
 
-// CTAs per SM of the join kernel's launch shapes.
-__host__ __device__ constexpr int join_ctas(int nt) { return nt > 512 ? 1 : 2; }
-
-template <int W, bool AGG, int NT, class Sink, bool FAST>
-__global__ void __launch_bounds__(NT, join_ctas(NT)) partition_join_kernel(
-    const PartTask *tasks, uint64_t ntasks, uint64_t lead, const JoinSlot *slots, hj_counters *work, uint32_t cap_max, RecArea ra,
-    uint32_t *oversize, int chk, uint32_t stage_at, void *stage) {
+// A CTA's probe of a slice of nsv vectors with a partition's aggregate table: the home
+// buckets of all of a lane's items are loaded before the first one is looked at.  No
+// partition filter: a padding tuple's key hashes to another partition, so it matches no
+// slot.
+template <int W>
+__device__ __forceinline__ void probe_smem_agg(const AggSoa<W> &at, const typename Tup<W>::Vec *Sv, uint32_t nsv, int chk,
+                                               ProbeAcc &acc, unsigned warp, unsigned nwarps, unsigned lane) {
     using T = typename Tup<W>::U;
     using Vec = typename Tup<W>::Vec;
     constexpr int PV = Tup<W>::kPerVec, U = 2, IT = U * PV;
+    constexpr uint32_t AG = AggSoa<W>::G;
+    const uint32_t gstride = nwarps * 32 * U;
+    Vec cur[U], nxt[U];
+    uint32_t g = warp * 32 * U;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const uint32_t rel = g + u * 32 + lane;
+        if (rel < nsv) cur[u] = ld_stream(Sv + rel);
+    }
+    for (; g < nsv; g += gstride) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint32_t rel = g + gstride + u * 32 + lane;
+            if (rel < nsv) nxt[u] = ld_stream(Sv + rel);
+        }
+        T k[IT], r[IT];
+        bool val[IT];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const bool in = g + u * 32 + lane < nsv;
+            if constexpr (W == 4) {
+                k[2 * u] = cur[u].x; r[2 * u] = cur[u].y; k[2 * u + 1] = cur[u].z; r[2 * u + 1] = cur[u].w;
+                val[2 * u] = in;
+                val[2 * u + 1] = in;
+            } else {
+                k[u] = cur[u].x; r[u] = cur[u].y;
+                val[u] = in;
+            }
+        }
+        uint32_t home[IT];
+        T kb[IT][AG];
+#pragma unroll
+        for (int i = 0; i < IT; ++i) {
+            home[i] = part_bucket<W>(k[i], at.nb);
+#pragma unroll
+            for (uint32_t q = 0; q < AG; ++q) kb[i][q] = at.empty;
+            if (val[i]) at.ld(home[i], kb[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < IT; ++i) {
+            uint32_t mm = 0;
+            bool e = false;
+#pragma unroll
+            for (uint32_t q = 0; q < AG; ++q) {
+                mm |= (uint32_t)(kb[i][q] == k[i]) << q;
+                e |= kb[i][q] == at.empty;
+            }
+            // (a lane past the slice's end holds a stale key: no slot)
+            uint32_t sl = val[i] && mm ? home[i] * AG + (uint32_t)(__ffs(mm) - 1) : ~0u;
+            if (val[i] && !mm && !e && at.overflowed(home[i]))  // the run continues (rare)
+                sl = at.find_from(k[i], home[i] + 1 == at.nb ? 0 : home[i] + 1);
+            if (sl != ~0u) {
+                const uint64_t n = at.cnt[sl];
+                acc.cnt += n;
+                if (chk) {
+                    const uint64_t sa = at.suma[sl], bb = mix_b(r[i]);
+                    acc.c0 += sa * bb;
+                    acc.c1 += sa + n * bb;
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) cur[u] = nxt[u];
+    }
+}
+
+// CTAs per SM of the join kernel's launch shapes.
+__host__ __device__ constexpr int join_ctas(int nt) { return nt > 512 ? 1 : 2; }
+
+template <int W, bool AGG, int NT, class Sink>
+__global__ void __launch_bounds__(NT, join_ctas(NT)) partition_join_kernel(
+    const PartTask *tasks, uint64_t ntasks, uint64_t lead, const JoinSlot *slots, hj_counters *work, uint32_t cap_max,
+    RecArea ra, uint32_t *oversize, int chk, uint32_t stage_at, void *stage) {
+    using T = typename Tup<W>::U;
+    using Vec = typename Tup<W>::Vec;
+    constexpr int PV = Tup<W>::kPerVec;
     constexpr uint32_t G = SoaTab<W>::G, AG = AggSoa<W>::G;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_full;
@@ -1330,12 +1312,12 @@ __global__ void __launch_bounds__(NT, join_ctas(NT)) partition_join_kernel(
     const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
 
     Sink sink;
-    if constexpr (std::is_same<Sink, ChunkSink<W>>::value) {
+    if constexpr (std::is_base_of<ChunkSink<W>, Sink>::value) {
         sink.slots = slots;
         sink.ra = ra;
     } else {
         using P = typename WarpStageSink<W>::P;
-        if constexpr (std::is_same<Sink, GlobalStageSink<W>>::value)
+        if constexpr (std::is_base_of<GlobalStageSink<W>, Sink>::value)
             sink.stage = (P *)((char *)stage + ((size_t)blockIdx.x * nwarps + warp) * kJoinStageBytes);
         else
             sink.stage = (P *)(smem + stage_at + warp * kJoinStageBytes);
@@ -1517,155 +1499,23 @@ __global__ void __launch_bounds__(NT, join_ctas(NT)) partition_join_kernel(
                     prefetch_l2(i < rl ? (const char *)nt.R + (uint64_t)i * 128 : (const char *)nt.S + (uint64_t)(i - rl) * 128);
             }
             bool unique = false;
-            if constexpr (FAST) unique = nsv >= 2 * nrv && !s_full && !__syncthreads_or(keys_repeat<W, NT>(tab));
+            if constexpr (!AGG) unique = nsv >= 2 * nrv && !s_full && !__syncthreads_or(keys_repeat<W, NT>(tab));
             if (s_full) {
                 if (threadIdx.x == 0) oversize[atomicAdd(&work->n_oversize, 1ull)] = (uint32_t)ti;
+            } else if constexpr (AGG) {
+                probe_smem_agg<W>(at, Sv, nsv, chk, acc, warp, nwarps, lane);
             } else {
-                if constexpr (FAST) {  // no aggregate, no checksum
-                    T *wq = (T *)(smem + walkq_offset(cap_max, 2 * W, W, false)) + (size_t)warp * 2 * kWalkQ;
-                    if (unique) probe_smem<W, 2, true>(tab, Sv, nsv, sink, warp, nwarps, lane, wq, wq + kWalkQ);
-                    else probe_smem<W, 2, false>(tab, Sv, nsv, sink, warp, nwarps, lane, wq, wq + kWalkQ);
-                } else {
-                const uint32_t gstride = nwarps * 32 * U;
-                Vec cur[U], nxt[U];
-                uint32_t g = warp * 32 * U;
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const uint32_t rel = g + u * 32 + lane;
-                    if (rel < nsv) cur[u] = ld_stream(Sv + rel);
-                }
-                for (; g < nsv; g += gstride) {
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const uint32_t rel = g + gstride + u * 32 + lane;
-                        if (rel < nsv) nxt[u] = ld_stream(Sv + rel);
-                    }
-                    T k[IT], r[IT];
-                    bool val[IT];
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const bool in = g + u * 32 + lane < nsv;
-                        if constexpr (W == 4) {
-                            k[2 * u] = cur[u].x; r[2 * u] = cur[u].y; k[2 * u + 1] = cur[u].z; r[2 * u + 1] = cur[u].w;
-                            val[2 * u] = in;
-                            val[2 * u + 1] = in;
-                        } else {
-                            k[u] = cur[u].x; r[u] = cur[u].y;
-                            val[u] = in;
-                        }
-                    }
-                    if constexpr (AGG) {
-                        // home buckets of all items first; no partition filter: a padding
-                        // tuple's key hashes to another partition, so it matches no slot
-                        uint32_t home[IT];
-                        T kb[IT][AG];
-#pragma unroll
-                        for (int i = 0; i < IT; ++i) {
-                            home[i] = part_bucket<W>(k[i], at.nb);
-#pragma unroll
-                            for (uint32_t q = 0; q < AG; ++q) kb[i][q] = at.empty;
-                            if (val[i]) at.ld(home[i], kb[i]);
-                        }
-#pragma unroll
-                        for (int i = 0; i < IT; ++i) {
-                            uint32_t mm = 0;
-                            bool e = false;
-#pragma unroll
-                            for (uint32_t q = 0; q < AG; ++q) {
-                                mm |= (uint32_t)(kb[i][q] == k[i]) << q;
-                                e |= kb[i][q] == at.empty;
-                            }
-                            // (a lane past the slice's end holds a stale key: no slot)
-                            uint32_t sl = val[i] && mm ? home[i] * AG + (uint32_t)(__ffs(mm) - 1) : ~0u;
-                            if (val[i] && !mm && !e && at.overflowed(home[i]))  // the run continues (rare)
-                                sl = at.find_from(k[i], home[i] + 1 == at.nb ? 0 : home[i] + 1);
-                            if (sl != ~0u) {
-                                const uint64_t n = at.cnt[sl];
-                                acc.cnt += n;
-                                if (chk) {
-                                    const uint64_t sa = at.suma[sl], bb = mix_b(r[i]);
-                                    acc.c0 += sa * bb;
-                                    acc.c1 += sa + n * bb;
-                                }
-                            }
-                        }
-                    } else {
-                        uint32_t cnt[IT], home[IT];
-                        T first[IT];
-                        bool live[IT];
-                        T kb[IT][G];
-                        // Home buckets of all items, key halves loaded together.  Padding
-                        // tuples need no filtering here: their keys hash to another
-                        // partition, so they equal neither a stored key nor the marker.
-#pragma unroll
-                        for (int i = 0; i < IT; ++i) {
-                            home[i] = part_bucket<W>(k[i], tab.nb);
-                            live[i] = val[i];
-#pragma unroll
-                            for (uint32_t q = 0; q < G; ++q) kb[i][q] = tab.empty;
-                            if (live[i]) tab.ld(home[i], 0, kb[i]);
-                        }
-#pragma unroll
-                        for (int i = 0; i < IT; ++i) {
-                            uint32_t mm = 0;
-                            bool e = false;
-#pragma unroll
-                            for (uint32_t q = 0; q < G; ++q) {
-                                mm |= (uint32_t)(kb[i][q] == k[i]) << q;
-                                e |= kb[i][q] == tab.empty;
-                            }
-                            uint32_t c = 0;
-                            T f = 0;
-                            if (live[i] && mm) {
-                                T rid[G];
-                                tab.ld(home[i], 1, rid);
-                                f = rid[G - 1];
-#pragma unroll
-                                for (int q = (int)G - 2; q >= 0; --q)
-                                    if ((mm >> q) & 1u) f = rid[q];
-                                c = __popc(mm);
-                            }
-                            if (live[i] && !e && tab.overflowed(home[i])) {  // the run continues (rare)
-                                const uint32_t nx = home[i] + 1 == tab.nb ? 0 : home[i] + 1;
-                                T f2 = 0;
-                                const uint32_t c2 = soa_lookup<W>(tab, k[i], nx, &f2);
-                                if (c == 0) f = f2;
-                                c += c2;
-                            }
-                            if (chk && c) {
-                                const uint64_t bs = mix_b(r[i]);
-                                soa_visit<W>(tab, k[i], home[i], [&](T rid) {
-                                    const uint64_t a = mix_a(rid);
-                                    acc.c0 += a * bs;
-                                    acc.c1 += a + bs;
-                                });
-                            }
-                            cnt[i] = c;
-                            first[i] = f;
-                        }
-                        sink.template append_group<IT>(cnt, first, r);
-                        // several matches: the whole warp walks each such key's run
-#pragma unroll
-                        for (int i = 0; i < IT; ++i) {
-                            unsigned multi = __ballot_sync(0xffffffffu, cnt[i] > 1);
-                            while (multi) {
-                                const int L = __ffs(multi) - 1;
-                                multi &= multi - 1;
-                                const T kk = __shfl_sync(0xffffffffu, k[i], L);
-                                const T ss = __shfl_sync(0xffffffffu, r[i], L);
-                                const uint32_t hh = __shfl_sync(0xffffffffu, home[i], L);
-                                soa_coop_emit<W>(tab, kk, ss, hh, sink);
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int u = 0; u < U; ++u) cur[u] = nxt[u];
-                }
-                }
+                T *wq = (T *)(smem + walkq_offset(cap_max, 2 * W, W, false)) + (size_t)warp * 2 * kWalkQ;
+                if (unique) probe_smem<W, 2, true>(tab, Sv, nsv, sink, warp, nwarps, lane, wq, wq + kWalkQ);
+                else probe_smem<W, 2, false>(tab, Sv, nsv, sink, warp, nwarps, lane, wq, wq + kWalkQ);
             }
         }
-        if constexpr (!FAST) flush_acc(jc, acc, AGG);
-        if constexpr (!AGG) sink.end_task();
+        if constexpr (AGG) {
+            flush_acc(jc, acc, true);
+        } else if constexpr (Sink::kCheck) {
+            flush_acc(jc, sink.acc, false);
+            sink.acc = ProbeAcc();
+        }
         if (warp == 0) {
             unsigned long long n = idx;
             if (idx == kNone) {
@@ -2000,10 +1850,10 @@ hj_status partition_join(hj_ctx *c, int width, int agg, const PartTask *tasks, u
     uint64_t want = (uint64_t)(3.0 * (mean + 6.0 * __builtin_sqrt(mean + 1.0) + 64.0));
     want = (want + 127) / 128 * 128;
     const uint64_t bitmap_bytes = 4096;
-    // the fast probe (no aggregate, no checksum) adds each warp's walk queue, output
-    // staged in shared memory its buffer, within what the shape's CTAs per SM can have
+    // the pair join adds each warp's walk queue, and staged output its buffer when that is in
+    // shared memory, within what the shape's CTAs per SM can have
     const uint64_t warps = (uint64_t)(cfg.nt / 32), total_max = join_ctas(cfg.nt) == 2 ? (112ull << 10) : (222ull << 10);
-    const uint64_t queues = !agg && !checksum ? warps * kWalkQ * 2 * width : 0;
+    const uint64_t queues = agg ? 0 : warps * kWalkQ * 2 * width;
     auto slots_beside = [&](uint64_t extra) {
         const uint64_t budget = std::min<uint64_t>(cfg.smem_limit + extra, total_max) - extra;
         return agg ? (budget - bitmap_bytes) / slot_bytes / 128 * 128
@@ -2026,39 +1876,35 @@ hj_status partition_join(hj_ctx *c, int width, int agg, const PartTask *tasks, u
     if (grid > ntasks) grid = (unsigned)ntasks;
     DevBuf gstage(c);  // (freed in stream order after the launch)
     if (in_global) HJ_TRY(gstage.alloc((uint64_t)grid * warps * kJoinStageBytes));
-#define HJ_PJ(WW, AA, NT, SK, FF)                                                                                     \
+#define HJ_PJ(WW, AA, NT, SK)                                                                                         \
     do {                                                                                                              \
-        auto kern = partition_join_kernel<WW, AA, NT, SK<WW>, FF>;                                                    \
+        auto kern = partition_join_kernel<WW, AA, NT, SK<WW>>;                                                        \
         HJ_TRY(allow_max_smem(c, (const void *)kern));                                                                \
         HJ_LAUNCH(c, "partition_join", kern, grid, NT, smem, tasks, ntasks, lead, slots, c->d_ctr, (uint32_t)cap_max, \
                   ra, oversize, checksum, (uint32_t)(smem - stage_bytes), gstage.p);                                  \
     } while (0)
-#define HJ_PJ_NT(WW, AA, SK, FF)                                             \
-    do {                                                                     \
-        if (join_ctas(cfg.nt) == 2) HJ_PJ(WW, AA, (AA ? 512 : 320), SK, FF); \
-        else HJ_PJ(WW, AA, (AA ? 1024 : 640), SK, FF);                       \
+#define HJ_PJ_NT(WW, AA, SK)                                             \
+    do {                                                                 \
+        if (join_ctas(cfg.nt) == 2) HJ_PJ(WW, AA, (AA ? 512 : 320), SK); \
+        else HJ_PJ(WW, AA, (AA ? 1024 : 640), SK);                       \
     } while (0)
-#define HJ_PJ_F(WW, SK)                                          \
-    do {                                                         \
-        if (checksum) HJ_PJ_NT(WW, false, SK, false);            \
-        else HJ_PJ_NT(WW, false, SK, true);                      \
-    } while (0)
-#define HJ_PJ_SK(WW)                                                             \
-    do {                                                                         \
-        if (!staged) HJ_PJ_F(WW, ChunkSink);                                     \
-        else if (!in_global) HJ_PJ_F(WW, WarpStageSink);                         \
-        else if (checksum) HJ_PJ(WW, false, 640, GlobalStageSink, false);        \
-        else HJ_PJ(WW, false, 640, GlobalStageSink, true);                       \
+#define HJ_PJ_SK(WW)                                                     \
+    do {                                                                 \
+        if (!staged && checksum) HJ_PJ_NT(WW, false, ChunkCheckSink);    \
+        else if (!staged) HJ_PJ_NT(WW, false, ChunkSink);                \
+        else if (in_global && checksum) HJ_PJ(WW, false, 640, GlobalStageCheckSink); \
+        else if (in_global) HJ_PJ(WW, false, 640, GlobalStageSink);      \
+        else if (checksum) HJ_PJ_NT(WW, false, WarpStageCheckSink);      \
+        else HJ_PJ_NT(WW, false, WarpStageSink);                         \
     } while (0)
     if (width == 4) {
-        if (agg) HJ_PJ_NT(4, true, ChunkSink, false); else HJ_PJ_SK(4);
+        if (agg) HJ_PJ_NT(4, true, ChunkSink); else HJ_PJ_SK(4);
     } else {
-        if (agg) HJ_PJ_NT(8, true, ChunkSink, false); else HJ_PJ_SK(8);
+        if (agg) HJ_PJ_NT(8, true, ChunkSink); else HJ_PJ_SK(8);
     }
 #undef HJ_PJ
 #undef HJ_PJ_NT
 #undef HJ_PJ_SK
-#undef HJ_PJ_F
     return HJ_OK;
 }
 

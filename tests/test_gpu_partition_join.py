@@ -89,6 +89,23 @@ def test_runs_of_repeated_keys(hjm, ctx, width, copies):
     _check(hjm, ctx, _rel(rng.permutation(keys), width), _rel(sk, width), radix_bits=1)
 
 
+@pytest.mark.parametrize("cap", [0, 700])
+@pytest.mark.parametrize("copies", [1, 2, 7, 40])
+@pytest.mark.parametrize("width", [4, 8])
+def test_pairs_with_checksums(hjm, ctx, width, copies, cap):
+    # the sums are taken where the pairs are appended, of pairs that pass the buffer too
+    rng = np.random.default_rng(copies)
+    n = 3000
+    r = _rel(rng.permutation(n) // copies + 1, width)
+    s = _rel(rng.integers(1, 2 * n // copies, 4 * n + 1), width)
+    res = hjm.hj_join(ctx, _gpu(r), _gpu(s), algo=hjm.HJ_ALGO_PHJ, radix_bits=2, passes=1, checksum=True,
+                      out_capacity=cap)
+    got = res.pairs_numpy().astype(np.uint64)
+    assert (res.count, *res.checksum) == oracle.join_aggregate(r, s)
+    res.free()
+    assert np.array_equal(oracle.sorted_pairs(got[:, 0], got[:, 1]), oracle.sorted_pairs(*oracle.hash_join(r, s)))
+
+
 @pytest.mark.parametrize("ns", [1280, 1281, 1279, 2559, 2600, 5120 + 3])
 @pytest.mark.parametrize("width", [4, 8])
 def test_slices_around_whole_groups(hjm, ctx, width, ns):
