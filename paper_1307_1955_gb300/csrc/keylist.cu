@@ -187,16 +187,22 @@ hj_status scan_entries(hj_ctx *c, Src src, Dst dst, uint64_t n, uint64_t *total_
 __device__ __forceinline__ unsigned lanes_lt() { return (1u << (threadIdx.x & 31)) - 1u; }
 
 constexpr uint64_t kGuessWalk = 64;
-// Heavy hitters a CTA lists: up to kHot keys that filled several lanes of a warp, found
-// in every kLookEvery-th of its tiles (comparing all lanes' keys costs 62 cycles per
-// warp, comparing with the listed ones a few).  Lanes of a warp that hold a listed key
-// add to its entry in shared memory together.
+// Heavy hitters a CTA lists: up to kHot keys that filled several lanes of a warp.  Lanes of
+// a warp that hold a listed key add to its entry in shared memory together.  Keys that are
+// not listed are compared with all lanes' in every kLookEvery-th of the CTA's tiles (62
+// cycles per warp), in the others with those of the first kLeads lanes that hold different
+// ones (a few): rows in the order of their keys, or of many heavy keys, never stay with what
+// a CTA listed, and an atomic per row on one address is what to avoid.  4.2e6 rows, 16 keys
+// of 1 % each, sorted: count 222 us comparing all lanes in every tile, 429 in every eighth
+// only, 224 like this.
 constexpr int kHot = 8;
 constexpr uint32_t kLookEvery = 8;
+constexpr int kLeads = 2;
 
-// Entry of key k among the listed keys (a free one taken), or -1.
+// Entry taken for key k, which was not listed a moment ago, or -1 if the list is full.
 template <int W> __device__ __forceinline__ int hot_entry(typename Tup<W>::U *hk, typename Tup<W>::U k) {
     using U = typename Tup<W>::U;
+    if (((volatile U *)hk)[kHot - 1] != Tup<W>::kAllOnes) return -1;
 #pragma unroll 1
     for (int j = 0; j < kHot; ++j) {
         const U cur = ((volatile U *)hk)[j];
@@ -211,14 +217,18 @@ template <int W> __device__ __forceinline__ int hot_entry(typename Tup<W>::U *hk
 
 // Adds m to key k's count, inserting the key (CAS on the key); returns 1 if this
 // call inserted it.  A walk that ends without a slot gives up a first table
-// (guess: *nkeys is pushed past any limit) or flags a full one.
+// (key_limit: *nkeys is pushed past it) or flags a full one.
 template <int W>
 __device__ __forceinline__ unsigned kl_add(AggSlot<W> *slots, uint64_t cap, typename Tup<W>::U k, uint64_t h,
-                                           unsigned m, bool guess, unsigned long long *nkeys, hj_counters *ctr) {
+                                           unsigned m, uint64_t key_limit, unsigned long long *nkeys,
+                                           hj_counters *ctr) {
     using U = typename Tup<W>::U;
+    const bool guess = key_limit != ~0ull;
     const uint64_t walk = guess && cap > kGuessWalk ? kGuessWalk : cap;
     uint64_t b = bucket_of<W>(h, cap);
     for (uint64_t it = 0; it < walk; ++it) {
+        // (a table that is filling up past its limit has long walks)
+        if (guess && it % 16 == 15 && *(volatile unsigned long long *)nkeys > key_limit) return 0;
         U old = *(volatile U *)&slots[b].key;
         if (old == Tup<W>::kAllOnes) old = cas_key<W>((U *)&slots[b].key, Tup<W>::kAllOnes, k);
         if (old == Tup<W>::kAllOnes || old == k) {
@@ -254,13 +264,36 @@ __device__ __forceinline__ int listed_key(const typename Tup<W>::U *hk, typename
     return at;
 }
 
+// The lanes that hold this lane's key (0 unless `on`): of all keys in every kLookEvery-th
+// tile, otherwise of the keys of the first kLeads lanes that are on and differ, each other
+// lane by itself.  All lanes call.
+template <int W> __device__ __forceinline__ unsigned same_key(typename Tup<W>::U k, bool on, bool look) {
+    unsigned left = __ballot_sync(0xffffffffu, on);
+    if (look) {
+        const unsigned g = __match_any_sync(0xffffffffu, k) & left;
+        return on ? g : 0u;
+    }
+    unsigned g = on ? 1u << (threadIdx.x & 31) : 0u;
+#pragma unroll
+    for (int i = 0; i < kLeads; ++i) {
+        if (!left) break;
+        const typename Tup<W>::U h = __shfl_sync(0xffffffffu, k, __ffs(left) - 1);
+        const unsigned m = __ballot_sync(0xffffffffu, on && k == h);
+        if (on && k == h) g = m;
+        left &= ~m;
+    }
+    return g;
+}
+
 // Step 1: every kept key in the table, its count added.  Each key inserted counts
 // in *nkeys; with a first table sized for fewer distinct keys than rows
-// (key_limit = half its slots) the CTAs stop after the tile in which they pass the
-// limit, walks end after kGuessWalk slots (at load <= 1/2 a longer one gives the table
-// up too), and the host builds again at full size.  What bounds it: one pass over R
-// (4.2e6 rows of which all but 6e3 hold one key 107 us with every lane group looking at
-// *nkeys, matching all lanes and adding per tile).
+// (key_limit = half its slots) warps stop as soon as they pass the limit and CTAs at the
+// end of their tile, walks end after kGuessWalk slots (at load <= 1/2 a longer one gives
+// the table up too) or when they see the limit passed, and the host builds again at full
+// size.  What bounds it: one pass over R (4.2e6 rows of which all but 6e3 hold one key
+// 107 us with every lane group looking at *nkeys, matching all lanes and adding per tile,
+// 28 like this; 3.5e6 rows, 400 keys of 4200 rows and 2e6 others 111 us and 116, and
+// 181 with every CTA ending its tile in the table that it fills up).
 template <int W>
 __global__ void __launch_bounds__(256) kl_count(const void *R, uint64_t n, AggSlot<W> *slots, uint64_t cap,
                                                 TableSide *side, hj_counters *ctr, PartFilter pf,
@@ -285,7 +318,6 @@ __global__ void __launch_bounds__(256) kl_count(const void *R, uint64_t n, AggSl
         const uint64_t v = tile * blockDim.x + threadIdx.x;
         U k[2] = {0, 0}, r[2] = {0, 0};
         if (v < nv) kl_load<W>(R, v, n, k, r);
-        unsigned fresh = 0;  // keys this lane inserted (first table only)
 #pragma unroll
         for (int e = 0; e < PV; ++e) {
             const uint64_t h = key_hash<W>(k[e]);
@@ -296,24 +328,21 @@ __global__ void __launch_bounds__(256) kl_count(const void *R, uint64_t n, AggSl
             const int at = listed_key<W>(hk, k[e], ok && !ones, &hm);
             if (at >= 0 && !(hm & lanes_lt())) atomicAdd(&hc[at], (unsigned)__popc(hm));
             const bool rest = ok && !ones && at < 0;
-            unsigned m = 1;  // tuples this lane counts
-            if (round % kLookEvery == 0) {
-                const unsigned g = __match_any_sync(0xffffffffu, k[e]) & __ballot_sync(0xffffffffu, rest);
-                m = rest && !(g & lanes_lt()) ? __popc(g) : 0;  // the group's lowest lane, for all
+            const unsigned g = same_key<W>(k[e], rest, round % kLookEvery == 0);
+            unsigned fresh = 0;  // keys this lane inserted
+            if (rest && !(g & lanes_lt())) {  // the group's lowest lane counts for all
+                const unsigned m = __popc(g);
+                const int j = m > 1 ? hot_entry<W>(hk, k[e]) : -1;
+                if (j >= 0) atomicAdd(&hc[j], m);
+                else fresh = kl_add<W>(slots, cap, k[e], h, m, key_limit, nkeys, ctr);
             }
-            if (!rest || !m) continue;
-            if (m > 1) {
-                const int j = hot_entry<W>(hk, k[e]);
-                if (j >= 0) {
-                    atomicAdd(&hc[j], m);
-                    continue;
-                }
-            }
-            fresh += kl_add<W>(slots, cap, k[e], h, m, guess, nkeys, ctr);
+            if (!guess) continue;
+            const unsigned tot = __popc(__ballot_sync(0xffffffffu, fresh));
+            unsigned over = 0;
+            if (lane == 0 && tot) over = atomicAdd(nkeys, (unsigned long long)tot) + tot > key_limit;
+            if (__shfl_sync(0xffffffffu, over, 0)) break;
         }
         if (guess) {  // (the warp is converged again here)
-            const unsigned tot = __reduce_add_sync(0xffffffffu, fresh);
-            if (lane == 0 && tot) atomicAdd(nkeys, (unsigned long long)tot);
             if (threadIdx.x == 0) stop = *(volatile unsigned long long *)nkeys > key_limit;
             __syncthreads();
             if (stop) return;  // given up: the host builds again
@@ -324,7 +353,7 @@ __global__ void __launch_bounds__(256) kl_count(const void *R, uint64_t n, AggSl
     if (threadIdx.x < kHot) {  // the listed keys: one add each
         const U hkey = hk[threadIdx.x];
         if (hkey != Tup<W>::kAllOnes && hc[threadIdx.x])
-            if (kl_add<W>(slots, cap, hkey, key_hash<W>(hkey), hc[threadIdx.x], guess, nkeys, ctr) && guess)
+            if (kl_add<W>(slots, cap, hkey, key_hash<W>(hkey), hc[threadIdx.x], key_limit, nkeys, ctr) && guess)
                 atomicAdd(nkeys, 1ull);
     }
 }
@@ -363,11 +392,8 @@ __global__ void __launch_bounds__(256) kl_scatter(const void *R, uint64_t n, Agg
             unsigned g = 0;
             int j = listed_key<W>(hk, k[e], ok && !ones, &g);
             const bool known = j >= 0;
-            if (!known) g = ok ? 1u << lane : 0u;
-            if (round % kLookEvery == 0) {
-                const unsigned same = __match_any_sync(0xffffffffu, k[e]) & __ballot_sync(0xffffffffu, ok && !known);
-                if (!known) g = ok ? same : 0u;
-            }
+            const unsigned same = same_key<W>(k[e], ok && !known, round % kLookEvery == 0);
+            if (!known) g = same;
             const int leader = g ? __ffs(g) - 1 : 0;
             // the leader claims the group's places: [at, at + popc(g)) of the key's
             // list, or of the all-ones keys' list counted down from the array's end,

@@ -169,3 +169,31 @@ def test_heavy_hitter_full_size_count(hjm, ctx):
         m = hjm.hj_join(ctx, R, S, checksum=True, algo=hjm.HJ_ALGO_PHJ)
         assert (m.count, *m.checksum) == agg
         m.free()
+
+
+@pytest.mark.parametrize("order", ["random", "sorted", "runs"])
+@pytest.mark.parametrize("n", [150_001, 600_001])
+@pytest.mark.parametrize("width", [4, 8])
+def test_more_heavy_keys_than_a_cta_lists(hjm, ctx, width, n, order):
+    # 40 heavy keys of 1500 rows and the all-ones key, the other keys once (more of them than
+    # the first table takes at the larger size) or, "runs", up to 7 times in a row; R in random
+    # order, or sorted, so that each tile meets other heavy keys than the ones before
+    dt = np.uint32 if width == 4 else np.uint64
+    rng = np.random.default_rng(n + width)
+    ones = np.uint64(2 ** (8 * width) - 1)
+    rk = np.concatenate([np.repeat(np.arange(1, 41, dtype=np.uint64) * np.uint64(5_000_000), 1500),
+                         np.full(900, ones, np.uint64)])
+    rest = np.arange(n - len(rk), dtype=np.uint64) // np.uint64(7 if order == "runs" else 1) * np.uint64(11) + np.uint64(3)
+    rk = np.concatenate([rk, rest])
+    rk = rng.permutation(rk) if order == "random" else np.sort(rk)
+    sk = np.concatenate([rng.choice(rest, 20_000), np.arange(1, 41, dtype=np.uint64) * np.uint64(5_000_000),
+                         np.full(3, ones, np.uint64), np.arange(9_000_001, 9_002_001, dtype=np.uint64)])
+
+    def rel(k):
+        a = np.stack([k.astype(dt), np.arange(len(k), dtype=dt)], 1)
+        return torch.from_numpy(a.view(np.int32 if width == 4 else np.int64)).to(DEV)
+
+    R, S = rel(rk), rel(rng.permutation(sk))
+    want, agg = _want(R, S)
+    _check(hjm, ctx, R, S, want, agg, algo=hjm.HJ_ALGO_SHJ)
+    _check(hjm, ctx, R, S, want, agg, algo=hjm.HJ_ALGO_PHJ, radix_bits=6)
