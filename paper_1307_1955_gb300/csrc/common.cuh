@@ -217,6 +217,16 @@ struct TableSide {
     unsigned long long repeats;     // pair table: not 0 unless every key in it is another (and not all ones)
 };
 
+// Status bits written by kernels into the context's device status word.
+enum : int {
+    kStatusTableFull = 1,
+    kStatusTimeout = 2,
+    kStatusBadInput = 4,
+    kStatusRecords = 8,    // a chunk-record area was too small
+    kStatusCompact = 16,   // device compaction found holes and tail pairs of different sizes
+    kStatusLongRun = 32,   // a pair-table insert walked past kMaxPairWalk slots (heavily repeated keys)
+};
+
 // Longest walk of a pair-table insert.  Unique keys at load factor <= 1/2 never
 // come near it; a key with many copies does (every copy walks past the earlier
 // ones), and the join then takes a key-list table instead.
@@ -258,11 +268,15 @@ template <> __device__ __forceinline__ uint32_t pair_bucket<8>(uint64_t h, uint3
 // table had no free slot (cannot happen while it has more slots than tuples) or the
 // walk passed max_walk slots.  Sets *repeat for the all-ones key and for a key met
 // on the way: slots are tried in the run's order and are never emptied, so of two
-// tuples with one key the later one passes the earlier one's slot and sees it.
+// tuples with one key the later one passes the earlier one's slot and sees it.  With
+// `status`, a walk also ends (false) once it sees kStatusLongRun there: the table is
+// given up, and the walks of the heavy keys' other rows would be for nothing (4.2e6 u64
+// rows, 64 sorted keys of 0.5 % each: build 38 -> 7.8 ms).
 template <int W>
 __device__ __forceinline__ bool pair_insert(typename PairSlot<W>::S *slots, uint32_t nb, TableSide *side,
                                             typename Tup<W>::U k, typename Tup<W>::U r, uint64_t h, bool *repeat,
-                                            uint64_t max_walk = kMaxPairWalk) {
+                                            uint64_t max_walk = kMaxPairWalk,
+                                            const unsigned long long *status = nullptr) {
     using PS = PairSlot<W>;
     constexpr uint32_t G = kBucketSlots<W>;
     if (k == Tup<W>::kAllOnes) {
@@ -276,6 +290,7 @@ __device__ __forceinline__ bool pair_insert(typename PairSlot<W>::S *slots, uint
     uint32_t b = pair_bucket<W>(h, nb);
     const uint32_t lim = (uint64_t)nb * G < max_walk ? nb : (uint32_t)(max_walk / G);
     for (uint32_t it = 0; it < lim; ++it) {
+        if (status && it % 16 == 15 && (*(const volatile unsigned long long *)status & kStatusLongRun)) return false;
 #pragma unroll
         for (uint32_t q = 0; q < G; ++q) {
             const typename PS::S o = PS::claim(&slots[(uint64_t)b * G + q], v);
@@ -413,15 +428,5 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
         if (mbar_try_wait(bar, parity)) return true;
     return false;
 }
-
-// Status bits written by kernels into the context's device status word.
-enum : int {
-    kStatusTableFull = 1,
-    kStatusTimeout = 2,
-    kStatusBadInput = 4,
-    kStatusRecords = 8,    // a chunk-record area was too small
-    kStatusCompact = 16,   // device compaction found holes and tail pairs of different sizes
-    kStatusLongRun = 32,   // a pair-table insert walked past kMaxPairWalk slots (heavily repeated keys)
-};
 
 }  // namespace hj

@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(256) table_build_kernel(const void *R, uint64_
             if (!pf.keep(h)) continue;
             const bool ok = AGG ? agg_insert<W>((AggSlot<W> *)slots, cap, side, g.key(e), mix_a(g.rid(e)), h)
                                 : pair_insert<W>((typename PairSlot<W>::S *)slots, (uint32_t)(cap / kBucketSlots<W>),
-                                                 side, g.key(e), g.rid(e), h, &repeat);
+                                                 side, g.key(e), g.rid(e), h, &repeat, kMaxPairWalk, &ctr->status);
             if (!ok) atomicOr(&ctr->status, (unsigned long long)(AGG || cap <= kMaxPairWalk ? kStatusTableFull
                                                                                          : kStatusLongRun));
         }
