@@ -556,10 +556,20 @@ hj_status join_phj(hj_ctx *c, const hj_rel *R, const hj_rel *S, const hj_opts &o
 //
 // A chunk whose pairs overflow its buffer, or that needed the global-table
 // fallback, is joined again on its own afterwards.
-// S rows per chunk: the link is idle while the last chunk joins and its pairs go home
-// alone, and a copy of 64 MB still runs at 95 % of its rate (5e6 x 4e7 tuples 2.25 ms,
-// 2.28 at 2^22 rows, 2.40 at 2^24; the copies alone take 1.99).
+// S rows per chunk.  The link is idle while the last chunk joins and its pairs go home
+// alone, and a copy of 64 MB still runs at 95 % of its rate: 2^23 rows (5e6 x 4e7 tuples 2.25
+// ms, 2.28 at 2^22 rows, 2.40 at 2^24; the copies alone take 1.99).  But every chunk builds
+// the tables of all of R again: where that takes as long as a chunk's copy, twice as many
+// rows (4-byte pairs: 2^24 x 2^28 tuples 13.1 ms against 13.2, 2^25 x 2^27 11.0 against 9.1;
+// counts, whose aggregate tables take longer: 2^23 x 2^26 3.50 against 3.62, 1.2e7 x 2^26
+// 4.45 against 4.31, 2^24 x 2^28 17.0 against 12.5; 8-byte tuples take twice the time on
+// the link: counts of 2^24 x 2^26 8.0 against 8.4).  Two or three chunks hide less of it:
+// counts of 2^23 x 2^24 tuples 1.57 ms in two chunks, 1.38 in one piece.
 constexpr uint64_t kHostChunk = 1ull << 23;
+uint64_t host_chunk_rows(int width, bool mat, uint64_t nR, uint64_t nS) {
+    const uint64_t most = kHostChunk * (width / 4) * (mat ? 4 : nS >= 4 * kHostChunk ? 2 : 1) / 2;
+    return nR > most ? 2 * kHostChunk : kHostChunk;
+}
 
 struct PipeSet {
     explicit PipeSet(hj_ctx *c, int w) : sink(c, w), dS(c) {}
@@ -933,7 +943,7 @@ bool host_streamed_plan(hj_ctx *c, const hj_rel *Rh, const hj_rel *Sh, const hj_
         c->model_ready = true;
     }
     const bool mat = o.mode == HJ_MATERIALIZE;
-    for (uint64_t ch = kHostChunk; ch >= (1ull << 20); ch >>= 1) {
+    for (uint64_t ch = host_chunk_rows(Rh->width, mat, Rh->n, Sh->n); ch >= (1ull << 20); ch >>= 1) {
         const std::vector<PlanCand> pcs =
             plan_candidates(c->model, Rh->width, !mat, mat, Rh->n, std::min<uint64_t>(Sh->n, ch), HJ_ALGO_PHJ, 0, 1);
         if (pcs.empty() || pcs[0].passes != 1) return false;  // R needs two passes: no streamed plan
@@ -1094,6 +1104,7 @@ hj_status hj_join_host(hj_ctx *c, const hj_rel *Rh, const hj_rel *Sh, const hj_o
         hj_opts o = opts ? *opts : default_opts();
         int algo, bits, passes;
         choose_plan(c, Rh->width, o.mode, Rh->n, Sh->n, o.algo, o.radix_bits, o.passes, &algo, &bits, &passes);
+        const uint64_t chunk_rows = host_chunk_rows(Rh->width, o.mode == HJ_MATERIALIZE, Rh->n, Sh->n);
         bool pipe = algo == HJ_ALGO_PHJ && passes == 1;
         if (!pipe && o.algo == HJ_ALGO_AUTO && o.passes <= 0) {
             // the in-memory plan is SHJ or two passes; the chunked join is bound by
@@ -1105,17 +1116,17 @@ hj_status hj_join_host(hj_ctx *c, const hj_rel *Rh, const hj_rel *Sh, const hj_o
             }
             const bool mat = o.mode == HJ_MATERIALIZE;
             std::vector<PlanCand> pcs = plan_candidates(c->model, Rh->width, !mat, mat, Rh->n,
-                                                        std::min<uint64_t>(Sh->n, kHostChunk), HJ_ALGO_PHJ,
+                                                        std::min<uint64_t>(Sh->n, chunk_rows), HJ_ALGO_PHJ,
                                                         o.radix_bits, 1);
             if (!pcs.empty() && pcs[0].passes == 1) {
                 pipe = true;
                 bits = pcs[0].bits;
             }
         }
-        if (pipe && Sh->n >= 2 * kHostChunk && Rh->n < 0xFFFFFFFFull && o.mode >= HJ_COUNT &&
+        if (pipe && Sh->n >= 2 * chunk_rows && Rh->n < 0xFFFFFFFFull && o.mode >= HJ_COUNT &&
             o.mode <= HJ_MATERIALIZE) {
             *res = hj_result{};
-            return join_host_pipelined(c, Rh, Sh, o, bits, kHostChunk, pairs_host, pairs_host_cap, res);
+            return join_host_pipelined(c, Rh, Sh, o, bits, chunk_rows, pairs_host, pairs_host_cap, res);
         }
     }
     DevBuf dR(c), dS(c);

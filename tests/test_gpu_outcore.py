@@ -170,3 +170,27 @@ def test_host_join_chunk_overflowing_its_buffer_is_rejoined(hjm, ctx):
     assert np.array_equal(keys[got[:, 0]], sk[got[:, 1]])
     code = np.sort(got[:, 0].astype(np.uint64) << np.uint64(32) | got[:, 1].astype(np.uint64))
     assert not np.any(code[1:] == code[:-1])
+
+
+@pytest.mark.parametrize("nr,ns,joins,pairs_joins", [(1 << 16, (1 << 24) + 77, 3, 3), ((1 << 22) + 3, (1 << 24) + 77, 1, 3),
+                                                     ((1 << 23) + 1, (1 << 25) + 77, 3, 5)])
+def test_host_chunks_grow_with_the_build_side(hjm, ctx, nr, ns, joins, pairs_joins):
+    # chunks of 2^23 rows, or of 2^24 (in one piece below 2^25) where the tables of R, which
+    # every chunk builds again, take as long as a chunk's copy: in count modes from half as
+    # many build rows on as for pairs
+    rng = np.random.default_rng(nr)
+    r = np.stack([rng.permutation(nr).astype(np.uint32), np.arange(nr, dtype=np.uint32)], 1)
+    s = np.stack([rng.integers(0, 4 * nr, ns, dtype=np.uint32), np.arange(ns, dtype=np.uint32)], 1)
+    R, S = (torch.from_numpy(a.view(np.int32)).pin_memory() for a in (r, s))
+    want = oracle.join_aggregate(r, s)
+    out = torch.empty((want[0], 2), dtype=torch.int32).pin_memory()
+    for expect, kw in ((joins, {"mode": hjm.HJ_COUNT_CHECKSUM}), (pairs_joins, {"pairs_out": out, "checksum": True})):
+        hjm.prof_reset(ctx)
+        hjm.prof_enable(ctx, True)
+        try:
+            res = hjm.hj_join_host(ctx, R, S, algo=hjm.HJ_ALGO_PHJ, **kw)
+            launched = hjm.prof_read(ctx)
+        finally:
+            hjm.prof_enable(ctx, False)
+        assert (res.count, *res.checksum) == want
+        assert launched["partition_join"][0] == expect, launched
