@@ -945,7 +945,8 @@ bool host_streamed_plan(hj_ctx *c, const hj_rel *Rh, const hj_rel *Sh, const hj_
     const bool mat = o.mode == HJ_MATERIALIZE;
     for (uint64_t ch = host_chunk_rows(Rh->width, mat, Rh->n, Sh->n); ch >= (1ull << 20); ch >>= 1) {
         const std::vector<PlanCand> pcs =
-            plan_candidates(c->model, Rh->width, !mat, mat, Rh->n, std::min<uint64_t>(Sh->n, ch), HJ_ALGO_PHJ, 0, 1);
+            plan_candidates(c->model, join_kind(c, Rh->width, o.mode, o.flags), Rh->n, std::min<uint64_t>(Sh->n, ch),
+                            HJ_ALGO_PHJ, 0, 1);
         if (pcs.empty() || pcs[0].passes != 1) return false;  // R needs two passes: no streamed plan
         if (host_streamed_bytes(c, Rh->width, mat, Rh->n, ch, pcs[0].bits) <= device_bytes) {
             *chunk_rows = ch;
@@ -982,7 +983,8 @@ hj_status hj_join_coproc(hj_ctx *c, const hj_rel *R, const hj_rel *S, const hj_o
     if (o.radix_bits < 0 || o.radix_bits > 24) return set_err(c, HJ_E_INVALID, "radix bits %d > 24", o.radix_bits);
     *res = hj_result{};
     int algo, bits, passes;
-    choose_plan(c, R->width, o.mode, R->n, S->n, HJ_ALGO_PHJ, o.radix_bits, o.passes, &algo, &bits, &passes);
+    choose_plan(c, join_kind(c, R->width, o.mode, o.flags), R->n, S->n, HJ_ALGO_PHJ, o.radix_bits, o.passes, &algo,
+                &bits, &passes);
     int threads = cpu_threads;
     if (!threads) threads = (int)std::max(1u, std::thread::hardware_concurrency());
     return join_coproc(c, R, S, o, bits, passes, cpu_share, threads, res, times);
@@ -1076,7 +1078,8 @@ hj_status hj_join(hj_ctx *c, const hj_rel *R, const hj_rel *S, const hj_opts *op
     if (o.radix_bits < 0 || o.radix_bits > 24) return set_err(c, HJ_E_INVALID, "radix bits %d > 24", o.radix_bits);
     *res = hj_result{};
     int algo, bits, passes;
-    choose_plan(c, R->width, o.mode, R->n, S->n, o.algo, o.radix_bits, o.passes, &algo, &bits, &passes);
+    choose_plan(c, join_kind(c, R->width, o.mode, o.flags), R->n, S->n, o.algo, o.radix_bits, o.passes, &algo, &bits,
+                &passes);
     hj_status st = algo == HJ_ALGO_SHJ ? join_shj(c, R, S, o, res) : join_phj(c, R, S, o, bits, passes, res);
     return st;
 }
@@ -1103,7 +1106,8 @@ hj_status hj_join_host(hj_ctx *c, const hj_rel *Rh, const hj_rel *Sh, const hj_o
         // a large S: chunked, copies overlapping a one-pass PHJ
         hj_opts o = opts ? *opts : default_opts();
         int algo, bits, passes;
-        choose_plan(c, Rh->width, o.mode, Rh->n, Sh->n, o.algo, o.radix_bits, o.passes, &algo, &bits, &passes);
+        const JoinKind jk = join_kind(c, Rh->width, o.mode, o.flags);
+        choose_plan(c, jk, Rh->n, Sh->n, o.algo, o.radix_bits, o.passes, &algo, &bits, &passes);
         const uint64_t chunk_rows = host_chunk_rows(Rh->width, o.mode == HJ_MATERIALIZE, Rh->n, Sh->n);
         bool pipe = algo == HJ_ALGO_PHJ && passes == 1;
         if (!pipe && o.algo == HJ_ALGO_AUTO && o.passes <= 0) {
@@ -1114,10 +1118,8 @@ hj_status hj_join_host(hj_ctx *c, const hj_rel *Rh, const hj_rel *Sh, const hj_o
                 c->model = cost_model_for(c->device);
                 c->model_ready = true;
             }
-            const bool mat = o.mode == HJ_MATERIALIZE;
-            std::vector<PlanCand> pcs = plan_candidates(c->model, Rh->width, !mat, mat, Rh->n,
-                                                        std::min<uint64_t>(Sh->n, chunk_rows), HJ_ALGO_PHJ,
-                                                        o.radix_bits, 1);
+            std::vector<PlanCand> pcs = plan_candidates(c->model, jk, Rh->n, std::min<uint64_t>(Sh->n, chunk_rows),
+                                                        HJ_ALGO_PHJ, o.radix_bits, 1);
             if (!pcs.empty() && pcs[0].passes == 1) {
                 pipe = true;
                 bits = pcs[0].bits;

@@ -210,15 +210,25 @@ struct PlanCand {
     double sec;
 };
 CostModel cost_model_for(int device);
-double predict_seconds(const CostModel &m, int width, bool agg, bool mat, uint64_t nR, uint64_t nS, int algo,
-                       int bits, int passes, double *steps);
+// What a plan depends on besides the sizes.
+struct JoinKind {
+    int width;
+    bool agg;     // a count mode, not pairs
+    bool chk;     // pairs with checksums
+    bool budget;  // a context with a memory budget (smaller tables)
+    // SHJ joins with the whole build side in shared memory (small_join)
+    bool small(uint64_t nR) const { return !agg && !chk && nR <= small_join_rows(width); }
+};
+JoinKind join_kind(const hj_ctx *c, int width, int mode, uint64_t flags);
+double predict_seconds(const CostModel &m, const JoinKind &jk, uint64_t nR, uint64_t nS, int algo, int bits,
+                       int passes, double *steps);
 // Candidates allowed by the forced fields (0 = free), cheapest first.
-std::vector<PlanCand> plan_candidates(const CostModel &m, int width, bool agg, bool mat, uint64_t nR, uint64_t nS,
-                                      int algo, int bits, int passes);
-uint64_t plan_key(int width, bool agg, uint64_t nR, uint64_t nS);
+std::vector<PlanCand> plan_candidates(const CostModel &m, const JoinKind &jk, uint64_t nR, uint64_t nS, int algo,
+                                      int bits, int passes);
+uint64_t plan_key(const JoinKind &jk, uint64_t nR, uint64_t nS);
 // The plan hj_join runs: a tuned plan for the size class if any, else the model's.
-void choose_plan(hj_ctx *c, int width, int mode, uint64_t nR, uint64_t nS, int algo, int bits, int passes,
-                 int *a_out, int *b_out, int *g_out);
+void choose_plan(hj_ctx *c, const JoinKind &jk, uint64_t nR, uint64_t nS, int algo, int bits, int passes, int *a_out,
+                 int *b_out, int *g_out);
 
 // --------------------------------------------------------------- coexec.cu
 // Host threads join partition pairs 0 .. np - 1 of padded partitioned copies in

@@ -92,19 +92,24 @@ static double fit_tuples(int width, bool agg) {
     return (200.0 * 1024 - 4096) / slot / 2.0;
 }
 
-double predict_seconds(const CostModel &m, int width, bool agg, bool mat, uint64_t nR, uint64_t nS, int algo,
-                       int bits, int passes, double *steps) {
+JoinKind join_kind(const hj_ctx *c, int width, int mode, uint64_t flags) {
+    const bool agg = mode != HJ_MATERIALIZE;
+    return JoinKind{width, agg, !agg && (flags & HJ_FLAG_CHECKSUM) != 0, c && c->budget != 0};
+}
+
+double predict_seconds(const CostModel &m, const JoinKind &jk, uint64_t nR, uint64_t nS, int algo, int bits,
+                       int passes, double *steps) {
+    const int width = jk.width;
+    const bool agg = jk.agg, mat = !agg;
     const double t = 2.0 * width, o = 2.0 * width, ir = issue_rate(m), b = bw(m);
     const double n = (double)nR + (double)nS, M = mat ? (double)nS : 0.0;  // one match per probe tuple
     double s[4] = {0, 0, 0, 0};  // hist, scatter, join / build, probe
-    if (algo == HJ_ALGO_SHJ && mat && nR <= small_join_rows(width)) {
+    if (algo == HJ_ALGO_SHJ && jk.small(nR)) {
         s[3] = std::max((t * nS + o * M) / b, nS * kIptSmallProbe * (width == 4 ? 1.0 : 1.6) / ir) + kSmallFixedS;
     } else if (algo == HJ_ALGO_SHJ) {
-        // the table: a power of two at least twice R, or (pairs, up to twice L2) four
-        // slots per tuple; probes of what does not stay in L2 read a sector from HBM
-        const double slot = agg ? (width == 4 ? 16.0 : 32.0) : t, four = 4.0 * nR * slot;
-        const double table = !agg && four <= 256.0 * (1 << 20) ? four
-                                                               : std::exp2(std::ceil(std::log2(2.0 * nR + 1.0))) * slot;
+        // probes of what does not stay in L2 read a sector of the table from HBM
+        const double slot = agg ? (width == 4 ? 16.0 : 32.0) : t;
+        const double table = (double)table_slots(width, agg, nR, jk.budget) * slot;
         const double miss = std::max(0.0, 1.0 - kL2Table * m.l2_bytes / std::max(table, 1.0));
         const double rnd = b * kRandomFraction;
         const double probe = width == 4 ? kIptShjProbe4 : agg ? kIptShjAgg8 : kIptShjProbe8;
@@ -138,17 +143,16 @@ double predict_seconds(const CostModel &m, int width, bool agg, bool mat, uint64
     return s[0] + s[1] + s[2] + s[3];
 }
 
-std::vector<PlanCand> plan_candidates(const CostModel &m, int width, bool agg, bool mat, uint64_t nR, uint64_t nS,
-                                      int algo, int bits, int passes) {
+std::vector<PlanCand> plan_candidates(const CostModel &m, const JoinKind &jk, uint64_t nR, uint64_t nS, int algo,
+                                      int bits, int passes) {
     std::vector<PlanCand> out;
     auto add = [&](int a, int bb, int g) {
-        PlanCand pc{a, bb, g, predict_seconds(m, width, agg, mat, nR, nS, a, bb, g, nullptr)};
+        PlanCand pc{a, bb, g, predict_seconds(m, jk, nR, nS, a, bb, g, nullptr)};
         out.push_back(pc);
     };
-    // the SHJ table must stay well inside the device (it is 2^ceil(log2(2|R|+1)) slots)
     if (algo == HJ_ALGO_AUTO || algo == HJ_ALGO_SHJ) add(HJ_ALGO_SHJ, 0, 0);
     if (algo == HJ_ALGO_AUTO || algo == HJ_ALGO_PHJ) {
-        const double fit = fit_tuples(width, agg);
+        const double fit = fit_tuples(jk.width, jk.agg);
         for (int b = 1; b <= 24; ++b) {
             if (bits > 0 && b != bits) continue;
             // every partition table must fit: skip fan-outs whose mean partition plus
@@ -170,7 +174,7 @@ std::vector<PlanCand> plan_candidates(const CostModel &m, int width, bool agg, b
     return out;
 }
 
-uint64_t plan_key(int width, bool agg, uint64_t nR, uint64_t nS) {
+uint64_t plan_key(const JoinKind &jk, uint64_t nR, uint64_t nS) {
     auto lg = [](uint64_t x) {
         int l = 0;
         while (x > 1) {
@@ -179,14 +183,15 @@ uint64_t plan_key(int width, bool agg, uint64_t nR, uint64_t nS) {
         }
         return (uint64_t)l;
     };
-    return ((uint64_t)width << 40) | ((uint64_t)agg << 32) | (lg(nR + 1) << 8) | lg(nS + 1);
+    // (SHJ is another join on either side of small(): a class of its own)
+    return ((uint64_t)jk.width << 40) | ((uint64_t)jk.small(nR) << 33) | ((uint64_t)jk.agg << 32) | (lg(nR + 1) << 8) |
+           lg(nS + 1);
 }
 
-void choose_plan(hj_ctx *c, int width, int mode, uint64_t nR, uint64_t nS, int algo, int bits, int passes,
-                 int *a_out, int *b_out, int *g_out) {
-    const bool agg = mode != HJ_MATERIALIZE, mat = mode == HJ_MATERIALIZE;
+void choose_plan(hj_ctx *c, const JoinKind &jk, uint64_t nR, uint64_t nS, int algo, int bits, int passes, int *a_out,
+                 int *b_out, int *g_out) {
     if (algo == HJ_ALGO_AUTO && bits <= 0 && passes <= 0 && c) {
-        auto it = c->tuned.find(plan_key(width, agg, nR, nS));
+        auto it = c->tuned.find(plan_key(jk, nR, nS));
         if (it != c->tuned.end()) {
             *a_out = it->second.algo;
             *b_out = it->second.bits;
@@ -204,7 +209,7 @@ void choose_plan(hj_ctx *c, int width, int mode, uint64_t nR, uint64_t nS, int a
         c->model = cost_model_for(c->device);
         c->model_ready = true;
     }
-    std::vector<PlanCand> pcs = plan_candidates(c->model, width, agg, mat, nR, nS, algo, bits, passes);
+    std::vector<PlanCand> pcs = plan_candidates(c->model, jk, nR, nS, algo, bits, passes);
     if (pcs.empty()) {  // forced shape the filters rejected: honour it
         *a_out = HJ_ALGO_PHJ;
         *b_out = bits > 0 ? bits : 12;
@@ -229,13 +234,13 @@ hj_status hj_plan(hj_ctx *c, const hj_rel *R, const hj_rel *S, const hj_opts *op
     hj_opts o{};
     o.mode = HJ_MATERIALIZE;
     if (opts) o = *opts;
-    const bool agg = o.mode != HJ_MATERIALIZE, mat = o.mode == HJ_MATERIALIZE;
+    const JoinKind jk = join_kind(c, R->width, o.mode, o.flags);
     CostModel m = c ? cost_model_for(c->device) : CostModel{};
     int a = o.algo, b = o.radix_bits, g = o.passes;
     if (c) {
-        choose_plan(c, R->width, o.mode, R->n, S->n, o.algo, o.radix_bits, o.passes, &a, &b, &g);
+        choose_plan(c, jk, R->n, S->n, o.algo, o.radix_bits, o.passes, &a, &b, &g);
     } else {
-        std::vector<PlanCand> pcs = plan_candidates(m, R->width, agg, mat, R->n, S->n, o.algo, o.radix_bits, o.passes);
+        std::vector<PlanCand> pcs = plan_candidates(m, jk, R->n, S->n, o.algo, o.radix_bits, o.passes);
         if (pcs.empty()) return HJ_E_INVALID;
         a = pcs[0].algo;
         b = pcs[0].bits;
@@ -246,7 +251,7 @@ hj_status hj_plan(hj_ctx *c, const hj_rel *R, const hj_rel *S, const hj_opts *op
     out->radix_bits = a == HJ_ALGO_PHJ ? b : 0;
     out->passes = a == HJ_ALGO_PHJ ? g : 0;
     double st[4];
-    out->predicted_ms = 1e3 * predict_seconds(m, R->width, agg, mat, R->n, S->n, a, b, g, st);
+    out->predicted_ms = 1e3 * predict_seconds(m, jk, R->n, S->n, a, b, g, st);
     for (int i = 0; i < 4; ++i) out->step_ms[i] = 1e3 * st[i];
     out->measured_ms = -1.0;
     return HJ_OK;
@@ -260,12 +265,12 @@ hj_status hj_tune(hj_ctx *c, const hj_rel *R, const hj_rel *S, const hj_opts *op
     o.mode = HJ_MATERIALIZE;
     if (opts) o = *opts;
     if (top_k <= 0) top_k = 4;
-    const bool agg = o.mode != HJ_MATERIALIZE, mat = o.mode == HJ_MATERIALIZE;
+    const JoinKind jk = join_kind(c, R->width, o.mode, o.flags);
     if (!c->model_ready) {
         c->model = cost_model_for(c->device);
         c->model_ready = true;
     }
-    std::vector<PlanCand> pcs = plan_candidates(c->model, R->width, agg, mat, R->n, S->n, HJ_ALGO_AUTO, 0, 0);
+    std::vector<PlanCand> pcs = plan_candidates(c->model, jk, R->n, S->n, HJ_ALGO_AUTO, 0, 0);
     if ((int)pcs.size() > top_k) pcs.resize(top_k);
     if (pcs.empty()) return set_err(c, HJ_E_UNSUPPORTED, "no plan candidate");
     cudaEvent_t e0, e1;
@@ -304,15 +309,14 @@ hj_status hj_tune(hj_ctx *c, const hj_rel *R, const hj_rel *S, const hj_opts *op
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (st != HJ_OK) return st;
-    c->tuned[plan_key(R->width, agg, R->n, S->n)] = TunedPlan{pick.algo, pick.bits, pick.passes};
+    c->tuned[plan_key(jk, R->n, S->n)] = TunedPlan{pick.algo, pick.bits, pick.passes};
     if (out) {
         *out = hj_plan_info{};
         out->algo = pick.algo;
         out->radix_bits = pick.algo == HJ_ALGO_PHJ ? pick.bits : 0;
         out->passes = pick.algo == HJ_ALGO_PHJ ? pick.passes : 0;
         double s4[4];
-        out->predicted_ms = 1e3 * predict_seconds(c->model, R->width, agg, mat, R->n, S->n, pick.algo, pick.bits,
-                                                  pick.passes, s4);
+        out->predicted_ms = 1e3 * predict_seconds(c->model, jk, R->n, S->n, pick.algo, pick.bits, pick.passes, s4);
         for (int i = 0; i < 4; ++i) out->step_ms[i] = 1e3 * s4[i];
         out->measured_ms = best;
     }

@@ -73,3 +73,26 @@ def test_count_modes_drop_the_output_bytes(hjm):
     mat = plan(hjm, 1 << 24, 1 << 28, algo=hjm.HJ_ALGO_PHJ, radix_bits=11, passes=1)
     cnt = plan(hjm, 1 << 24, 1 << 28, algo=hjm.HJ_ALGO_PHJ, radix_bits=11, passes=1, mode=hjm.HJ_COUNT)
     assert cnt["predicted_ms"] <= mat["predicted_ms"]
+
+
+@pytest.mark.parametrize("width,rows", [(4, 8192), (8, 4096)])
+def test_the_model_prices_the_join_that_shj_runs(hjm, width, rows):
+    # the one-launch join of a build side in shared memory is taken for pairs without
+    # checksums only: with them, and in count modes, SHJ probes a table in global memory
+    import ctypes
+
+    lib, ns = hjm.load_library(), 1 << 22
+
+    def shj(nr, mode=hjm.HJ_MATERIALIZE, flags=0):
+        r, s = hjm.hj_rel(None, nr, width, 0), hjm.hj_rel(None, ns, width, 0)
+        o = hjm.hj_opts(hjm.HJ_ALGO_SHJ, mode, 0, 0, 0, flags)
+        p = hjm.hj_plan_info()
+        assert lib.hj_plan(None, ctypes.byref(r), ctypes.byref(s), ctypes.byref(o), ctypes.byref(p)) == hjm.HJ_OK
+        return list(p.step_ms), p.predicted_ms
+
+    assert shj(rows)[0][2] == 0.0  # no table built
+    assert shj(rows, flags=hjm.HJ_FLAG_CHECKSUM)[0][2] > 0.0
+    assert shj(rows, flags=hjm.HJ_FLAG_CHECKSUM)[1] > 1.2 * shj(rows)[1]
+    assert shj(rows + 1)[0][2] > 0.0
+    assert shj(rows + 1, flags=hjm.HJ_FLAG_CHECKSUM) == shj(rows + 1)
+    assert shj(rows, mode=hjm.HJ_COUNT)[0][2] > 0.0
