@@ -1,18 +1,18 @@
 // batch.cu -- many independent joins in a few launches (hj_join_batch).
 //
 // Every join partitions on the radix bits that its build size calls for (2048 4-byte or
-// 1024 8-byte build tuples per partition at most while 2^11 digits do, at least one bit so that every partition is padded and
-// filtered the same way).  Two launches partition all relations of all joins at once
-// (one histogram, one scatter over their chunks, each relation read in place), one
-// lists the partition pairs, and ONE persistent launch of the shared-memory join
-// kernel runs every (join, partition) task, taking tasks from a work counter so that
-// joins of very different sizes share the GPU.  The chunk tables are made on the host
-// and travel in one copy; the pair buffers are allocated while the partitioning runs.
-// Pairs are placed by exact per-task claims into each join's own buffer (the staging
-// sink), so no compaction is needed.  When the workspace of all joins would exceed
-// the HBM budget, joins run in waves.  With four launches to a wave there is nothing
-// left for a CUDA graph to shorten (capture and instantiation took longer than they
-// saved), so HJ_FLAG_GRAPH changes nothing.
+// 1024 8-byte build tuples per partition at most while 2^11 digits do, at least one bit
+// so that every partition is padded and filtered the same way).  Two launches partition
+// all relations of all joins at once (one histogram, one scatter over their chunks, each
+// relation read in place), one lists the partition pairs, and ONE persistent launch of
+// the shared-memory join kernel runs every (join, partition) task, taking tasks from a
+// work counter so that joins of very different sizes share the GPU.  The chunk tables
+// are made on the host and travel in one copy; the pair buffers are allocated while the
+// partitioning runs.  Pairs are placed by exact per-task claims into each join's own
+// buffer (the staging sinks), so no compaction is needed.  When the workspace of all
+// joins would exceed the HBM budget, joins run in waves.  With four launches to a wave
+// there is nothing left for a CUDA graph to shorten (capture and instantiation took
+// longer than they saved), so HJ_FLAG_GRAPH changes nothing.
 #include <algorithm>
 #include <cmath>
 #include <memory>

@@ -42,8 +42,7 @@ template <> struct PairOut<8> {
 };
 
 // Output context of a launch: the pair buffer of one join and its counters.  With
-// `dense`, every append claims exactly its pairs from ctr->count (no chunks, no
-// holes).  With `stage` (this warp's shared-memory buffer of `scap` pairs), a warp
+// `stage` (this warp's shared-memory buffer of `scap` pairs), a warp
 // collects its pairs there and claims exactly as many rows of ctr->count when the
 // buffer fills or the warp is done, then copies them out with coalesced stores:
 // no holes either, one atomic per buffer.  Otherwise warps take whole chunks from
@@ -53,7 +52,6 @@ struct OutCtx {
     uint64_t pcap;
     hj_counters *ctr;
     unsigned int join = 0;
-    bool dense = false;
     void *stage = nullptr;
     unsigned scap = 0;
 };
@@ -108,13 +106,6 @@ __device__ __forceinline__ void warp_append(OutState &st, const OutCtx &oc, bool
         st.used += k;
         return;
     }
-    if (oc.dense) {
-        unsigned long long b = 0;
-        if (lane == 0) b = atomicAdd(&oc.ctr->count, (unsigned long long)k);
-        b = __shfl_sync(0xffffffffu, b, 0);
-        if (has && b + rank < oc.pcap) PairOut<W>::put(oc.pairs, b + rank, a, b_);
-        return;
-    }
     const unsigned room = kChunkPairs - st.used;
     unsigned long long nb = 0;
     if (k > room) {
@@ -135,16 +126,11 @@ __device__ __forceinline__ void warp_append(OutState &st, const OutCtx &oc, bool
     st.pairs += k;
 }
 
-// Append one pair per lane and item with cnt[i] == 1 (IT <= 4 items; a staging
-// buffer holds at least 32 * IT pairs): one room test for all of them.
+// Staged output of one pair per lane and item with cnt[i] == 1 (the buffer holds at least
+// 32 * IT pairs): one room test for all of them.
 template <int W, int IT>
 __device__ __forceinline__ void warp_append_group(OutState &st, const OutCtx &oc, const uint32_t *cnt,
                                                   const typename Tup<W>::U *a, const typename Tup<W>::U *b) {
-    if (!oc.stage) {
-#pragma unroll
-        for (int i = 0; i < IT; ++i) warp_append<W>(st, oc, cnt[i] == 1, a[i], b[i]);
-        return;
-    }
     using P = typename PairVec<W>::T;
     const unsigned lt = (1u << (threadIdx.x & 31)) - 1u;
     unsigned m[IT], tot = 0;
@@ -166,10 +152,9 @@ __device__ __forceinline__ void warp_append_group(OutState &st, const OutCtx &oc
     st.used += tot;
 }
 
-// Record the warp's partly filled chunk and add its pair count.  All lanes call.
+// Record the warp's partly filled chunk and add its pair count (chunked output).  All lanes call.
 __device__ __forceinline__ void warp_finish(const OutState &st, const OutCtx &oc, const RecArea &ra) {
     if ((threadIdx.x & 31) != 0) return;
-    if (oc.dense || oc.stage) return;  // exact claims count themselves and leave no holes
     if (st.claimed && st.used < kChunkPairs) {
         unsigned long long i = atomicAdd(ra.n, 1ull);
         if (i < ra.cap) {

@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(256, kProbeCtas) pair_probe_kernel(const void 
     RunQueue<W> &q = *(RunQueue<W> *)(mine + kProbeStageBytes);
     uint32_t qn = 0;
     OutState st;
-    OutCtx oc{pairs, pcap, ctr, 0u, false};
+    OutCtx oc{pairs, pcap, ctr};
     oc.stage = mine;
     oc.scap = kProbeStage<W>;
     st.used = 0;
@@ -534,7 +534,8 @@ hj_status table_build(hj_ctx *c, hj_table *t, const void *R, uint64_t n, PartFil
     if (!n) return HJ_OK;
     const unsigned grid = items_grid(c, n, t->width == 4 ? 512 : 256, 32);
     TableSide *side = (TableSide *)t->side;
-#define HJ_TB(WW, AA) HJ_LAUNCH(c, "table_build", (table_build_kernel<WW, AA>), grid, 256, 0, R, n, t->slots, t->cap, side, c->d_ctr, pf)
+#define HJ_TB(WW, AA)                                                                                             \
+    HJ_LAUNCH(c, "table_build", (table_build_kernel<WW, AA>), grid, 256, 0, R, n, t->slots, t->cap, side, c->d_ctr, pf)
     if (t->width == 4) {
         if (t->agg) HJ_TB(4, true); else HJ_TB(4, false);
     } else {
@@ -555,9 +556,9 @@ hj_status table_probe(hj_ctx *c, const hj_table *t, const void *S, uint64_t n, v
                       t->slots, t->cap, side, ctr, pf);                                                             \
         else {                                                                                                      \
             HJ_TRY(allow_max_smem(c, (const void *)pair_probe_kernel<WW, CC>));                                     \
-            HJ_LAUNCH(c, "table_probe", (pair_probe_kernel<WW, CC>), items_grid(c, n, 256 * kProbeItems, kProbeCtas), 256,   \
-                      8 * kProbeWarpBytes<WW>, S, n, t->slots, (uint32_t)(t->cap / kBucketSlots<WW>), side, pairs,     \
-                      pcap, ctr);                                                                                   \
+            HJ_LAUNCH(c, "table_probe", (pair_probe_kernel<WW, CC>),                                                \
+                      items_grid(c, n, 256 * kProbeItems, kProbeCtas), 256, 8 * kProbeWarpBytes<WW>, S, n,          \
+                      t->slots, (uint32_t)(t->cap / kBucketSlots<WW>), side, pairs, pcap, ctr);                     \
         }                                                                                                           \
     } while (0)
     if (t->width == 4) {
@@ -683,8 +684,8 @@ __device__ __forceinline__ void soa_coop_emit(const SoaTab<W> &t, typename Tup<W
 // partly used chunks are recorded and compacted on the device afterwards.  Used
 // for a single join: no extra traffic, a small fix-up at the end.
 //
-// WarpStageSink (below): every warp stages its pairs in a private buffer and
-// claims exact rows of the join's buffer per buffer-full.  Used for batches of
+// WarpStageSink, GlobalStageSink: every warp stages its pairs in a private buffer
+// and claims exact rows of the join's buffer per buffer-full.  Used for batches of
 // joins, where per-warp chunks would leave a partly used chunk per warp per join.
 // The join's pair count is the claim cursor (ctr->count).
 template <int W> struct ChunkSink {
@@ -701,7 +702,7 @@ template <int W> struct ChunkSink {
         if (j == join) return;
         if (join != ~0u) warp_finish(st, oc, ra);
         st = OutState();
-        oc = OutCtx{slots[j].pairs, slots[j].pcap, slots[j].ctr, j, false};
+        oc = OutCtx{slots[j].pairs, slots[j].pcap, slots[j].ctr, j};
         join = j;
         room = 0;
     }
@@ -775,8 +776,9 @@ template <int W> struct ChunkSink {
 
 // Per-warp staged exact output (batches of joins, whose many joins per launch
 // would leave a partly filled chunk per warp and join): each warp collects its
-// pairs in a private buffer of scap pairs in shared memory and, when the buffer fills or the warp moves on to another join,
-// claims exactly that many rows of the join's buffer with one atomic add and
+// pairs in a private buffer of scap pairs in shared memory and, when the buffer fills or
+// the warp moves on to another join, claims exactly that many rows of the join's buffer
+// with one atomic add and
 // copies them out with coalesced stores.  Output is dense as written (no
 // compaction) and the sink needs no CTA barrier.  scap >= 32 x the items of a
 // group, so one flush always makes room.
@@ -1346,8 +1348,8 @@ __global__ void __launch_bounds__(NT, join_ctas(NT)) partition_join_kernel(
         sink.scap = kJoinStageBytes / (2 * W);
         sink.slots = slots;
     }
-    // While more than two of the first `lead` tasks per CTA remain, tasks are taken one ahead: during a
-    // task's build warp 0 reads the record of the next one (whose index it took at the
+    // While more than two of the first `lead` tasks per CTA remain, tasks are taken one
+    // ahead: during a task's build warp 0 reads the record of the next one (whose index it took at the
     // end of the task before), and during its probe the next one's build rows and first
     // probe rows are asked into L2.  The last tasks are taken as CTAs fall idle.
     constexpr unsigned kTaskWords = sizeof(PartTask) / 4;
@@ -1470,44 +1472,40 @@ __global__ void __launch_bounds__(NT, join_ctas(NT)) partition_join_kernel(
                 };
                 for (uint32_t v0 = threadIdx.x; v0 < nrv; v0 += RB * NT) {
                     if (v0 != threadIdx.x) load_r(v0);
-                    constexpr int QV = RB, QT = QV * PV;  // vectors and tuples of a step
+                    constexpr int QT = RB * PV;  // tuples of a step
+                    T k[QT], r[QT];
+                    uint32_t bkt[QT], q[QT];
+                    bool in[QT];
 #pragma unroll
-                    for (int u0 = 0; u0 < RB; u0 += QV) {
-                        T k[QT], r[QT];
-                        uint32_t bkt[QT], q[QT];
-                        bool in[QT];
-#pragma unroll
-                        for (int i = 0; i < QT; ++i) {
-                            const Vec &x = rx[u0 + i / PV];
-                            if constexpr (W == 4) {
-                                k[i] = i % 2 ? x.z : x.x;
-                                r[i] = i % 2 ? x.w : x.y;
-                            } else {
-                                k[i] = x.x;
-                                r[i] = x.y;
-                            }
-                            // a padding row carries 0 or a pass's second sentinel: only
-                            // such keys are hashed to see whether the row is the partition's
-                            in[i] = v0 + (u0 + i / PV) * NT < nrv &&
-                                    !((k[i] == T(0) || k[i] == pk1 || k[i] == pk2) &&
-                                      !pf.keep(hashw<W>(k[i])));
-                            bkt[i] = part_bucket<W>(k[i], tab.nb);
-                            q[i] = in[i] ? tried(bkt[i]) : 0u;
+                    for (int i = 0; i < QT; ++i) {
+                        const Vec &x = rx[i / PV];
+                        if constexpr (W == 4) {
+                            k[i] = i % 2 ? x.z : x.x;
+                            r[i] = i % 2 ? x.w : x.y;
+                        } else {
+                            k[i] = x.x;
+                            r[i] = x.y;
                         }
+                        // a padding row carries 0 or a pass's second sentinel: only
+                        // such keys are hashed to see whether the row is the partition's
+                        in[i] = v0 + (i / PV) * NT < nrv &&
+                                !((k[i] == T(0) || k[i] == pk1 || k[i] == pk2) && !pf.keep(hashw<W>(k[i])));
+                        bkt[i] = part_bucket<W>(k[i], tab.nb);
+                        q[i] = in[i] ? tried(bkt[i]) : 0u;
+                    }
 #pragma unroll
-                        for (int i = 0; i < QT; ++i) {
-                            if (!in[i]) continue;
-                            for (uint32_t it = 1; q[i] >= G && it < lim; ++it) {
-                                bkt[i] = bkt[i] + 1 == tab.nb ? 0 : bkt[i] + 1;
-                                q[i] = tried(bkt[i]);
-                            }
-                            if (q[i] < G) {
-                                T *slot = &kv[bkt[i] * G + q[i]];
-                                slot[0] = k[i];
-                                slot[cap] = r[i];  // the same slot of the rid region
-                            } else {
-                                s_full = 1;
-                            }
+                    for (int i = 0; i < QT; ++i) {
+                        if (!in[i]) continue;
+                        for (uint32_t it = 1; q[i] >= G && it < lim; ++it) {
+                            bkt[i] = bkt[i] + 1 == tab.nb ? 0 : bkt[i] + 1;
+                            q[i] = tried(bkt[i]);
+                        }
+                        if (q[i] < G) {
+                            T *slot = &kv[bkt[i] * G + q[i]];
+                            slot[0] = k[i];
+                            slot[cap] = r[i];  // the same slot of the rid region
+                        } else {
+                            s_full = 1;
                         }
                     }
                 }
@@ -1518,7 +1516,8 @@ __global__ void __launch_bounds__(NT, join_ctas(NT)) partition_join_kernel(
                 const PartTask &nt = s_task[cur_task ^ 1];
                 const uint32_t rl = (nt.nr / PV + 7) / 8, sl = (min(nt.ns / PV, kAheadVecs) + 7) / 8;
                 for (uint32_t i = threadIdx.x; i < rl + sl; i += NT)
-                    prefetch_l2(i < rl ? (const char *)nt.R + (uint64_t)i * 128 : (const char *)nt.S + (uint64_t)(i - rl) * 128);
+                    prefetch_l2(i < rl ? (const char *)nt.R + (uint64_t)i * 128
+                                       : (const char *)nt.S + (uint64_t)(i - rl) * 128);
             }
             bool unique = false;
             if constexpr (!AGG) unique = nsv >= 2 * nrv && !s_full && !__syncthreads_or(keys_repeat<W, NT>(tab));
@@ -1663,7 +1662,9 @@ __global__ void __launch_bounds__(NT, join_ctas(NT)) small_join_kernel(const voi
         }
     }
     __syncthreads();
-    if (s_full) {  // (the same in every CTA)
+    if (s_full) {
+        // (near the walk's limit it depends on the order of a CTA's inserts: one CTA that
+        // gives up discards the whole attempt)
         if (threadIdx.x == 0) atomicOr(&ctr->status, (unsigned long long)kStatusLongRun);
         return;
     }
@@ -1697,7 +1698,8 @@ __global__ void __launch_bounds__(NT, join_ctas(NT)) small_join_kernel(const voi
     sink.finish();
 }
 
-// (what a table of two and a half slots per tuple holds in a CTA's shared memory)
+// (what a table of two and a half slots per tuple, 8-byte ones 2.4, holds in a CTA's shared
+// memory)
 uint64_t small_join_rows(int width) { return width == 4 ? 8192 : 4096; }
 
 hj_status small_join(hj_ctx *c, int width, const void *R, uint64_t nr, const void *S, uint64_t ns, void *pairs,
@@ -1739,8 +1741,6 @@ hj_status small_join(hj_ctx *c, int width, const void *R, uint64_t nr, const voi
     return HJ_OK;
 }
 
-// Tasks of one join partitioned into NP padded partitions: task p covers rows
-// [roff[p], roff[p+1]) of Rp and [soff[p], soff[p+1]) of Sp.
 // Tasks of one join partitioned into NP padded partitions.  Partition p covers
 // rows [roff[p], roff[p+1]) of Rp and [soff[p], soff[p+1]) of Sp.  Its S rows are
 // cut into slices of at most `slice` rows (a multiple of the sector's tuples, so

@@ -899,8 +899,9 @@ __global__ void __launch_bounds__(kTmaThreads, 1) scatter_tma_kernel(
 // pipe (a claim 3.7 and a slot store 6.2 cycles per warp, a flush about 5) and the two
 // barriers of a tile.  One tile in registers covers a third of the loads' latency:
 // the tile after it is asked into L2 (2^26 tuples at 2^11 digits 362 -> 282 us; three
-// tiles ahead 301), and its loads go out one vector at a time (269 us).  Sectors written by a lane each, carried tuples moved to the front
-// and no L2 prefetch took 387 us, and 401 .. 430 us at 2^5 .. 2^8 digits (now 208).
+// tiles ahead 301), and its loads go out one vector at a time (269 us).  Sectors written by
+// a lane each, carried tuples moved to the front and no L2 prefetch took 387 us, and
+// 401 .. 430 us at 2^5 .. 2^8 digits (now 208).
 constexpr int kRegionThreads = 1024;
 constexpr int kRegionVecs = 4;  // 16-byte vectors per thread per tile
 constexpr size_t kRegionSmem = 227u * 1024u - 1024u;
@@ -1519,15 +1520,13 @@ static hj_status launch_padded(hj_ctx *c, int bits, unsigned na, unsigned nb, co
 // Scatter configuration (threads, vectors per thread) for a fan-out: 8192-tuple
 // tiles of 4-byte tuples while the per-digit state leaves room, 4096 otherwise.
 struct ScatterCfg {
-    int nt, vpt;
     uint64_t tile;
     bool tma;
 };
 static ScatterCfg scatter_cfg(int width, int bits) {
-    // up to 2^11 digits the TMA-staged kernel fits shared memory
-    if (bits <= 11) return ScatterCfg{kTmaThreads, 0, (uint64_t)(width == 4 ? TmaShape<4>::T : TmaShape<8>::T), true};  // 2^bits <= 2 * kTmaThreads
-    if (width == 4) return ScatterCfg{1024, 2, 4096, false};
-    return ScatterCfg{1024, 2, 2048, false};
+    // up to 2^11 digits (2 * kTmaThreads) the TMA-staged kernel fits shared memory
+    if (bits <= 11) return ScatterCfg{(uint64_t)(width == 4 ? TmaShape<4>::T : TmaShape<8>::T), true};
+    return ScatterCfg{width == 4 ? 4096ull : 2048ull, false};  // 1024 threads x 2 vectors
 }
 
 // Chunk size of a pass: about one chunk per SM over the whole input (one scatter
@@ -1605,13 +1604,12 @@ hj_status partition_pass(hj_ctx *c, int width, const void *in, uint64_t n_total,
     }
     uint64_t k0, k1;
     sentinel_keys(width, shift, bits, &k0, &k1);
-#define HJ_SC(WW, NT, VPT)                                                                                    \
-    do {                                                                                                      \
-        auto kern = scatter_kernel<WW, NT, VPT>;                                                              \
-        const size_t ssmem = scatter_smem_bytes<WW, NT, VPT>((uint32_t)P);                                    \
-        HJ_TRY(allow_max_smem(c, (const void *)kern));                                                       \
-        HJ_LAUNCH(c, "partition_scatter", kern, (unsigned)max_chunks, NT, ssmem, in, n_total, seg_off, nseg, cb, \
-                  chunk, shift, bits, Hs, out, pad, k0, k1);                                                  \
+#define HJ_SC(WW)                                                                                                  \
+    do {                                                                                                           \
+        auto kern = scatter_kernel<WW, 1024, 2>;                                                                   \
+        HJ_TRY(allow_max_smem(c, (const void *)kern));                                                             \
+        HJ_LAUNCH(c, "partition_scatter", kern, (unsigned)max_chunks, 1024, (scatter_smem_bytes<WW, 1024, 2>((uint32_t)P)), \
+                  in, n_total, seg_off, nseg, cb, chunk, shift, bits, Hs, out, pad, k0, k1);                       \
     } while (0)
     const size_t tma_smem = width == 4 ? scatter_tma_smem_bytes<4>((uint32_t)P) : scatter_tma_smem_bytes<8>((uint32_t)P);
     if (cfg.tma && pad) {
@@ -1634,9 +1632,9 @@ hj_status partition_pass(hj_ctx *c, int width, const void *in, uint64_t n_total,
                       n_total, seg_off, nseg, cb, chunk, shift, bits, Hs, out, pad, k0, k1, &c->d_ctr->fault, polls);
         }
     } else if (width == 4) {
-        if (cfg.nt == 512) HJ_SC(4, 512, 8); else HJ_SC(4, 1024, 2);
+        HJ_SC(4);
     } else {
-        if (cfg.nt == 512) HJ_SC(8, 512, 4); else HJ_SC(8, 1024, 2);
+        HJ_SC(8);
     }
 #undef HJ_SC
     return HJ_OK;

@@ -41,7 +41,8 @@ __global__ void static_build_kernel(const void *R, uint64_t n, void *slots, uint
         if (!pair_insert<W>((typename PairSlot<W>::S *)slots, nb, &hdr->side, k, r, key_hash<W>(k), &repeat,
                             kStaticMaxWalk))
             atomicOr(&hdr->ctr.status,
-                     (unsigned long long)((uint64_t)nb * kBucketSlots<W> <= kStaticMaxWalk ? kStatusTableFull : kStatusLongRun));
+                     (unsigned long long)((uint64_t)nb * kBucketSlots<W> <= kStaticMaxWalk ? kStatusTableFull
+                                                                                          : kStatusLongRun));
     }
 }
 
