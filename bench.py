@@ -748,7 +748,7 @@ def run_batch(args, wl, ws, rank, local):
     pms, _ = timed(plain, psteps)
     plain_value = weak_value(tuples_step, psteps, ws, pms)
 
-    # kernel times from one profiled step without the graph (events are not captured)
+    # kernel times from one profiled step
     hj.prof_reset(ctx)
     hj.prof_enable(ctx, True)
     batched(graph=False)

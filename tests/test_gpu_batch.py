@@ -139,7 +139,7 @@ def test_batch_many_joins_with_many_oversize_partitions(hjm, ctx, mode):
 def test_batch_full_size_counts_and_sampled_pairs(hjm, ctx):
     # The 4096-join batch at full size (|R| log-uniform in [2^10, 2^22], |S| = 4 |R|, about
     # 1.1e10 tuples), in the launch configuration the bench times (pairs materialised,
-    # one CUDA graph per wave).  R keys are exactly 1..|R|, so an S tuple matches once
+    # HJ_FLAG_GRAPH set).  R keys are exactly 1..|R|, so an S tuple matches once
     # if its key is at most |R| and never otherwise: every join's count is checked
     # against that property, and sampled joins' pairs against the oracle.
     specs = W.batched_specs(4096, W.DEFAULT_SEED)
@@ -199,6 +199,35 @@ def test_batch_partitions_every_fanout_at_once(hjm, ctx, width):
         assert (cnt[j].count, *cnt[j].checksum) == oracle.join_aggregate(R, S), j
         assert np.array_equal(_sorted(res[j].pairs_numpy()), want), j
         res[j].free()
+
+
+@pytest.mark.parametrize("skew", [False, True])
+@pytest.mark.parametrize("width,bits", [(4, 10), (4, 11), (8, 10), (8, 11)])
+def test_batch_partitions_on_many_digits(hjm, ctx, width, bits, skew):
+    # the smallest build side on 2^10 and 2^11 digits, where a digit has the fewest slots (12
+    # or 6 at 2^11), beside a small join; with `skew` half of S's keys share three digits,
+    # which overflow their slots in every tile, and wrap around them
+    step = 2048 if width == 4 else 1024
+    dt = np.uint32 if width == 4 else np.uint64
+    rng = np.random.default_rng(bits + width)
+    host, Rs, Ss = [], [], []
+    for nr, ns in (((step + 1 << (bits - 1)) + 3, 300_001), (3000, 7001)):
+        R = np.stack([rng.permutation(np.arange(1, nr + 1)).astype(dt), np.arange(nr, dtype=dt)], 1)
+        S = np.stack([rng.integers(1, 2 * nr, ns).astype(dt), np.arange(ns, dtype=dt)], 1)
+        if skew:
+            S[::2, 0] = rng.choice(np.array([5, 9, 2 * nr + 1], dt), len(S[::2]))
+        host.append((R, S))
+        for a, rels in ((R, Rs), (S, Ss)):
+            rels.append(torch.from_numpy(a.view(np.int32 if width == 4 else np.int64)).to(DEV))
+    res = hjm.hj_join_batch(ctx, Rs, Ss)
+    assert res[0].radix_bits == bits
+    for j, (R, S) in enumerate(host):
+        want = oracle.sorted_pairs(*oracle.hash_join(R, S))
+        assert np.array_equal(_sorted(res[j].pairs_numpy()), want), j
+        res[j].free()
+    cnt = hjm.hj_join_batch(ctx, Ss, Rs, mode=hjm.HJ_COUNT_CHECKSUM)  # the skewed side builds
+    for j, (R, S) in enumerate(host):
+        assert (cnt[j].count, *cnt[j].checksum) == oracle.join_aggregate(S, R), j
 
 
 @pytest.mark.parametrize("width,nr", [(4, 25_000_000), (8, 12_000_000)])

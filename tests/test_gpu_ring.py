@@ -1,15 +1,13 @@
-"""The ring scatter -- the partition scatter that 4-byte joins take at 2^11 digits
-(the plan the tuner picks for the 2^24 x 2^28 join) and 2^10, and 8-byte joins at
-2^9 .. 2^11 -- against the CPU oracle,
-element by element, on inputs that drive each of its paths: rings that overflow to
-the far end of their run (keys crowded into two digits), duplicate build keys, a
-batch whose group partitions on 11 bits (the per-segment input path), and its
-bounded wait made to run out on purpose (a short limit; the kernel returns and the
-host reports HJ_E_TIMEOUT, no GPU fault).  hj_debug_scatter forces the ring or the
-region scatter, and both kernels are checked at every width and fan-out the ring
-is built for, on ragged sizes and on crowded digits; the region scatter is also
-checked at the low fan-outs where it keeps up to 256 slots per digit.  Join results are integers: every comparison is
-exact."""
+"""The scatters of a padded partition pass against the CPU oracle, element by element: the
+region scatter, which joins take at every fan-out, and the ring scatter, which runs on
+request (hj_debug_scatter) at 2^9 .. 2^11 digits and under a wait limit.  Inputs drive
+each of their paths: digits whose slots overflow to the far end of their run (keys
+crowded into two digits), duplicate build keys, batches that partition on up to 11 bits,
+and the ring's bounded wait made to run out on purpose (a short limit; the kernel
+returns and the host reports HJ_E_TIMEOUT, no GPU fault).  Both kernels are checked at
+every width and fan-out the ring is built for, on ragged sizes and on crowded digits;
+the region scatter also at the low fan-outs.  Join results are integers: every
+comparison is exact."""
 import numpy as np
 import pytest
 import torch
@@ -174,10 +172,9 @@ def test_duplicate_build_keys_at_eleven_bits(hjm, ctx):
 
 
 def test_batch_group_on_eleven_bits(hjm, ctx):
-    # Two joins with |R| > 2^23 make a batch group that partitions on 11 bits (each
-    # join one segment of the pass, read from its own array); a small join beside
-    # them takes another group.  Every join's pairs, count and checksums against
-    # the oracle.
+    # Two joins with |R| > 2^23 partition on 11 bits in the launches that partition a
+    # small join beside them on 2.  Every join's pairs, count and checksums against the
+    # oracle.
     sizes = [((1 << 23) + 1030, (1 << 23) + 77), ((1 << 23) + 2049, (1 << 22) + 5), (5000, 20_001)]
     Rs, Ss = [], []
     for j, (nr, ns) in enumerate(sizes):
