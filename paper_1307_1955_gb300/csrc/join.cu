@@ -350,7 +350,7 @@ __global__ void agg_table_init(AggSlot<W> *slots, uint64_t cap) {
 }
 
 template <int W, bool AGG>
-__global__ void __launch_bounds__(256) table_build_kernel(const void *R, uint64_t n, void *slots, uint64_t cap,
+__global__ void __launch_bounds__(256, 8) table_build_kernel(const void *R, uint64_t n, void *slots, uint64_t cap,
                                                           TableSide *side, hj_counters *ctr, PartFilter pf) {
     constexpr int PV = Tup<W>::kPerVec;
     const uint64_t nvec = (n + PV - 1) / PV;
@@ -660,18 +660,16 @@ __device__ __forceinline__ void soa_coop_emit(const SoaTab<W> &t, typename Tup<W
     using T = typename Tup<W>::U;
     constexpr uint32_t G = SoaTab<W>::G, BPW = 32 / G;
     const unsigned lane = threadIdx.x & 31, jb = lane / G, q = lane % G;
+#pragma unroll 1
     for (uint32_t off = 0; off < t.nb; off += BPW) {
         const bool inr = off + jb < t.nb;
         uint32_t b = home + off + jb;
         if (b >= t.nb) b -= t.nb;
         const T key = inr ? t.ld1(b, 0, q) : t.empty;
         const T rid = inr ? t.ld1(b, 1, q) : T(0);
-        const unsigned emp = __ballot_sync(0xffffffffu, key == t.empty);
-        const bool bucket_empty_slot = ((emp >> (jb * G)) & ((1u << G) - 1u)) != 0;
-        const bool bucket_end = !inr || bucket_empty_slot || !t.overflowed(b);
-        const unsigned endm = __ballot_sync(0xffffffffu, bucket_end && q == 0);
-        const unsigned last_lane = endm ? (unsigned)(__ffs(endm) - 1) + G - 1 : 31u;
-        const bool m = inr && lane <= last_lane && key == kk;
+        // (slots fill in order: a bucket whose last one is empty ends the run)
+        const unsigned endm = __ballot_sync(0xffffffffu, q == G - 1 && (!inr || key == t.empty || !t.overflowed(b)));
+        const bool m = inr && key == kk && lane <= (endm ? (unsigned)(__ffs(endm) - 1) : 31u);
         sink.append(m, rid, ss);
         if (endm) break;
     }
@@ -919,7 +917,9 @@ __device__ __forceinline__ void drain_walks(const SoaTab<W> &tab, const typename
 #pragma unroll 1
     for (uint32_t it = 1; it < tab.nb; ++it) {
         unsigned on = __ballot_sync(0xffffffffu, active);
-        if (!on || (it > 3 && __popc(on) <= kLongWalks)) {  // the long runs that are left: 32 slots at a time
+        if (!on) break;
+        if (!UNIQ && it > 3 && __popc(on) <= kLongWalks) {  // the long runs that are left: 32 slots at a time
+#pragma unroll 1
             while (on) {
                 const int L = __ffs(on) - 1;
                 on &= on - 1;
