@@ -872,10 +872,11 @@ constexpr uint32_t kMaxSmemWalk = 64;
 
 // When no more walks than this are left of 32 after three buckets, the warp takes one after
 // the other, 32 slots at a time, in place of all at once, a bucket at a time (each key of R
-// 16 times: 3580 us without this, 3330 with).  Before that the walks left are short ones,
-// which end sooner together (taken one by one from the first bucket on: 2^24 x 2^28 tuples
-// of different keys 2330 -> 2500 us).
-constexpr int kLongWalks = 2;
+// 4 / 16 / 40 times: 930 / 3300 / 8370 us with 2, 955 / 3150 / 8130 with 4, 975 / 3170 / 7910
+// with 8; 16 times 3580 without).  Before that, and with a table of different keys, the
+// walks left are short ones, which end sooner together (taken one by one from the first
+// bucket on: 2^24 x 2^28 tuples of different keys 2330 -> 2500 us).
+constexpr int kLongWalks = 4;
 
 // Entries per warp of the queue of pending run walks (probe keys and rids whose
 // run goes on past a full home bucket).
@@ -992,8 +993,8 @@ template <int W, int NT> __device__ __forceinline__ bool keys_repeat(const SoaTa
 // key is twice in the table) a match ends the search; otherwise the further matches of the
 // home buckets go out one per item and step.  (A warp that walked one such item after the
 // other lived from many warps, 32 of them; with 20, |R| = 2^22 4-byte tuples of each key
-// twice / 4 / 16 times with 2^24: 3640 / 3860 / 5860 us, like this 575 / 937 / 3330; each key
-// four times with 8 bytes 4260 and 1665.)  With MARK the marker of empty slots may be a key:
+// twice / 4 / 16 times with 2^24: 3640 / 3860 / 5860 us, like this 575 / 955 / 3150; each key
+// four times with 8 bytes 4260 and 1710.)  With MARK the marker of empty slots may be a key:
 // its build rids are the `side` list.
 template <int W> struct SideList {
     const typename Tup<W>::U *rids = nullptr;
